@@ -525,15 +525,14 @@ __global__ void k_probe_direction(int level, long long p0, long long n, const in
 __global__ void k_probe_traverse(long long n, const long long *p0, const int32_t *d, int gx, int gy, int gz,
                                  int32_t *cells, float *ds, int32_t *nseg, int32_t *esc) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        Walk w;
-        walk_init(w, (int)p0[3 * i], (int)p0[3 * i + 1], (int)p0[3 * i + 2], d[3 * i], d[3 * i + 1], d[3 * i + 2]);
         int key[4];
         float s[4];
         bool e = false;
-        const unsigned m = walk_step(w, gx, gy, gz, 0, key, s, e);
+        walk_step(true, (int)p0[3 * i], (int)p0[3 * i + 1], (int)p0[3 * i + 2], d[3 * i], d[3 * i + 1], d[3 * i + 2], gx,
+                  gy, gz, 0, key, s, e);
         int k = 0;
         for (int j = 0; j < 4; ++j) {
-            if (!(m & (1u << j))) continue;
+            if (key[j] < 0) continue;
             const int c = key[j];
             cells[12 * i + 3 * k] = c % gx;
             cells[12 * i + 3 * k + 1] = (c / gx) % gy;

@@ -62,91 +62,90 @@ __host__ __device__ constexpr size_t march_shared_bytes(int nsims) {
     return (size_t)nsims * (NACC * sizeof(unsigned long long) + sizeof(MarchSim));
 }
 
-// (1 - e^-t)/t for 0 <= t < 1/8: its Taylor series through t^4 (the next
-// term, t^5/720, is under the single-precision epsilon there)
-__device__ __forceinline__ float2 series_q2(float2 t) {
-    const float2 nt = make_float2(-t.x, -t.y);
-    float2 q = make_float2(1.0f / 120.0f, 1.0f / 120.0f);
-    q = __ffma2_rn(q, nt, make_float2(1.0f / 24.0f, 1.0f / 24.0f));
+// (1 - e^-t)/t for 0 <= t < 1/8, from -t: its Taylor series through t^4 (the
+// next term, t^5/720, is under the single-precision epsilon there)
+__device__ __forceinline__ float2 series_q2(float2 nt) {
+    float2 q = __ffma2_rn(make_float2(1.0f / 120.0f, 1.0f / 120.0f), nt, make_float2(1.0f / 24.0f, 1.0f / 24.0f));
     q = __ffma2_rn(q, nt, make_float2(1.0f / 6.0f, 1.0f / 6.0f));
     q = __ffma2_rn(q, nt, make_float2(0.5f, 0.5f));
     return __ffma2_rn(q, nt, make_float2(1.0f, 1.0f));
 }
-__device__ __forceinline__ float series_q(float t) {
-    float q = 1.0f / 120.0f;
-    q = fmaf(q, -t, 1.0f / 24.0f);
-    q = fmaf(q, -t, 1.0f / 6.0f);
-    q = fmaf(q, -t, 0.5f);
-    return fmaf(q, -t, 1.0f);
+__device__ __forceinline__ float series_q(float nt) {
+    float q = fmaf(1.0f / 120.0f, nt, 1.0f / 24.0f);
+    q = fmaf(q, nt, 1.0f / 6.0f);
+    q = fmaf(q, nt, 0.5f);
+    return fmaf(q, nt, 1.0f);
 }
 
 // Attenuation of the photons ph[b] entering a segment of length dse (cells)
 // through a cell of optical depth per cell k = (HI at sigma_ref, sub-grid),
-// with its deposits (Eq. 13, Eq. 17): v[0] += absorbed photons, v[1] +=
+// with its deposits (Eq. 13, Eq. 17): v[0] = absorbed photons, v[1] =
 // sum_b sigma_b N_b (1 - e^-tau_b)/kappa_b, v[2] the same weighted by the
-// excess energy.  A bin with tau < 1/8 takes 1 - e^-tau = tau q(tau) with
-// the series q, so (1 - e^-tau)/kappa = dse q (no exponential, no
-// division) and keeps N - N tau q; a thicker bin takes the hardware
-// exponential and the division by kappa (N dse when kappa = 0).  SMALL:
-// every bin of every lane of the warp is thin, and only the series is
-// evaluated; the per-bin results are the same either way, so a ray's photons
-// do not depend on the rays it shares a warp with.  Bins go in pairs on the
-// paired single-precision units.
+// excess energy.  A bin with tau < 1/8 takes (1 - e^-tau)/kappa = dse q(tau)
+// with the series q (no exponential, no division); with phi = N dse q it
+// absorbs kappa phi and keeps N - kappa phi (one rounding).  A thicker bin
+// takes the hardware exponential and the division by kappa.  SMALL: every bin
+// of every lane of the warp is thin, and only the series is evaluated; the
+// per-bin results are the same either way, so a ray's photons do not depend
+// on the rays it shares a warp with.  Bins go in pairs on the paired
+// single-precision units, and the opacity enters negated, so that every
+// product of the thin path is an operand of a fused multiply-add: twelve
+// paired operations a pair of bins (eighteen with the opacity positive).
 template <int NB, bool SMALL>
 __device__ __forceinline__ void seg_attenuate(float2 k, float dse, const float *sig, const float *sige, float (&ph)[NB],
                                               float (&v)[4]) {
+    constexpr float NLOG2E = 1.44269504f;            // e^-tau = 2^(-tau log2 e)
     float2 w0 = make_float2(0.f, 0.f), w1 = w0, w2 = w0;
-    const float2 kx2 = make_float2(k.x, k.x), ky2 = make_float2(k.y, k.y), ds2 = make_float2(dse, dse);
+    const float2 kx2 = make_float2(-k.x, -k.x), ky2 = make_float2(-k.y, -k.y), ds2 = make_float2(dse, dse);
 #pragma unroll
     for (int b = 0; b + 1 < NB; b += 2) {
         const float2 sg = make_float2(sig[b], sig[b + 1]);
         const float2 se = make_float2(sige[b], sige[b + 1]);
-        const float2 kb = __ffma2_rn(kx2, sg, ky2);
-        const float2 tau = __fmul2_rn(kb, ds2);
+        const float2 nk = __ffma2_rn(kx2, sg, ky2);
+        const float2 nt = __fmul2_rn(nk, ds2);
         const float2 p2 = make_float2(ph[b], ph[b + 1]);
         const float2 pd = __fmul2_rn(p2, ds2);
-        float2 a, phin, pn;
+        float2 phin, pn;
         if (SMALL) {
-            const float2 q = series_q2(tau);
-            a = __fmul2_rn(p2, __fmul2_rn(q, tau));
-            phin = __fmul2_rn(pd, q);
-            pn = __fadd2_rn(p2, make_float2(-a.x, -a.y));
+            phin = __fmul2_rn(pd, series_q2(nt));
+            pn = __ffma2_rn(nk, phin, p2);
+            w0 = __ffma2_rn(nk, phin, w0);
         } else {
-            const float2 u = make_float2(fminf(tau.x, 0.125f), fminf(tau.y, 0.125f));
-            const float2 q = series_q2(u);
-            const float2 as = __fmul2_rn(p2, __fmul2_rn(q, u));
+            const bool s0 = nt.x > -0.125f, s1 = nt.y > -0.125f;
+            const float2 q = series_q2(make_float2(fmaxf(nt.x, -0.125f), fmaxf(nt.y, -0.125f)));
             const float2 ps = __fmul2_rn(pd, q);
-            const float ex0 = __expf(-tau.x), ex1 = __expf(-tau.y);
-            const bool s0 = tau.x < 0.125f, s1 = tau.y < 0.125f;
-            a = make_float2(s0 ? as.x : p2.x * (1.0f - ex0), s1 ? as.y : p2.y * (1.0f - ex1));
-            pn = make_float2(s0 ? p2.x - as.x : p2.x * ex0, s1 ? p2.y - as.y : p2.y * ex1);
-            phin = make_float2(s0 ? ps.x : (kb.x > 0.0f ? __fdividef(a.x, kb.x) : pd.x),
-                               s1 ? ps.y : (kb.y > 0.0f ? __fdividef(a.y, kb.y) : pd.y));
+            const float2 ns = __ffma2_rn(nk, ps, p2);
+            const float2 l2 = __fmul2_rn(nt, make_float2(NLOG2E, NLOG2E));
+            const float2 ex = make_float2(exp2_approx(l2.x), exp2_approx(l2.y));
+            const float2 nx = __fmul2_rn(p2, ex);                             // what is left
+            const float2 ab = __fmul2_rn(p2, __ffma2_rn(ex, make_float2(-1.0f, -1.0f), make_float2(1.0f, 1.0f)));
+            const float2 na = __fmul2_rn(nk, ps);
+            // (a bin in the division's lane has tau >= 1/8, so its kappa is not zero)
+            phin = make_float2(s0 ? ps.x : ab.x * rcp_approx(-nk.x), s1 ? ps.y : ab.y * rcp_approx(-nk.y));
+            pn = make_float2(s0 ? ns.x : nx.x, s1 ? ns.y : nx.y);
+            w0 = __fadd2_rn(w0, make_float2(s0 ? na.x : -ab.x, s1 ? na.y : -ab.y));
         }
         ph[b] = pn.x;
         ph[b + 1] = pn.y;
-        w0 = __fadd2_rn(w0, a);
         w1 = __ffma2_rn(sg, phin, w1);
         w2 = __ffma2_rn(se, phin, w2);
     }
-    v[0] = w0.x + w0.y;
+    v[0] = -(w0.x + w0.y);
     v[1] = w1.x + w1.y;
     v[2] = w2.x + w2.y;
     if (NB & 1) {
         const int b = NB - 1;
-        const float kb = fmaf(k.x, sig[b], k.y);
-        const float tau = kb * dse;
-        const float pd = ph[b] * dse;
-        float a, phin;
-        if (SMALL || tau < 0.125f) {
-            const float q = series_q(tau);
-            a = ph[b] * (q * tau);
-            phin = pd * q;
-            ph[b] -= a;
+        const float nk = fmaf(-k.x, sig[b], -k.y);
+        const float nt = nk * dse;
+        float phin, a;
+        if (SMALL || nt > -0.125f) {
+            phin = ph[b] * dse * series_q(nt);
+            a = -nk * phin;
+            ph[b] = fmaf(nk, phin, ph[b]);
         } else {
-            const float ex = __expf(-tau);
+            const float ex = exp2_approx(nt * NLOG2E);
             a = ph[b] * (1.0f - ex);
-            phin = kb > 0.0f ? __fdividef(a, kb) : pd;
+            phin = a * rcp_approx(-nk);
             ph[b] *= ex;
         }
         v[0] += a;
@@ -275,10 +274,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             int key[4];
             float ds[4];
             bool esc = false;
-            int nseg = 0;
-            unsigned vmask = 0u;
             {
-                Walk w;
                 // a queued ray is inside the box at the start of its step, so
                 // its position (at most 1000 cells of 2^21) fits 32 bits
                 int px, py, pz;
@@ -291,14 +287,11 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                     py = ((2 * ec.y + 1) << (FRAC_BITS - 1)) + age * dy;
                     pz = ((2 * ec.z + 1) << (FRAC_BITS - 1)) + age * dz;
                 }
-                walk_init(w, px, py, pz, dx, dy, dz);
-                // slots may be empty (tied crossings): every later phase
-                // visits the four slots in order and skips the empty ones
-#pragma unroll
-                for (int j = 0; j < 4; ++j) { key[j] = -1; ds[j] = 0.0f; }
-                if (valid) vmask = walk_step(w, S.nx, S.ny, S.nz, (int)S.coff, key, ds, esc);
-                nseg = __popc(vmask);
+                // slots may be empty: every later phase visits the four slots
+                // in order and skips the empty ones (negative keys)
+                walk_step(valid, px, py, pz, dx, dy, dz, S.nx, S.ny, S.nz, (int)S.coff, key, ds, esc);
             }
+            int nseg = 4 + (key[0] >> 31) + (key[1] >> 31) + (key[2] >> 31) + (key[3] >> 31);
             // (2) opacities of the crossed cells (Generalized mode: also the
             // ionised fraction and the screen's share)
             float2 kc[4];
@@ -340,7 +333,10 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                         for (int b = 0; b < NB; ++b) ph[b] *= keep;
                         if (rg[j] >= 1.0f) {
                             screened = true;
-                            nseg = __popc(vmask & ((2u << j) - 1u));
+                            nseg = j + 1;
+#pragma unroll
+                            for (int i2 = 0; i2 < 4; ++i2)
+                                if (i2 < j) nseg += key[i2] >> 31;
                         }
                     }
                 }
@@ -405,8 +401,15 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             }
             // compacted output into the warp's run of slots: the remainder of
             // the current run first, then a new run reserved with one atomic
-            const int incl = warp_incl_scan(nout);
-            const int tot = __shfl_sync(FULL, incl, 31);
+            // (without a split in the warp a ballot gives the positions; the
+            // shuffle scan only where a lane has children)
+            const unsigned outm = __ballot_sync(FULL, nout != 0);
+            int k0 = __popc(outm & ((1u << lane) - 1u)), tot = __popc(outm);   // this lane's first output position
+            if (__any_sync(FULL, nout > 1)) {
+                const int incl = warp_incl_scan(nout);
+                tot = __shfl_sync(FULL, incl, 31);
+                k0 = incl - nout;
+            }
             if (tot > 0) {
                 const unsigned s0 = slab;
                 const int left = slab_left;
@@ -441,7 +444,6 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                 }
                 w_out += tot;
                 if (fits && nout > 0) {
-                    const int k0 = incl - nout;  // this lane's first output position
                     auto slot_of = [&](int k) -> unsigned {
                         return k < left ? s0 + (unsigned)k : s1 + (unsigned)(k - left);
                     };
