@@ -436,17 +436,17 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
     DevBuf<Ctl> dctl;
     DevBuf<SimDev> dsim;
     DevBuf<SimAcc> dacc;
-    DevBuf<uint32_t> qpl[2], qem[2], qma[2], hist, sel, tkey, cand, ckey, lead_slot, bcnt, bled;
+    DevBuf<char> qmem[2];
+    DevBuf<uint32_t> hist, sel, tkey, cand, ckey, lead_slot, bcnt, bled;
     DevBuf<uint4> tgrp, gcm;
-    DevBuf<int32_t> qbi[2], qd[2], qm[2], tsim, rsim, lead_sim;
-    DevBuf<float> qph[2], qthr[2], grp, n0;
+    DevBuf<int32_t> tsim, rsim, lead_sim;
+    DevBuf<float> grp, n0;
     DevBuf<int4> ecell, rot;
     DevBuf<long long> pref, cell0;
     bool ok = dctl.alloc(1) == cudaSuccess && dsim.alloc(1) == cudaSuccess && dacc.alloc(1) == cudaSuccess;
-    for (int k = 0; k < 2 && ok; ++k)
-        ok = qpl[k].alloc(mq) == cudaSuccess && qem[k].alloc(mq) == cudaSuccess && qma[k].alloc(mq) == cudaSuccess &&
-             qbi[k].alloc(mq) == cudaSuccess && qd[k].alloc(3 * mq) == cudaSuccess && qm[k].alloc(3 * mq) == cudaSuccess &&
-             qph[k].alloc(nb * mq) == cudaSuccess && qthr[k].alloc(mq) == cudaSuccess;
+    size_t qbytes = 0;
+    queue_at(nullptr, mq, nb, true, &qbytes);
+    for (int k = 0; k < 2 && ok; ++k) ok = qmem[k].alloc(qbytes) == cudaSuccess;
     ok = ok && hist.alloc(HIST_BINS) == cudaSuccess && sel.alloc(8) == cudaSuccess && tkey.alloc(m) == cudaSuccess &&
          tsim.alloc(m) == cudaSuccess && gcm.alloc(ncell * ndir) == cudaSuccess && tgrp.alloc(ml) == cudaSuccess &&
          cand.alloc(ml) == cudaSuccess && ckey.alloc(ml) == cudaSuccess && bcnt.alloc(MERGE_MAX_BLOCKS) == cudaSuccess &&
@@ -456,24 +456,17 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
          pref.alloc(2) == cudaSuccess && cell0.alloc(1) == cudaSuccess && rsim.alloc(1) == cudaSuccess &&
          lead_slot.alloc(ml) == cudaSuccess && lead_sim.alloc(ml) == cudaSuccess;
     if (!ok) return free_fail(FLEXRT_E_OOM, "probe_merge: device allocation failed");
-    // queue layout: structure of arrays, photons bin-major
-    auto queue = [&](int k) {
-        Queue q{};
-        q.pl = qpl[k].p; q.em = qem[k].p; q.bi = qbi[k].p;
-        q.dx = qd[k].p; q.dy = qd[k].p + mq; q.dz = qd[k].p + 2 * mq;
-        for (int b = 0; b < nb; ++b) q.ph[b] = qph[k].p + b * mq;
-        q.mx = qm[k].p; q.my = qm[k].p + mq; q.mz = qm[k].p + 2 * mq;
-        q.ma = qma[k].p; q.mthr = qthr[k].p;
-        return q;
-    };
-    const Queue q0 = queue(0), q1 = queue(1);
-    std::vector<int32_t> d3(3 * mq), m3(3 * mq);
-    std::vector<float> ph(nb * mq);
-    std::vector<uint32_t> ma(mq);
+    const Queue q0 = queue_at(qmem[0].p, mq, nb, true, nullptr), q1 = queue_at(qmem[1].p, mq, nb, true, nullptr);
+    std::vector<char> host(qbytes);
+    const Queue qh = queue_at(host.data(), mq, nb, true, nullptr);
     for (int64_t i = 0; i < n; ++i) {
-        for (int a = 0; a < 3; ++a) { d3[a * mq + i] = in->dir[3 * i + a]; m3[a * mq + i] = in->pos[3 * i + a]; }
-        for (int b = 0; b < nb; ++b) ph[b * mq + i] = in->photons[(size_t)nb * i + b];
-        ma[i] = in->aux[i] & 0x8000ffffu;              // simulation 0
+        const int32_t *d = in->dir + 3 * i, *x = in->pos + 3 * i;
+        qh.a[i] = make_uint4(in->emitter[i], (uint32_t)in->birth[i], (uint32_t)d[0], (uint32_t)d[1]);
+        *tail_word(qh, nb, 0, i) = (uint32_t)d[2];
+        *tail_word(qh, nb, 1, i) = in->pixlev[i];
+        for (int b = 0; b < nb; ++b) std::memcpy(tail_word(qh, nb, 2 + b, i), in->photons + (size_t)nb * i + b, 4);
+        qh.m[i] = make_uint4((uint32_t)x[0], (uint32_t)x[1], (uint32_t)x[2], in->aux[i] & 0x8000ffffu);   // simulation 0
+        qh.mthr[i] = in->thr[i];
     }
     std::vector<int4> ec(std::max(p->n_emitters, 1));
     for (int k = 0; k < p->n_emitters; ++k)
@@ -484,9 +477,7 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
         return bytes == 0 || cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     };
     ok = up(dctl.p, &ctl, sizeof(ctl)) && up(dsim.p, &h, sizeof(h)) && up(dacc.p, &acc, sizeof(acc)) &&
-         up(q1.pl, in->pixlev, n * 4) && up(q1.em, in->emitter, n * 4) && up(q1.bi, in->birth, n * 4) &&
-         up(qd[1].p, d3.data(), 3 * mq * 4) && up(qm[1].p, m3.data(), 3 * mq * 4) &&
-         up(qph[1].p, ph.data(), nb * mq * 4) && up(q1.ma, ma.data(), mq * 4) && up(q1.mthr, in->thr, n * 4) && up(ecell.p, ec.data(), ec.size() * sizeof(int4)) &&
+         up(qmem[1].p, host.data(), qbytes) && up(ecell.p, ec.data(), ec.size() * sizeof(int4)) &&
          up(n0.p, p->emitter_n0, p->n_emitters * sizeof(float)) && up(pref.p, pr, sizeof(pr)) &&
          up(cell0.p, &c0, sizeof(c0)) && up(rsim.p, &s0, sizeof(s0));
     ok = ok && cudaMemset(hist.p, 0, HIST_BINS * 4) == cudaSuccess && cudaMemset(sel.p, 0, 32) == cudaSuccess &&
@@ -509,34 +500,24 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
         return free_fail(FLEXRT_E_CUDA, "probe_merge: read-back failed");
     // the rays stay in queue 1; the merge leaves holes where its groups'
     // members were (skipped here) and appends the merged rays
-    const int k = 1;
     const long long cnt = std::min<long long>(hc.cnt[1], mq);
-    std::vector<uint32_t> opl(mq), oem(mq), oma(mq);
-    std::vector<int32_t> obi(mq), od(3 * mq), om(3 * mq);
-    std::vector<float> oph(nb * mq), othr(mq);
-    auto down = [](void *dst, const void *src, size_t bytes) {
-        return bytes == 0 || cudaMemcpy(dst, src, bytes, cudaMemcpyDeviceToHost) == cudaSuccess;
-    };
-    const Queue qq = k ? q1 : q0;
-    ok = down(opl.data(), qq.pl, mq * 4) && down(oem.data(), qq.em, mq * 4) && down(obi.data(), qq.bi, mq * 4) &&
-         down(od.data(), qd[k].p, 3 * mq * 4) && down(om.data(), qm[k].p, 3 * mq * 4) &&
-         down(oph.data(), qph[k].p, nb * mq * 4) && down(oma.data(), qq.ma, mq * 4) && down(othr.data(), qq.mthr, mq * 4);
-    if (!ok) return free_fail(FLEXRT_E_CUDA, "probe_merge: read-back failed");
+    HostRays hr;
+    if (read_queue(q1, nb, true, cnt, hr) != cudaSuccess) return free_fail(FLEXRT_E_CUDA, "probe_merge: read-back failed");
     long long o = 0;
     for (long long i = 0; i < cnt; ++i) {
-        if (opl[i] == DEAD_RAY) continue;
+        if (hr.pl[i] == DEAD_RAY) continue;
         if (o < cap) {
-            const bool mg = (oem[i] & 0x80000000u) != 0;
-            out->pixlev[o] = opl[i];
-            out->emitter[o] = oem[i];
-            out->birth[o] = obi[i];
+            const bool mg = (hr.em[i] & 0x80000000u) != 0;
+            out->pixlev[o] = hr.pl[i];
+            out->emitter[o] = hr.em[i];
+            out->birth[o] = hr.bi[i];
             for (int a2 = 0; a2 < 3; ++a2) {
-                out->dir[3 * o + a2] = od[a2 * mq + i];
-                out->pos[3 * o + a2] = mg ? om[a2 * mq + i] : 0;
+                out->dir[3 * o + a2] = hr.d[a2 * cnt + i];
+                out->pos[3 * o + a2] = mg ? hr.pos[a2 * cnt + i] : 0;
             }
-            for (int b = 0; b < nb; ++b) out->photons[(size_t)nb * o + b] = oph[b * mq + i];
-            out->aux[o] = mg ? (oma[i] & 0x8000ffffu) : 0u;
-            out->thr[o] = mg ? othr[i] : 0.0f;
+            for (int b = 0; b < nb; ++b) out->photons[(size_t)nb * o + b] = hr.ph[b * cnt + i];
+            out->aux[o] = mg ? (hr.ma[i] & 0x8000ffffu) : 0u;
+            out->thr[o] = mg ? hr.thr[i] : 0.0f;
         }
         ++o;
     }

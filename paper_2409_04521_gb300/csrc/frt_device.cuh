@@ -13,6 +13,8 @@
 namespace frt {
 
 constexpr unsigned FULL = 0xffffffffu;
+template <int N>
+struct Int { static constexpr int value = N; };
 __device__ __constant__ static const double DPI = 3.141592653589793238462643383279502884;
 
 // ---------------------------------------------------------------------------
@@ -500,6 +502,82 @@ __device__ __forceinline__ int warp_incl_scan(int x) {
         if (lane >= o) x += t;
     }
     return x;
+}
+
+// ---------------------------------------------------------------------------
+// Ray records (frt_types.h): tail words of one ray as vector pieces.  STREAM:
+// evict-first accesses (the queue streams through once per step, and the
+// cells' opacities and deposit buffers stay resident in L2).
+// ---------------------------------------------------------------------------
+template <int NB, bool STREAM>
+__device__ __forceinline__ void load_tail(const Queue &q, unsigned i, uint32_t (&w)[2 + NB]) {
+    constexpr int T = 2 + NB, N4 = T / 4;
+#pragma unroll
+    for (int k = 0; k < N4; ++k) {
+        const uint4 v = STREAM ? __ldcs(q.t4[k] + i) : q.t4[k][i];
+        w[4 * k] = v.x; w[4 * k + 1] = v.y; w[4 * k + 2] = v.z; w[4 * k + 3] = v.w;
+    }
+    if (T & 2) {
+        const uint2 v = STREAM ? __ldcs(q.t2 + i) : q.t2[i];
+        w[4 * N4] = v.x; w[4 * N4 + 1] = v.y;
+    }
+    if (T & 1) w[T - 1] = STREAM ? __ldcs(q.t1 + i) : q.t1[i];
+}
+template <int NB, bool STREAM>
+__device__ __forceinline__ void store_tail(const Queue &q, unsigned i, const uint32_t (&w)[2 + NB]) {
+    constexpr int T = 2 + NB, N4 = T / 4;
+#pragma unroll
+    for (int k = 0; k < N4; ++k) {
+        const uint4 v = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
+        if (STREAM) __stcs(q.t4[k] + i, v); else q.t4[k][i] = v;
+    }
+    if (T & 2) {
+        const uint2 v = make_uint2(w[4 * N4], w[4 * N4 + 1]);
+        if (STREAM) __stcs(q.t2 + i, v); else q.t2[i] = v;
+    }
+    if (T & 1) { if (STREAM) __stcs(q.t1 + i, w[T - 1]); else q.t1[i] = w[T - 1]; }
+}
+// the same for a bin count known at run time; words past the record are zero
+template <bool STREAM>
+__device__ __forceinline__ void load_tail_n(const Queue &q, int nb, unsigned i, uint32_t (&w)[2 + MAXB]) {
+#pragma unroll
+    for (int k = 0; k < 2 + MAXB; ++k) w[k] = 0u;
+    auto get = [&](auto tag) {
+        constexpr int NB = decltype(tag)::value;
+        uint32_t v[2 + NB];
+        load_tail<NB, STREAM>(q, i, v);
+#pragma unroll
+        for (int k = 0; k < 2 + NB; ++k) w[k] = v[k];
+    };
+    switch (nb) {
+        case 1: get(Int<1>()); break;
+        case 2: get(Int<2>()); break;
+        case 3: get(Int<3>()); break;
+        case 4: get(Int<4>()); break;
+        case 5: get(Int<5>()); break;
+        case 6: get(Int<6>()); break;
+        case 7: get(Int<7>()); break;
+        default: get(Int<8>()); break;
+    }
+}
+__device__ __forceinline__ void store_tail_n(const Queue &q, int nb, unsigned i, const uint32_t (&w)[2 + MAXB]) {
+    auto put = [&](auto tag) {
+        constexpr int NB = decltype(tag)::value;
+        uint32_t v[2 + NB];
+#pragma unroll
+        for (int k = 0; k < 2 + NB; ++k) v[k] = w[k];
+        store_tail<NB, false>(q, i, v);
+    };
+    switch (nb) {
+        case 1: put(Int<1>()); break;
+        case 2: put(Int<2>()); break;
+        case 3: put(Int<3>()); break;
+        case 4: put(Int<4>()); break;
+        case 5: put(Int<5>()); break;
+        case 6: put(Int<6>()); break;
+        case 7: put(Int<7>()); break;
+        default: put(Int<8>()); break;
+    }
 }
 
 // exact 2^-k for 0 <= k < 126

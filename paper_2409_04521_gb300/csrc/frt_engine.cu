@@ -50,6 +50,65 @@ size_t ray_bytes(int nb, bool merge) { return 6 * sizeof(int32_t) + (size_t)nb *
 
 }  // namespace
 
+Queue queue_at(void *base, long long cap, int nb, bool merged, size_t *bytes) {
+    Queue q{};
+    char *p = static_cast<char *>(base);
+    size_t tot = 0;
+    auto piece = [&](size_t per) {
+        char *r = p + tot;
+        tot += ((size_t)cap * per + 255) & ~(size_t)255;
+        return (void *)r;
+    };
+    const int T = 2 + nb;
+    q.a = (uint4 *)piece(16);
+    for (int k = 0; k < T / 4; ++k) q.t4[k] = (uint4 *)piece(16);
+    if (T & 2) q.t2 = (uint2 *)piece(8);
+    if (T & 1) q.t1 = (uint32_t *)piece(4);
+    if (merged) {
+        q.m = (uint4 *)piece(16);
+        q.mthr = (float *)piece(4);
+    }
+    if (bytes) *bytes = tot;
+    return q;
+}
+
+cudaError_t read_queue(const Queue &q, int nb, bool merged, long long n, HostRays &out) {
+    out.pl.resize(n); out.em.resize(n); out.bi.resize(n); out.d.resize(3 * n); out.ph.resize((size_t)nb * n);
+    out.ma.resize(merged ? n : 0); out.pos.resize(merged ? 3 * n : 0); out.thr.resize(merged ? n : 0);
+    if (n == 0) return cudaSuccess;
+    size_t bytes = 0;
+    queue_at(nullptr, n, nb, merged, &bytes);
+    std::vector<char> host(bytes);
+    const Queue h = queue_at(host.data(), n, nb, merged, nullptr);
+    cudaError_t e = cudaSuccess;
+    auto get = [&](void *dst, const void *src, size_t per) {
+        if (dst && e == cudaSuccess) e = cudaMemcpy(dst, src, (size_t)n * per, cudaMemcpyDeviceToHost);
+    };
+    get(h.a, q.a, 16);
+    for (int k = 0; k < 2; ++k) get(h.t4[k], q.t4[k], 16);
+    get(h.t2, q.t2, 8);
+    get(h.t1, q.t1, 4);
+    get(h.m, q.m, 16);
+    get(h.mthr, q.mthr, 4);
+    if (e != cudaSuccess) return e;
+    for (long long i = 0; i < n; ++i) {
+        out.pl[i] = *tail_word(h, nb, 1, i);
+        out.em[i] = h.a[i].x;
+        out.bi[i] = (int32_t)h.a[i].y;
+        out.d[i] = (int32_t)h.a[i].z;
+        out.d[n + i] = (int32_t)h.a[i].w;
+        out.d[2 * n + i] = (int32_t)*tail_word(h, nb, 0, i);
+        for (int b = 0; b < nb; ++b) std::memcpy(&out.ph[(size_t)b * n + i], tail_word(h, nb, 2 + b, i), 4);
+        if (merged) {
+            const uint4 m = h.m[i];
+            out.pos[i] = (int32_t)m.x; out.pos[n + i] = (int32_t)m.y; out.pos[2 * n + i] = (int32_t)m.z;
+            out.ma[i] = m.w;
+            out.thr[i] = h.mthr[i];
+        }
+    }
+    return cudaSuccess;
+}
+
 cudaError_t get_pixtab(int device, int level, cudaStream_t st, const int4 **out) {
     std::lock_guard<std::mutex> lk(g_tab_mu);
     PixTable &t = g_tabs[device];
@@ -198,33 +257,14 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
     if (cap >= (1LL << 31) - (1LL << 24)) return fail(FLEXRT_E_INVALID, "ray capacity above the 32-bit queue index");
     qcap_ = cap;
 
-    // ray queues: one allocation, structure of arrays, two buffers
+    // ray queues: one allocation, two buffers
     {
-        // each array starts on a 256-byte boundary (vector loads of the queue)
-        const size_t a = ((size_t)cap * 4 + 255) & ~(size_t)255, per = a * (ray_bytes(cfg_.nb, mrg) / 4);
+        size_t per = 0;
+        queue_at(nullptr, cap, cfg_.nb, mrg, &per);
         char *base = nullptr;
         if (dev_alloc((void **)&base, 2 * per + 256) != cudaSuccess) return fail(FLEXRT_E_OOM, "ray queue allocation failed");
         qmem_ = base;
-        for (int k = 0; k < 2; ++k) {
-            char *p = base + k * per;
-            q_[k].pl = (uint32_t *)p; p += a;
-            q_[k].em = (uint32_t *)p; p += a;
-            q_[k].bi = (int32_t *)p; p += a;
-            q_[k].dx = (int32_t *)p; p += a;
-            q_[k].dy = (int32_t *)p; p += a;
-            q_[k].dz = (int32_t *)p; p += a;
-            for (int b = 0; b < MAXB; ++b) {
-                q_[k].ph[b] = b < cfg_.nb ? (float *)p : nullptr;
-                if (b < cfg_.nb) p += a;
-            }
-            if (mrg) {
-                q_[k].mx = (int32_t *)p; p += a;
-                q_[k].my = (int32_t *)p; p += a;
-                q_[k].mz = (int32_t *)p; p += a;
-                q_[k].ma = (uint32_t *)p; p += a;
-                q_[k].mthr = (float *)p; p += a;
-            }
-        }
+        for (int k = 0; k < 2; ++k) q_[k] = queue_at(base + k * per, cap, cfg_.nb, mrg, nullptr);
     }
     const long long nc = cfg_.cell_capacity;
     const int ms = cfg_.max_sims;
@@ -1020,29 +1060,13 @@ flexrt_status Engine::rays(int s, int64_t cap, int32_t *level, int64_t *pixel, i
     const int qs = mid_step_ ? hc.par ^ 1 : hc.par;     // between the stages: the march's output
     const long long m = hc.cnt[qs];
     if (mid_step_) *n = 0;
-    if (m == 0 || cap == 0) {
-        if (mid_step_ && m > 0) {
-            std::vector<uint32_t> pl(m), em(m), ma(merge_built() ? m : 0);
-            CK(cudaMemcpy(pl.data(), q_[qs].pl, m * 4, cudaMemcpyDeviceToHost));
-            CK(cudaMemcpy(em.data(), q_[qs].em, m * 4, cudaMemcpyDeviceToHost));
-            if (!ma.empty()) CK(cudaMemcpy(ma.data(), q_[qs].ma, m * 4, cudaMemcpyDeviceToHost));
-            *n = (int64_t)member_rays(pl, em, ma, s, sl->em0, sl->em_n).size();
-        }
-        return FLEXRT_OK;
-    }
-    const Queue &q = q_[qs];
-    std::vector<uint32_t> pl(m), em(m), ma(merge_built() ? m : 0);
-    std::vector<int32_t> bi(m), d(3 * m);
-    CK(cudaMemcpy(pl.data(), q.pl, m * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(em.data(), q.em, m * 4, cudaMemcpyDeviceToHost));
-    if (!ma.empty()) CK(cudaMemcpy(ma.data(), q.ma, m * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(bi.data(), q.bi, m * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(d.data(), q.dx, m * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(d.data() + m, q.dy, m * 4, cudaMemcpyDeviceToHost));
-    CK(cudaMemcpy(d.data() + 2 * m, q.dz, m * 4, cudaMemcpyDeviceToHost));
-    std::vector<std::vector<float>> ph(photons ? sl->h.nb : 0, std::vector<float>(m));
-    for (int b = 0; b < (int)ph.size(); ++b) CK(cudaMemcpy(ph[b].data(), q.ph[b], m * 4, cudaMemcpyDeviceToHost));
-    const std::vector<long long> idx = member_rays(pl, em, ma, s, sl->em0, sl->em_n);
+    if (m == 0 || (cap == 0 && !mid_step_)) return FLEXRT_OK;
+    HostRays hr;
+    CK(read_queue(q_[qs], cfg_.nb, merge_built(), m, hr));
+    const std::vector<uint32_t> &pl = hr.pl, &em = hr.em;
+    const std::vector<int32_t> &bi = hr.bi, &d = hr.d;
+    const int nph = photons ? sl->h.nb : 0;
+    const std::vector<long long> idx = member_rays(pl, em, hr.ma, s, sl->em0, sl->em_n);
     if (mid_step_) *n = (int64_t)idx.size();
     for (long long k = 0; k < (long long)idx.size() && k < cap; ++k) {
         const long long i = idx[k];
@@ -1052,7 +1076,7 @@ flexrt_status Engine::rays(int s, int64_t cap, int32_t *level, int64_t *pixel, i
             emitter[k] = (em[i] & MERGED_BIT) ? -1 - (int32_t)(em[i] & ~MERGED_BIT) : (int32_t)(em[i] - sl->em0);
         if (birth) birth[k] = bi[i];
         if (dir) { dir[3 * k] = d[i]; dir[3 * k + 1] = d[m + i]; dir[3 * k + 2] = d[2 * m + i]; }
-        for (int b = 0; b < (int)ph.size(); ++b) photons[(size_t)sl->h.nb * k + b] = (double)ph[b][i] * sl->h.nref;
+        for (int b = 0; b < nph; ++b) photons[(size_t)sl->h.nb * k + b] = (double)hr.ph[(size_t)b * m + i] * sl->h.nref;
     }
     return FLEXRT_OK;
 }
@@ -1066,22 +1090,10 @@ flexrt_status Engine::rays_merged(int s, int64_t cap, int32_t *merged, int32_t *
     CK(cudaMemcpy(&hc, ctl_, sizeof(hc), cudaMemcpyDeviceToHost));
     const int qs = mid_step_ ? hc.par ^ 1 : hc.par;
     const long long m = hc.cnt[qs];
-    const Queue &q = q_[qs];
-    std::vector<uint32_t> pl(m), em(m), ma(merge_built() ? m : 0);
-    std::vector<int32_t> mx(ma.size()), my(ma.size()), mz(ma.size());
-    std::vector<float> mt(ma.size());
-    if (m > 0) {
-        CK(cudaMemcpy(pl.data(), q.pl, m * 4, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(em.data(), q.em, m * 4, cudaMemcpyDeviceToHost));
-    }
-    if (!ma.empty()) {
-        CK(cudaMemcpy(ma.data(), q.ma, m * 4, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(mx.data(), q.mx, m * 4, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(my.data(), q.my, m * 4, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(mz.data(), q.mz, m * 4, cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(mt.data(), q.mthr, m * 4, cudaMemcpyDeviceToHost));
-    }
-    const std::vector<long long> idx = member_rays(pl, em, ma, s, sl->em0, sl->em_n);
+    HostRays hr;
+    CK(read_queue(q_[qs], cfg_.nb, merge_built(), m, hr));
+    const std::vector<uint32_t> &em = hr.em, &ma = hr.ma;
+    const std::vector<long long> idx = member_rays(hr.pl, em, ma, s, sl->em0, sl->em_n);
     *n = (int64_t)idx.size();
     for (long long k = 0; k < (long long)idx.size() && k < cap; ++k) {
         const long long i = idx[k];
@@ -1090,9 +1102,9 @@ flexrt_status Engine::rays_merged(int s, int64_t cap, int32_t *merged, int32_t *
         if (vertex) vertex[k] = mg && (ma[i] >> 31) ? 1 : 0;
         if (dist) dist[k] = mg ? (int32_t)(ma[i] & 0xffffu) : 0;
         if (pos) {
-            pos[3 * k] = mg ? mx[i] : 0; pos[3 * k + 1] = mg ? my[i] : 0; pos[3 * k + 2] = mg ? mz[i] : 0;
+            for (int a = 0; a < 3; ++a) pos[3 * k + a] = mg ? hr.pos[a * m + i] : 0;
         }
-        if (thr) thr[k] = mg ? (double)mt[i] * sl->h.nref : 0.0;
+        if (thr) thr[k] = mg ? (double)hr.thr[i] * sl->h.nref : 0.0;
     }
     return FLEXRT_OK;
 }
@@ -1217,14 +1229,10 @@ flexrt_status Engine::save_state(int s, void *buf, int64_t cap, int64_t *bytes) 
         {cells_.rho + sl->cell0, nc * 4},
         {em_.n0 + sl->em0, (size_t)ne * 4}, {em_.ring + sl->em0 * rw * 3, (size_t)ne * rw * 3 * sizeof(int4)}};
     if (ne == 0) { parts[8].second = 0; parts[9].second = 0; }
-    const Queue &q = q_[hc.par];
-    const void *qa[] = {q.pl, q.em, q.bi, q.dx, q.dy, q.dz};
-    for (const void *a : qa) parts.push_back({a, (size_t)nray * 4});
-    for (int b = 0; b < nb; ++b) parts.push_back({q.ph[b], (size_t)nray * 4});
-    if (mf) {
-        const void *ma[] = {q.mx, q.my, q.mz, q.ma, q.mthr};
-        for (const void *a : ma) parts.push_back({a, (size_t)nray * 4});
-    }
+    // the records as one array a word, in the other queue's memory (unused
+    // between steps)
+    const int words = 6 + nb + (mf ? 5 : 0);
+    parts.push_back({q_[hc.par ^ 1].a, (size_t)nray * words * 4});
     size_t tot = sizeof(StateHeader);
     for (auto &p : parts) tot += p.second;
     *bytes = (int64_t)tot;
@@ -1241,6 +1249,8 @@ flexrt_status Engine::save_state(int s, void *buf, int64_t cap, int64_t *bytes) 
     char *o = (char *)buf;
     std::memcpy(o, &h, sizeof(h));
     o += sizeof(h);
+    CK(launch_queue_words(q_[hc.par], nb, mf, nray, reinterpret_cast<uint32_t *>(q_[hc.par ^ 1].a), false, st_));
+    CK(cudaStreamSynchronize(st_));
     for (auto &p : parts) {
         if (p.second) CK(cudaMemcpy(o, p.first, p.second, cudaMemcpyDeviceToHost));
         o += p.second;
@@ -1271,14 +1281,8 @@ flexrt_status Engine::load_state(int s, const void *buf, int64_t bytes) {
         {cells_.rho + sl->cell0, nc * 4},
         {em_.n0 + sl->em0, (size_t)ne * 4}, {em_.ring + sl->em0 * rw * 3, (size_t)ne * rw * 3 * sizeof(int4)}};
     if (ne == 0) { parts[8].second = 0; parts[9].second = 0; }
-    const Queue &q = q_[0];
-    void *qa[] = {q.pl, q.em, q.bi, q.dx, q.dy, q.dz};
-    for (void *a : qa) parts.push_back({a, (size_t)nray * 4});
-    for (int b = 0; b < nb; ++b) parts.push_back({q.ph[b], (size_t)nray * 4});
-    if (merge_built()) {
-        void *ma[] = {q.mx, q.my, q.mz, q.ma, q.mthr};
-        for (void *a : ma) parts.push_back({a, (size_t)nray * 4});
-    }
+    const int words = 6 + nb + (merge_built() ? 5 : 0);
+    parts.push_back({q_[1].a, (size_t)nray * words * 4});      // one array a word, joined into queue 0 below
     size_t tot = sizeof(StateHeader);
     for (auto &p : parts) tot += p.second;
     if ((int64_t)tot != bytes) return fail(FLEXRT_E_INVALID, "checkpoint size does not match its header");
@@ -1288,6 +1292,7 @@ flexrt_status Engine::load_state(int s, const void *buf, int64_t bytes) {
         if (p.second) CK(cudaMemcpy(p.first, src, p.second, cudaMemcpyHostToDevice));
         src += p.second;
     }
+    CK(launch_queue_words(q_[0], nb, merge_built(), nray, reinterpret_cast<uint32_t *>(q_[1].a), true, st_));
     // the live rays in queue 0, nothing in flight in queue 1, no latched error
     const long long cnt[2] = {nray, 0};
     const int32_t par_err[2] = {0, 0};

@@ -15,6 +15,19 @@ namespace frt {
 // Process-wide fixed-point pixel-vector table of levels 0..level on `device`.
 cudaError_t get_pixtab(int device, int level, cudaStream_t st, const int4 **out);
 
+// The pieces of a queue of cap records (frt_types.h) placed one after another
+// from `base`, each on a 256-byte boundary; *bytes gets their total.  Works
+// on host and device addresses.
+Queue queue_at(void *base, long long cap, int nb, bool merged, size_t *bytes);
+
+// Host copy of a queue's first n records, one array a word.
+struct HostRays {
+    std::vector<uint32_t> pl, em, ma;
+    std::vector<int32_t> bi, d, pos;               // d: n of dx, then dy, then dz; pos likewise
+    std::vector<float> ph, thr;                    // ph: n of each bin
+};
+cudaError_t read_queue(const Queue &q, int nb, bool merged, long long n, HostRays &out);
+
 // First-fit allocator of [0, capacity) index ranges.
 class RangeAllocator {
   public:

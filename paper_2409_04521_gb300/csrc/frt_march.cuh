@@ -210,46 +210,31 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
         float t_esc = 0.0f, t_out = 0.0f;
         unsigned t_cnt = 0u, t_rout = 0u;
         int t_sim = -1, t_n = 0;
-        // the ray's words, loaded at the top of its iteration (loading the next
-        // ray's one iteration ahead cost more in spilled registers than it hid)
-        uint32_t npl = DEAD_RAY, ne_ = 0;
-        int nbi = 0, ndx = 0, ndy = 0, ndz = 0;
-        float nph[NB];
-        int nmx = 0, nmy = 0, nmz = 0;
-        uint32_t nma = 0;
-        float nmthr = 0.0f;
-        auto load_ray = [&](unsigned j) {
-            // the queue streams through once per step: evict-first loads keep
-            // the cells' opacities and deposit buffers resident in L2
-            npl = DEAD_RAY;
-            if (j < n) npl = __ldcs(qi.pl + j);
-            if (npl != DEAD_RAY) {
-                ne_ = __ldcs(qi.em + j); nbi = __ldcs(qi.bi + j);
-                ndx = __ldcs(qi.dx + j); ndy = __ldcs(qi.dy + j); ndz = __ldcs(qi.dz + j);
-#pragma unroll
-                for (int b = 0; b < NB; ++b) nph[b] = __ldcs(qi.ph[b] + j);
-                if (MRG && (ne_ & MERGED_BIT)) {
-                    nmx = __ldcs(qi.mx + j); nmy = __ldcs(qi.my + j); nmz = __ldcs(qi.mz + j);
-                    nma = __ldcs(qi.ma + j); nmthr = __ldcs(qi.mthr + j);
-                }
-            } else {
-                ne_ = 0; nbi = 0; ndx = ndy = ndz = 0;
-#pragma unroll
-                for (int b = 0; b < NB; ++b) nph[b] = 0.0f;
-            }
-        };
         for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < nr; i += stride) {
-            load_ray(i);
-            const uint32_t pl = npl, e = ne_;
-            const int bi = nbi, dx = ndx, dy = ndy, dz = ndz;
-            const int mx = nmx, my = nmy, mz = nmz;
-            const uint32_t ma = nma;
-            const float mthr = nmthr;
+            // the ray's words: every piece at once, the pixel word among them
+            // (a dead slot's other words are old ones, and are not used)
+            uint4 ra = make_uint4(0u, 0u, 0u, 0u);
+            uint32_t w[2 + NB];
+            w[1] = DEAD_RAY;
+            if (i < n) {
+                ra = __ldcs(qi.a + i);
+                load_tail<NB, true>(qi, i, w);
+            }
+            const uint32_t e = ra.x, pl = w[1];
+            const int bi = (int)ra.y, dx = (int)ra.z, dy = (int)ra.w, dz = (int)w[0];
             float ph[NB];
 #pragma unroll
-            for (int b = 0; b < NB; ++b) ph[b] = nph[b];
+            for (int b = 0; b < NB; ++b) ph[b] = __uint_as_float(w[2 + b]);
             bool valid = pl != DEAD_RAY;
             const bool mrg = MRG && valid && (e & MERGED_BIT);
+            int mx = 0, my = 0, mz = 0;
+            uint32_t ma = 0;
+            float mthr = 0.0f;
+            if (mrg) {
+                const uint4 rm = __ldcs(qi.m + i);
+                mx = (int)rm.x; my = (int)rm.y; mz = (int)rm.z; ma = rm.w;
+                mthr = __ldcs(qi.mthr + i);
+            }
             int sim = 0;
             int4 ec = make_int4(0, 0, 0, 0);
             if (mrg) {
@@ -449,13 +434,13 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                     };
                     if (nout == 1) {
                         const unsigned o = slot_of(k0);
-                        __stcs(qo.pl + o, pl); __stcs(qo.em + o, e); __stcs(qo.bi + o, bi);
-                        __stcs(qo.dx + o, dx); __stcs(qo.dy + o, dy); __stcs(qo.dz + o, dz);
+                        __stcs(qo.a + o, ra);
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) __stcs(qo.ph[b] + o, ph[b]);
+                        for (int b = 0; b < NB; ++b) w[2 + b] = __float_as_uint(ph[b]);
+                        store_tail<NB, true>(qo, o, w);
                         if (mrg) {
-                            __stcs(qo.mx + o, mx); __stcs(qo.my + o, my); __stcs(qo.mz + o, mz);
-                            __stcs(qo.ma + o, ma); __stcs(qo.mthr + o, mthr);
+                            __stcs(qo.m + o, make_uint4((uint32_t)mx, (uint32_t)my, (uint32_t)mz, ma));
+                            __stcs(qo.mthr + o, mthr);
                         }
                     } else {
                         const int L = lev + m;
@@ -472,9 +457,9 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                         }
                         const bool vert = mrg && (ma >> 31);
                         const float scale = pow2_neg(2 * m);
-                        float cph[NB];
+                        uint32_t cw[2 + NB];
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) cph[b] = ph[b] * scale;
+                        for (int b = 0; b < NB; ++b) cw[2 + b] = __float_as_uint(ph[b] * scale);
                         for (int c = 0; c < nout; ++c) {
                             const uint32_t pix = vert ? vertex_child(S.l_merge, pl & PIX_MASK, lev, m, (uint32_t)c)
                                                       : pix0 + (uint32_t)c;
@@ -482,14 +467,12 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                             int32_t cx, cy, cz;
                             rotate_dir(rows, vq, cx, cy, cz);
                             const unsigned oc = slot_of(k0 + c);
-                            qo.pl[oc] = ((uint32_t)L << LEVEL_SHIFT) | pix;
-                            qo.em[oc] = e; qo.bi[oc] = bi;
-                            qo.dx[oc] = cx; qo.dy[oc] = cy; qo.dz[oc] = cz;
-#pragma unroll
-                            for (int b = 0; b < NB; ++b) qo.ph[b][oc] = cph[b];
+                            cw[0] = (uint32_t)cz;
+                            cw[1] = ((uint32_t)L << LEVEL_SHIFT) | pix;
+                            qo.a[oc] = make_uint4(e, (uint32_t)bi, (uint32_t)cx, (uint32_t)cy);
+                            store_tail<NB, false>(qo, oc, cw);
                             if (mrg) {
-                                qo.mx[oc] = mx; qo.my[oc] = my; qo.mz[oc] = mz;
-                                qo.ma[oc] = ma & 0x7fffffffu;
+                                qo.m[oc] = make_uint4((uint32_t)mx, (uint32_t)my, (uint32_t)mz, ma & 0x7fffffffu);
                                 qo.mthr[oc] = mthr * scale;
                             }
                         }
@@ -498,7 +481,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             }
             ++w_it;
         }
-        for (int k = lane; k < slab_left; k += 32) qo.pl[slab + k] = DEAD_RAY;
+        for (int k = lane; k < slab_left; k += 32) *pixel_word(qo, NB, slab + k) = DEAD_RAY;
         flush_tallies(t_esc, t_out, t_cnt, t_rout, t_sim, sh_acc);
     }
     __syncthreads();

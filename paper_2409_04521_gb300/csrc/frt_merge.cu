@@ -118,7 +118,7 @@ __device__ __forceinline__ void hist_add(uint32_t *hist, long long bin) {
 
 // the simulation a queued ray belongs to
 __device__ __forceinline__ int ray_sim(const Queue &q, const Emitters &em, long long i, uint32_t e) {
-    return (e & MERGED_BIT) ? (int)((q.ma[i] >> 16) & 0x7fffu) : __ldg(&em.cell[e]).w;
+    return (e & MERGED_BIT) ? (int)((q.m[i].w >> 16) & 0x7fffu) : __ldg(&em.cell[e]).w;
 }
 
 // whether a block of a pass with barriers runs: the control words are read
@@ -257,11 +257,10 @@ __global__ void __launch_bounds__(256) k_mhist1(MergeArgs A) {
         if (i < n) {
             // the ray's words together (a single simulation needs no
             // emitter lookup); bins past a member's own are zero
-            const uint32_t pl = q.pl[i];
-            const uint32_t e = A.nsims > 1 ? q.em[i] : 0u;
-            float ph[MAXB];
-#pragma unroll
-            for (int b = 0; b < MAXB; ++b) ph[b] = b < A.nbq ? q.ph[b][i] : 0.0f;
+            const uint32_t e = A.nsims > 1 ? q.a[i].x : 0u;
+            uint32_t w[2 + MAXB];
+            load_tail_n<false>(q, A.nbq, (unsigned)i, w);
+            const uint32_t pl = w[1];
             int sim = -1;
             uint32_t key = 0;
             if (pl != DEAD_RAY) {
@@ -269,7 +268,7 @@ __global__ void __launch_bounds__(256) k_mhist1(MergeArgs A) {
                 if (merges(A.sims[s], A.acc[s])) {
                     float T = 0.0f;
 #pragma unroll
-                    for (int b = 0; b < MAXB; ++b) T += ph[b];
+                    for (int b = 0; b < MAXB; ++b) T += __uint_as_float(w[2 + b]);
                     key = __float_as_uint(T);
                     sim = s;
                     bin = hist_row(A.w, s) + (key >> 16);
@@ -535,17 +534,21 @@ __global__ void __launch_bounds__(256, 4) k_mgroup(MergeArgs A) {
             const uint32_t tref = sel[SEL_T];
             if (sel[SEL_STATE] == SEL_DONE && !(sel[SEL_EXEMPT] && key >= tref)) {
                 const SimDev &S = A.sims[sim];
-                const uint32_t e = q.em[i], pl = q.pl[i];
-                const int bi = q.bi[i];
-                const int dx = q.dx[i], dy = q.dy[i], dz = q.dz[i];
+                const uint4 ra = q.a[i];
+                const uint32_t e = ra.x;
+                const int bi = (int)ra.y, dx = (int)ra.z, dy = (int)ra.w;
+                const uint2 rt = A.nbq >= 2 ? *reinterpret_cast<const uint2 *>(q.t4[0] + i) : q.t2[i];
+                const int dz = (int)rt.x;
+                const uint32_t pl = rt.y;
                 const int lev = (int)(pl >> LEVEL_SHIFT);
                 // end point of this step's march and the distance travelled
                 long long p[3];
                 int dist;
                 if (e & MERGED_BIT) {
                     const long long k = S.step - bi;
-                    p[0] = q.mx[i] + k * dx; p[1] = q.my[i] + k * dy; p[2] = q.mz[i] + k * dz;
-                    dist = (int)(q.ma[i] & 0xffffu) + (int)k;
+                    const uint4 rm = q.m[i];
+                    p[0] = (int)rm.x + k * dx; p[1] = (int)rm.y + k * dy; p[2] = (int)rm.z + k * dz;
+                    dist = (int)(rm.w & 0xffffu) + (int)k;
                 } else {
                     const int4 ec = __ldg(&A.em.cell[e]);
                     const long long k = S.step - bi + 1;
@@ -636,18 +639,20 @@ __global__ void __launch_bounds__(256, 4) k_mweight(MergeArgs A) {
         if (slot >= 0) {
             sim = A.nsims > 1 ? A.w.tsim[qi] : 0;
             const SimDev &S = A.sims[sim];
-            const uint32_t e = q.em[qi];
+            const uint32_t e = q.a[qi].x;
             nbf = S.nb;
+            uint32_t w[2 + MAXB];
+            load_tail_n<false>(q, A.nbq, qi, w);
 #pragma unroll
             for (int b = 0; b < MAXB; ++b)
-                if (b < nbf) f[b] = q.ph[b][qi];
+                if (b < nbf) f[b] = __uint_as_float(w[2 + b]);
             const int lev = (int)((pk.y >> 21) & 0xfu);
             const float thr = (e & MERGED_BIT) ? q.mthr[qi]
                                                : S.eps_term * __ldg(&A.em.n0[e]) * pow2_neg(2 * (lev - S.l_src));
 #pragma unroll
             for (int b = 0; b <= MAXB; ++b)
                 if (b == nbf) f[b] = thr;
-            q.pl[qi] = DEAD_RAY;
+            *pixel_word(q, A.nbq, qi) = DEAD_RAY;
         }
         unsigned long long v[GSUMS] = {0, 0, 0, 0, 0, 0};
         if (slot >= 0) {
@@ -789,15 +794,15 @@ __global__ void __launch_bounds__(256, 4) k_memit(MergeArgs A) {
         int32_t dx, dy, dz;
         rotate_dir(rows, vq, dx, dy, dz);
         const long long o = mbase + (long long)pre + j;
-        q.pl[o] = ((uint32_t)L2 << LEVEL_SHIFT) | pm;
-        q.em[o] = MERGED_BIT | (uint32_t)local;
-        q.bi[o] = S.step;
-        q.dx[o] = dx; q.dy[o] = dy; q.dz[o] = dz;
+        uint32_t w[2 + MAXB];
+        w[0] = (uint32_t)dz;
+        w[1] = ((uint32_t)L2 << LEVEL_SHIFT) | pm;
 #pragma unroll
-        for (int b = 0; b < MAXB; ++b)
-            if (b < nbq) q.ph[b][o] = b < S.nb ? gph[b] : 0.0f;
-        q.mx[o] = P[0]; q.my[o] = P[1]; q.mz[o] = P[2];
-        q.ma[o] = (L2 > S.l_merge ? 0x80000000u : 0u) | ((uint32_t)sim << 16) | (uint32_t)Adist;
+        for (int b = 0; b < MAXB; ++b) w[2 + b] = __float_as_uint(b < S.nb ? gph[b] : 0.0f);
+        q.a[o] = make_uint4(MERGED_BIT | (uint32_t)local, (uint32_t)S.step, (uint32_t)dx, (uint32_t)dy);
+        store_tail_n(q, nbq, (unsigned)o, w);
+        q.m[o] = make_uint4((uint32_t)P[0], (uint32_t)P[1], (uint32_t)P[2],
+                            (L2 > S.l_merge ? 0x80000000u : 0u) | ((uint32_t)sim << 16) | (uint32_t)Adist);
         q.mthr[o] = gph[S.nb];
         // the group is cleared for the next step
         float4 *gz = reinterpret_cast<float4 *>(gp);

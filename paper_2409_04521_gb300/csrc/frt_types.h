@@ -104,18 +104,38 @@ struct Ctl {
     long long pad2;
 };
 
-// Structure-of-arrays ray queue.
+// Ray queue.  A record is 6 + nb words -- emitter, birth step, direction (dx,
+// dy, dz), level << 28 | NESTED pixel, photons per bin -- kept in arrays of
+// 16-, 8- and 4-byte pieces, so that a warp reads or writes a record in a few
+// coalesced vector accesses (three at four bins, where an array a word took
+// ten, with ten addresses):
+//   a   emitter id, birth step, dx, dy
+//   the tail words dz, pixel word, photons[0..nb): as many 16-byte pieces t4
+//   as they fill, then an 8-byte piece t2 and a 4-byte piece t1 for the rest
+// Merged rays only (Sec. 3.3; null when merging is not built in):
+//   m   position at the merge (2^-21 cell), vertex << 31 | simulation << 16 |
+//       distance travelled at the merge
+//   mthr  termination threshold, code photons
 struct Queue {
-    uint32_t *pl;            // level << 28 | NESTED pixel
-    uint32_t *em;            // emitter id
-    int32_t *bi;             // birth step
-    int32_t *dx, *dy, *dz;   // direction, 2^-21 cell per step
-    float *ph[MAXB];         // code photons per bin
-    // merged rays only (Sec. 3.3); null when merging is not built in
-    int32_t *mx, *my, *mz;   // position at the merge, 2^-21 cell
-    uint32_t *ma;            // vertex << 31 | simulation << 16 | distance travelled at the merge
-    float *mthr;             // termination threshold, code photons
+    uint4 *a;
+    uint4 *t4[2];
+    uint2 *t2;
+    uint32_t *t1;
+    uint4 *m;
+    float *mthr;
 };
+
+// tail word w (0: dz, 1: pixel word, 2 + b: photons of bin b) of ray i
+__host__ __device__ inline uint32_t *tail_word(const Queue &q, int nb, int w, long long i) {
+    const int n4 = (2 + nb) >> 2;
+    if (w < 4 * n4) return reinterpret_cast<uint32_t *>(q.t4[w >> 2] + i) + (w & 3);
+    if (((2 + nb) & 2) && w < 4 * n4 + 2) return reinterpret_cast<uint32_t *>(q.t2 + i) + (w - 4 * n4);
+    return q.t1 + i;
+}
+// the pixel word of ray i (DEAD_RAY marks an unused slot)
+__host__ __device__ inline uint32_t *pixel_word(const Queue &q, int nb, long long i) {
+    return nb >= 2 ? reinterpret_cast<uint32_t *>(q.t4[0] + i) + 1 : reinterpret_cast<uint32_t *>(q.t2 + i) + 1;
+}
 
 struct Cells {
     double *nH;              // cm^-3 physical
