@@ -444,8 +444,7 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
     DevBuf<int4> ecell, rot;
     DevBuf<long long> pref, cell0;
     bool ok = dctl.alloc(1) == cudaSuccess && dsim.alloc(1) == cudaSuccess && dacc.alloc(1) == cudaSuccess;
-    size_t qbytes = 0;
-    queue_at(nullptr, mq, nb, true, &qbytes);
+    const size_t qbytes = queue_bytes(mq, nb, true);
     for (int k = 0; k < 2 && ok; ++k) ok = qmem[k].alloc(qbytes) == cudaSuccess;
     ok = ok && hist.alloc(HIST_BINS) == cudaSuccess && sel.alloc(8) == cudaSuccess && tkey.alloc(m) == cudaSuccess &&
          tsim.alloc(m) == cudaSuccess && gcm.alloc(ncell * ndir) == cudaSuccess && tgrp.alloc(ml) == cudaSuccess &&
@@ -456,17 +455,17 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
          pref.alloc(2) == cudaSuccess && cell0.alloc(1) == cudaSuccess && rsim.alloc(1) == cudaSuccess &&
          lead_slot.alloc(ml) == cudaSuccess && lead_sim.alloc(ml) == cudaSuccess;
     if (!ok) return free_fail(FLEXRT_E_OOM, "probe_merge: device allocation failed");
-    const Queue q0 = queue_at(qmem[0].p, mq, nb, true, nullptr), q1 = queue_at(qmem[1].p, mq, nb, true, nullptr);
+    const Queue q0 = queue_at(qmem[0].p, nb, true), q1 = queue_at(qmem[1].p, nb, true);
     std::vector<char> host(qbytes);
-    const Queue qh = queue_at(host.data(), mq, nb, true, nullptr);
+    const Queue qh = queue_at(host.data(), nb, true);
     for (int64_t i = 0; i < n; ++i) {
         const int32_t *d = in->dir + 3 * i, *x = in->pos + 3 * i;
-        qh.a[i] = make_uint4(in->emitter[i], (uint32_t)in->birth[i], (uint32_t)d[0], (uint32_t)d[1]);
-        *tail_word(qh, nb, 0, i) = (uint32_t)d[2];
-        *tail_word(qh, nb, 1, i) = in->pixlev[i];
-        for (int b = 0; b < nb; ++b) std::memcpy(tail_word(qh, nb, 2 + b, i), in->photons + (size_t)nb * i + b, 4);
-        qh.m[i] = make_uint4((uint32_t)x[0], (uint32_t)x[1], (uint32_t)x[2], in->aux[i] & 0x8000ffffu);   // simulation 0
-        qh.mthr[i] = in->thr[i];
+        *ray_head(qh, i) = make_uint4(in->emitter[i], (uint32_t)in->birth[i], (uint32_t)d[0], (uint32_t)d[1]);
+        *tail_word(qh, 0, i) = (uint32_t)d[2];
+        *pixel_word(qh, i) = in->pixlev[i];
+        for (int b = 0; b < nb; ++b) std::memcpy(tail_word(qh, 2 + b, i), in->photons + (size_t)nb * i + b, 4);
+        *ray_merge(qh, i) = make_uint4((uint32_t)x[0], (uint32_t)x[1], (uint32_t)x[2], in->aux[i] & 0x8000ffffu);   // simulation 0
+        *ray_thr(qh, i) = in->thr[i];
     }
     std::vector<int4> ec(std::max(p->n_emitters, 1));
     for (int k = 0; k < p->n_emitters; ++k)
@@ -502,7 +501,7 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
     // members were (skipped here) and appends the merged rays
     const long long cnt = std::min<long long>(hc.cnt[1], mq);
     HostRays hr;
-    if (read_queue(q1, nb, true, cnt, hr) != cudaSuccess) return free_fail(FLEXRT_E_CUDA, "probe_merge: read-back failed");
+    if (read_queue(q1, true, cnt, hr) != cudaSuccess) return free_fail(FLEXRT_E_CUDA, "probe_merge: read-back failed");
     long long o = 0;
     for (long long i = 0; i < cnt; ++i) {
         if (hr.pl[i] == DEAD_RAY) continue;

@@ -168,18 +168,17 @@ __device__ inline void rotation_rows(uint64_t seed, long long e, long long s, in
     for (int r = 0; r < 3; ++r) rows[r] = make_int4(q[3 * r], q[3 * r + 1], q[3 * r + 2], 0);
 }
 
-// round(X / 2^27), ties to even (X = Rq . vq, 2^48 scale -> 2^21 scale)
-__device__ __forceinline__ int32_t rne_shift27(long long X) {
-    long long q = X >> 27;                 // arithmetic shift = floor
-    long long r = X - (q << 27);
-    const long long half = 1LL << 26;
-    q += (r > half) | ((r == half) & (q & 1));
-    return (int32_t)q;
+// one component of Rq . vq (2^48 scale) in 2^21 scale: round(X / 2^27), ties to
+// even.  Half is added by the first product; a tie then leaves 27 zero bits.
+__device__ __forceinline__ int32_t rotate_row(int4 r, int4 v) {
+    const long long X = (long long)r.x * v.x + (1LL << 26) + (long long)r.y * v.y + (long long)r.z * v.z;
+    const int32_t q = (int32_t)(X >> 27);                // arithmetic shift = floor
+    return ((uint32_t)X & ((1u << 27) - 1u)) == 0u ? q & ~1 : q;
 }
 __device__ __forceinline__ void rotate_dir(const int4 rows[3], int4 v, int32_t &dx, int32_t &dy, int32_t &dz) {
-    dx = rne_shift27((long long)rows[0].x * v.x + (long long)rows[0].y * v.y + (long long)rows[0].z * v.z);
-    dy = rne_shift27((long long)rows[1].x * v.x + (long long)rows[1].y * v.y + (long long)rows[1].z * v.z);
-    dz = rne_shift27((long long)rows[2].x * v.x + (long long)rows[2].y * v.y + (long long)rows[2].z * v.z);
+    dx = rotate_row(rows[0], v);
+    dy = rotate_row(rows[1], v);
+    dz = rotate_row(rows[2], v);
 }
 
 // ---------------------------------------------------------------------------
@@ -505,51 +504,61 @@ __device__ __forceinline__ int warp_incl_scan(int x) {
 }
 
 // ---------------------------------------------------------------------------
-// Ray records (frt_types.h): tail words of one ray as vector pieces.  STREAM:
+// Ray records (frt_types.h): tail words of record r of a tile as vector pieces.  STREAM:
 // evict-first accesses (the queue streams through once per step, and the
 // cells' opacities and deposit buffers stay resident in L2).
 // ---------------------------------------------------------------------------
 template <int NB, bool STREAM>
-__device__ __forceinline__ void load_tail(const Queue &q, unsigned i, uint32_t (&w)[2 + NB]) {
+__device__ __forceinline__ void load_tail(const char *tile, unsigned r, uint32_t (&w)[2 + NB]) {
     constexpr int T = 2 + NB, N4 = T / 4;
 #pragma unroll
     for (int k = 0; k < N4; ++k) {
-        const uint4 v = STREAM ? __ldcs(q.t4[k] + i) : q.t4[k][i];
+        const uint4 *p = reinterpret_cast<const uint4 *>(tile + 512 * (1 + k)) + r;
+        const uint4 v = STREAM ? __ldcs(p) : *p;
         w[4 * k] = v.x; w[4 * k + 1] = v.y; w[4 * k + 2] = v.z; w[4 * k + 3] = v.w;
     }
     if (T & 2) {
-        const uint2 v = STREAM ? __ldcs(q.t2 + i) : q.t2[i];
+        const uint2 *p = reinterpret_cast<const uint2 *>(tile + 512 * (1 + N4)) + r;
+        const uint2 v = STREAM ? __ldcs(p) : *p;
         w[4 * N4] = v.x; w[4 * N4 + 1] = v.y;
     }
-    if (T & 1) w[T - 1] = STREAM ? __ldcs(q.t1 + i) : q.t1[i];
+    if (T & 1) {
+        const uint32_t *p = reinterpret_cast<const uint32_t *>(tile + 512 * (1 + N4) + ((T & 2) ? 256 : 0)) + r;
+        w[T - 1] = STREAM ? __ldcs(p) : *p;
+    }
 }
 template <int NB, bool STREAM>
-__device__ __forceinline__ void store_tail(const Queue &q, unsigned i, const uint32_t (&w)[2 + NB]) {
+__device__ __forceinline__ void store_tail(char *tile, unsigned r, const uint32_t (&w)[2 + NB]) {
     constexpr int T = 2 + NB, N4 = T / 4;
 #pragma unroll
     for (int k = 0; k < N4; ++k) {
         const uint4 v = make_uint4(w[4 * k], w[4 * k + 1], w[4 * k + 2], w[4 * k + 3]);
-        if (STREAM) __stcs(q.t4[k] + i, v); else q.t4[k][i] = v;
+        uint4 *p = reinterpret_cast<uint4 *>(tile + 512 * (1 + k)) + r;
+        if (STREAM) __stcs(p, v); else *p = v;
     }
     if (T & 2) {
         const uint2 v = make_uint2(w[4 * N4], w[4 * N4 + 1]);
-        if (STREAM) __stcs(q.t2 + i, v); else q.t2[i] = v;
+        uint2 *p = reinterpret_cast<uint2 *>(tile + 512 * (1 + N4)) + r;
+        if (STREAM) __stcs(p, v); else *p = v;
     }
-    if (T & 1) { if (STREAM) __stcs(q.t1 + i, w[T - 1]); else q.t1[i] = w[T - 1]; }
+    if (T & 1) {
+        uint32_t *p = reinterpret_cast<uint32_t *>(tile + 512 * (1 + N4) + ((T & 2) ? 256 : 0)) + r;
+        if (STREAM) __stcs(p, w[T - 1]); else *p = w[T - 1];
+    }
 }
 // the same for a bin count known at run time; words past the record are zero
 template <bool STREAM>
-__device__ __forceinline__ void load_tail_n(const Queue &q, int nb, unsigned i, uint32_t (&w)[2 + MAXB]) {
+__device__ __forceinline__ void load_tail_n(const Queue &q, unsigned i, uint32_t (&w)[2 + MAXB]) {
 #pragma unroll
     for (int k = 0; k < 2 + MAXB; ++k) w[k] = 0u;
     auto get = [&](auto tag) {
         constexpr int NB = decltype(tag)::value;
         uint32_t v[2 + NB];
-        load_tail<NB, STREAM>(q, i, v);
+        load_tail<NB, STREAM>(tile_of(q, i), i & 31u, v);
 #pragma unroll
         for (int k = 0; k < 2 + NB; ++k) w[k] = v[k];
     };
-    switch (nb) {
+    switch (q.nb) {
         case 1: get(Int<1>()); break;
         case 2: get(Int<2>()); break;
         case 3: get(Int<3>()); break;
@@ -560,15 +569,15 @@ __device__ __forceinline__ void load_tail_n(const Queue &q, int nb, unsigned i, 
         default: get(Int<8>()); break;
     }
 }
-__device__ __forceinline__ void store_tail_n(const Queue &q, int nb, unsigned i, const uint32_t (&w)[2 + MAXB]) {
+__device__ __forceinline__ void store_tail_n(const Queue &q, unsigned i, const uint32_t (&w)[2 + MAXB]) {
     auto put = [&](auto tag) {
         constexpr int NB = decltype(tag)::value;
         uint32_t v[2 + NB];
 #pragma unroll
         for (int k = 0; k < 2 + NB; ++k) v[k] = w[k];
-        store_tail<NB, false>(q, i, v);
+        store_tail<NB, false>(tile_of(q, i), i & 31u, v);
     };
-    switch (nb) {
+    switch (q.nb) {
         case 1: put(Int<1>()); break;
         case 2: put(Int<2>()); break;
         case 3: put(Int<3>()); break;

@@ -50,60 +50,29 @@ size_t ray_bytes(int nb, bool merge) { return 6 * sizeof(int32_t) + (size_t)nb *
 
 }  // namespace
 
-Queue queue_at(void *base, long long cap, int nb, bool merged, size_t *bytes) {
-    Queue q{};
-    char *p = static_cast<char *>(base);
-    size_t tot = 0;
-    auto piece = [&](size_t per) {
-        char *r = p + tot;
-        tot += ((size_t)cap * per + 255) & ~(size_t)255;
-        return (void *)r;
-    };
-    const int T = 2 + nb;
-    q.a = (uint4 *)piece(16);
-    for (int k = 0; k < T / 4; ++k) q.t4[k] = (uint4 *)piece(16);
-    if (T & 2) q.t2 = (uint2 *)piece(8);
-    if (T & 1) q.t1 = (uint32_t *)piece(4);
-    if (merged) {
-        q.m = (uint4 *)piece(16);
-        q.mthr = (float *)piece(4);
-    }
-    if (bytes) *bytes = tot;
-    return q;
-}
-
-cudaError_t read_queue(const Queue &q, int nb, bool merged, long long n, HostRays &out) {
+cudaError_t read_queue(const Queue &q, bool merged, long long n, HostRays &out) {
+    const int nb = q.nb;
     out.pl.resize(n); out.em.resize(n); out.bi.resize(n); out.d.resize(3 * n); out.ph.resize((size_t)nb * n);
     out.ma.resize(merged ? n : 0); out.pos.resize(merged ? 3 * n : 0); out.thr.resize(merged ? n : 0);
     if (n == 0) return cudaSuccess;
-    size_t bytes = 0;
-    queue_at(nullptr, n, nb, merged, &bytes);
-    std::vector<char> host(bytes);
-    const Queue h = queue_at(host.data(), n, nb, merged, nullptr);
-    cudaError_t e = cudaSuccess;
-    auto get = [&](void *dst, const void *src, size_t per) {
-        if (dst && e == cudaSuccess) e = cudaMemcpy(dst, src, (size_t)n * per, cudaMemcpyDeviceToHost);
-    };
-    get(h.a, q.a, 16);
-    for (int k = 0; k < 2; ++k) get(h.t4[k], q.t4[k], 16);
-    get(h.t2, q.t2, 8);
-    get(h.t1, q.t1, 4);
-    get(h.m, q.m, 16);
-    get(h.mthr, q.mthr, 4);
+    std::vector<char> host(queue_bytes(n, nb, merged));
+    cudaError_t e = cudaMemcpy(host.data(), q.base, host.size(), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return e;
+    const Queue h = queue_at(host.data(), nb, merged);
     for (long long i = 0; i < n; ++i) {
-        out.pl[i] = *tail_word(h, nb, 1, i);
-        out.em[i] = h.a[i].x;
-        out.bi[i] = (int32_t)h.a[i].y;
-        out.d[i] = (int32_t)h.a[i].z;
-        out.d[n + i] = (int32_t)h.a[i].w;
-        out.d[2 * n + i] = (int32_t)*tail_word(h, nb, 0, i);
-        for (int b = 0; b < nb; ++b) std::memcpy(&out.ph[(size_t)b * n + i], tail_word(h, nb, 2 + b, i), 4);
+        const uint4 a = *ray_head(h, i);
+        out.pl[i] = *pixel_word(h, i);
+        out.em[i] = a.x;
+        out.bi[i] = (int32_t)a.y;
+        out.d[i] = (int32_t)a.z;
+        out.d[n + i] = (int32_t)a.w;
+        out.d[2 * n + i] = (int32_t)*tail_word(h, 0, i);
+        for (int b = 0; b < nb; ++b) std::memcpy(&out.ph[(size_t)b * n + i], tail_word(h, 2 + b, i), 4);
         if (merged) {
-            const uint4 m = h.m[i];
+            const uint4 m = *ray_merge(h, i);
             out.pos[i] = (int32_t)m.x; out.pos[n + i] = (int32_t)m.y; out.pos[2 * n + i] = (int32_t)m.z;
             out.ma[i] = m.w;
-            out.thr[i] = h.mthr[i];
+            out.thr[i] = *ray_thr(h, i);
         }
     }
     return cudaSuccess;
@@ -259,12 +228,11 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
 
     // ray queues: one allocation, two buffers
     {
-        size_t per = 0;
-        queue_at(nullptr, cap, cfg_.nb, mrg, &per);
+        const size_t per = (queue_bytes(cap, cfg_.nb, mrg) + 255) & ~(size_t)255;
         char *base = nullptr;
         if (dev_alloc((void **)&base, 2 * per + 256) != cudaSuccess) return fail(FLEXRT_E_OOM, "ray queue allocation failed");
         qmem_ = base;
-        for (int k = 0; k < 2; ++k) q_[k] = queue_at(base + k * per, cap, cfg_.nb, mrg, nullptr);
+        for (int k = 0; k < 2; ++k) q_[k] = queue_at(base + k * per, cfg_.nb, mrg);
     }
     const long long nc = cfg_.cell_capacity;
     const int ms = cfg_.max_sims;
@@ -546,6 +514,16 @@ flexrt_status Engine::add_sim(const SimDev &proto, const double *n_H, int *slot_
             return fail(FLEXRT_E_INVALID, "members of one engine must use the same gamma_iters");
     const long long c0 = cell_alloc_.alloc(proto.ncell);
     if (c0 < 0) return fail(FLEXRT_E_CAPACITY, "cell arena full");
+    {
+        // the deepest level its rays may reach: a ray cast by an emitter is
+        // younger than the ring; a merged ray's distance is not so bounded
+        int L = proto.l_src;
+        while (L < proto.l_max && (proto.merge || proto.K[L] <= em_.ring_w)) ++L;
+        if (L > ltab_ && !far_possible_) {
+            far_possible_ = true;
+            graph_dirty_ = true;
+        }
+    }
     Slot &sl = slots_[s];
     sl = Slot();
     sl.used = true;
@@ -795,6 +773,7 @@ flexrt_status Engine::launch_stage(int stage) {
         tic();
         CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, st_, ext_variants()));
         toc(1);
+        if (far_possible_) CK(launch_far(ea, sm_count_, st_));
         return FLEXRT_OK;
     }
     if (merge_built()) {
@@ -1062,7 +1041,7 @@ flexrt_status Engine::rays(int s, int64_t cap, int32_t *level, int64_t *pixel, i
     if (mid_step_) *n = 0;
     if (m == 0 || (cap == 0 && !mid_step_)) return FLEXRT_OK;
     HostRays hr;
-    CK(read_queue(q_[qs], cfg_.nb, merge_built(), m, hr));
+    CK(read_queue(q_[qs], merge_built(), m, hr));
     const std::vector<uint32_t> &pl = hr.pl, &em = hr.em;
     const std::vector<int32_t> &bi = hr.bi, &d = hr.d;
     const int nph = photons ? sl->h.nb : 0;
@@ -1091,7 +1070,7 @@ flexrt_status Engine::rays_merged(int s, int64_t cap, int32_t *merged, int32_t *
     const int qs = mid_step_ ? hc.par ^ 1 : hc.par;
     const long long m = hc.cnt[qs];
     HostRays hr;
-    CK(read_queue(q_[qs], cfg_.nb, merge_built(), m, hr));
+    CK(read_queue(q_[qs], merge_built(), m, hr));
     const std::vector<uint32_t> &em = hr.em, &ma = hr.ma;
     const std::vector<long long> idx = member_rays(hr.pl, em, ma, s, sl->em0, sl->em_n);
     *n = (int64_t)idx.size();
@@ -1232,7 +1211,7 @@ flexrt_status Engine::save_state(int s, void *buf, int64_t cap, int64_t *bytes) 
     // the records as one array a word, in the other queue's memory (unused
     // between steps)
     const int words = 6 + nb + (mf ? 5 : 0);
-    parts.push_back({q_[hc.par ^ 1].a, (size_t)nray * words * 4});
+    parts.push_back({q_[hc.par ^ 1].base, (size_t)nray * words * 4});
     size_t tot = sizeof(StateHeader);
     for (auto &p : parts) tot += p.second;
     *bytes = (int64_t)tot;
@@ -1249,7 +1228,7 @@ flexrt_status Engine::save_state(int s, void *buf, int64_t cap, int64_t *bytes) 
     char *o = (char *)buf;
     std::memcpy(o, &h, sizeof(h));
     o += sizeof(h);
-    CK(launch_queue_words(q_[hc.par], nb, mf, nray, reinterpret_cast<uint32_t *>(q_[hc.par ^ 1].a), false, st_));
+    CK(launch_queue_words(q_[hc.par], mf, nray, reinterpret_cast<uint32_t *>(q_[hc.par ^ 1].base), false, st_));
     CK(cudaStreamSynchronize(st_));
     for (auto &p : parts) {
         if (p.second) CK(cudaMemcpy(o, p.first, p.second, cudaMemcpyDeviceToHost));
@@ -1282,7 +1261,7 @@ flexrt_status Engine::load_state(int s, const void *buf, int64_t bytes) {
         {em_.n0 + sl->em0, (size_t)ne * 4}, {em_.ring + sl->em0 * rw * 3, (size_t)ne * rw * 3 * sizeof(int4)}};
     if (ne == 0) { parts[8].second = 0; parts[9].second = 0; }
     const int words = 6 + nb + (merge_built() ? 5 : 0);
-    parts.push_back({q_[1].a, (size_t)nray * words * 4});      // one array a word, joined into queue 0 below
+    parts.push_back({q_[1].base, (size_t)nray * words * 4});      // one array a word, joined into queue 0 below
     size_t tot = sizeof(StateHeader);
     for (auto &p : parts) tot += p.second;
     if ((int64_t)tot != bytes) return fail(FLEXRT_E_INVALID, "checkpoint size does not match its header");
@@ -1292,7 +1271,7 @@ flexrt_status Engine::load_state(int s, const void *buf, int64_t bytes) {
         if (p.second) CK(cudaMemcpy(p.first, src, p.second, cudaMemcpyHostToDevice));
         src += p.second;
     }
-    CK(launch_queue_words(q_[0], nb, merge_built(), nray, reinterpret_cast<uint32_t *>(q_[1].a), true, st_));
+    CK(launch_queue_words(q_[0], merge_built(), nray, reinterpret_cast<uint32_t *>(q_[1].base), true, st_));
     // the live rays in queue 0, nothing in flight in queue 1, no latched error
     const long long cnt[2] = {nray, 0};
     const int32_t par_err[2] = {0, 0};

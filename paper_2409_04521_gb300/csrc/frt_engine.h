@@ -15,10 +15,11 @@ namespace frt {
 // Process-wide fixed-point pixel-vector table of levels 0..level on `device`.
 cudaError_t get_pixtab(int device, int level, cudaStream_t st, const int4 **out);
 
-// The pieces of a queue of cap records (frt_types.h) placed one after another
-// from `base`, each on a 256-byte boundary; *bytes gets their total.  Works
-// on host and device addresses.
-Queue queue_at(void *base, long long cap, int nb, bool merged, size_t *bytes);
+// A queue of cap records at `base` (host or device): its bytes, and its view.
+inline size_t queue_bytes(long long cap, int nb, bool merged) {
+    return (size_t)((cap + 31) / 32) * tile_bytes(nb, merged);
+}
+inline Queue queue_at(void *base, int nb, bool merged) { return Queue{static_cast<char *>(base), tile_bytes(nb, merged), nb}; }
 
 // Host copy of a queue's first n records, one array a word.
 struct HostRays {
@@ -26,7 +27,7 @@ struct HostRays {
     std::vector<int32_t> bi, d, pos;               // d: n of dx, then dy, then dz; pos likewise
     std::vector<float> ph, thr;                    // ph: n of each bin
 };
-cudaError_t read_queue(const Queue &q, int nb, bool merged, long long n, HostRays &out);
+cudaError_t read_queue(const Queue &q, bool merged, long long n, HostRays &out);
 
 // First-fit allocator of [0, capacity) index ranges.
 class RangeAllocator {
@@ -155,6 +156,7 @@ class Engine {
     void *mwmem_ = nullptr;
     const int4 *pixtab_ = nullptr;
     int ltab_ = 0;
+    bool far_possible_ = false;   // a member's rays may reach levels beyond the table
     int em_cap_ = 0;
     long long qcap_ = 0;       // allocated queue slots (capacity plus run-tail margin)
     RangeAllocator cell_alloc_, em_alloc_;

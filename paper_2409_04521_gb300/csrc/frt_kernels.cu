@@ -221,8 +221,8 @@ __global__ void __launch_bounds__(128) k_emit(EmitArgs A) {
             w[1] = ((uint32_t)lk << LEVEL_SHIFT) | p;
 #pragma unroll
             for (int b = 0; b < MAXB; ++b) w[2 + b] = __float_as_uint(b < S.nb ? S.frac[b] * nk : 0.0f);
-            q.a[o] = make_uint4((uint32_t)ek, (uint32_t)sk, (uint32_t)dx, (uint32_t)dy);
-            store_tail_n(q, A.nb, o, w);
+            *ray_head(q, o) = make_uint4((uint32_t)ek, (uint32_t)sk, (uint32_t)dx, (uint32_t)dy);
+            store_tail_n(q, o, w);
         };
         const int here = min(32, n - (j - lane));  // emitters of this warp (its first one is j - lane < n)
         const int l0 = __shfl_sync(FULL, l, 0);
@@ -257,23 +257,54 @@ __global__ void __launch_bounds__(128) k_emit(EmitArgs A) {
 }
 
 // ---------------------------------------------------------------------------
+// directions of the march's children beyond the pixel table (levels that
+// hardly any run reaches).  In the march itself the double-precision vector
+// took 15 registers of every ray.  Launched only by engines with a member
+// that can reach such a level; the march's flag says whether one did.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) k_far(EmitArgs A) {
+    const Ctl *C = A.ctl;
+    if (!C->far || C->err) return;
+    const Queue q = A.q[C->par ^ 1];
+    const long long n = C->cnt[C->par ^ 1];
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const uint32_t pl = *pixel_word(q, i);
+        if (pl == DEAD_RAY || (int)(pl >> LEVEL_SHIFT) <= A.ltab) continue;
+        const uint4 a = *ray_head(q, i);
+        if ((int32_t)a.z != DIR_FAR) continue;
+        int4 rows[3];
+        if (a.x & MERGED_BIT) {
+            const SimDev &S = A.sims[(ray_merge(q, i)->w >> 16) & 0x7fffu];
+            rotation_rows(S.seed, (1LL << 31) + (long long)(a.x & ~MERGED_BIT), (int)a.y, S.rotate, rows);
+        } else {
+            const int4 *rg = A.em.ring + ((long long)a.x * A.em.ring_w + (int)a.y % A.em.ring_w) * 3;
+            rows[0] = rg[0]; rows[1] = rg[1]; rows[2] = rg[2];
+        }
+        int32_t dx, dy, dz;
+        rotate_dir(rows, healpix_vq((int)(pl >> LEVEL_SHIFT), pl & PIX_MASK), dx, dy, dz);
+        *ray_head(q, i) = make_uint4(a.x, a.y, (uint32_t)dx, (uint32_t)dy);
+        *tail_word(q, 0, i) = (uint32_t)dz;
+    }
+}
+
+// ---------------------------------------------------------------------------
 // a queue's records to and from one array a word (checkpoints): word-major,
 // in the order pixel word, emitter, birth, dx, dy, dz, photons, then the
 // merged rays' position, merge word and threshold
 // ---------------------------------------------------------------------------
-__global__ void k_queue_words(Queue q, int nb, int merged, long long n, uint32_t *words, int join) {
+__global__ void k_queue_words(Queue q, int merged, long long n, uint32_t *words, int join) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         uint32_t *x[6 + MAXB + 5];
-        uint32_t *a = reinterpret_cast<uint32_t *>(q.a + i);
+        uint32_t *a = reinterpret_cast<uint32_t *>(ray_head(q, i));
         int k = 0;
-        x[k++] = tail_word(q, nb, 1, i);
+        x[k++] = tail_word(q, 1, i);
         x[k++] = a; x[k++] = a + 1; x[k++] = a + 2; x[k++] = a + 3;
-        x[k++] = tail_word(q, nb, 0, i);
-        for (int b = 0; b < nb; ++b) x[k++] = tail_word(q, nb, 2 + b, i);
+        x[k++] = tail_word(q, 0, i);
+        for (int b = 0; b < q.nb; ++b) x[k++] = tail_word(q, 2 + b, i);
         if (merged) {
-            uint32_t *m = reinterpret_cast<uint32_t *>(q.m + i);
+            uint32_t *m = reinterpret_cast<uint32_t *>(ray_merge(q, i));
             for (int c = 0; c < 4; ++c) x[k++] = m + c;
-            x[k++] = reinterpret_cast<uint32_t *>(q.mthr + i);
+            x[k++] = reinterpret_cast<uint32_t *>(ray_thr(q, i));
         }
         for (int c = 0; c < k; ++c) {
             if (join) *x[c] = words[c * n + i];
@@ -526,6 +557,7 @@ __global__ void k_end(Ctl *C, SimDev *sims, SimAcc *acc, int nsims) {
             C->par = par ^ 1;
         }
         C->merged = 0;
+        C->far = 0;
     }
 }
 
@@ -540,7 +572,10 @@ __global__ void k_iter_reset(Ctl *C, SimAcc *acc, int nsims) {
         a.p_abs = a.p_esc = a.p_out = a.p_in = 0.0;
         a.p_seg = a.p_rays_in = a.p_rays_out = a.p_lost = 0.0;
     }
-    if (threadIdx.x == 0) C->cnt[C->par ^ 1] = 0;
+    if (threadIdx.x == 0) {
+        C->cnt[C->par ^ 1] = 0;
+        C->far = 0;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -625,11 +660,15 @@ cudaError_t launch_emit(const EmitArgs &a, int blocks, cudaStream_t st) {
     k_emit<<<blocks, 128, 0, st>>>(a);
     return cudaGetLastError();
 }
-cudaError_t launch_queue_words(const Queue &q, int nb, bool merged, long long n, uint32_t *words, bool join,
+cudaError_t launch_far(const EmitArgs &a, int blocks, cudaStream_t st) {
+    k_far<<<blocks, 256, 0, st>>>(a);
+    return cudaGetLastError();
+}
+cudaError_t launch_queue_words(const Queue &q, bool merged, long long n, uint32_t *words, bool join,
                                cudaStream_t st) {
     if (n < 1) return cudaSuccess;
     const int blocks = (int)std::min<long long>((n + 255) / 256, 4096);
-    k_queue_words<<<blocks, 256, 0, st>>>(q, nb, merged ? 1 : 0, n, words, join ? 1 : 0);
+    k_queue_words<<<blocks, 256, 0, st>>>(q, merged ? 1 : 0, n, words, join ? 1 : 0);
     return cudaGetLastError();
 }
 // Kernel variants: every bin count with the default (AGG 0, 2 blocks/SM);
@@ -655,15 +694,18 @@ static MarchFn march_fn_plain(int nb, int agg, int minb) {
     FRT_V(3)
     FRT_V(4)
 #undef FRT_V
-    if (agg != 0 || minb != 2) return nullptr;
-    switch (nb) {
-        case 2: return k_march<2, 0, 2, 0>;
-        case 5: return k_march<5, 0, 2, 0>;
-        case 6: return k_march<6, 0, 2, 0>;
-        case 7: return k_march<7, 0, 2, 0>;
-        case 8: return k_march<8, 0, 2, 0>;
-        default: return nullptr;
+#define FRT_W(NB)                                                                   \
+    if (nb == NB && agg == 0) {                                                    \
+        if (minb == 2) return k_march<NB, 0, 2, 0>;                                \
+        if (minb == 3) return k_march<NB, 0, 3, 0>;                                \
     }
+    FRT_W(2)
+    FRT_W(5)
+    FRT_W(6)
+    FRT_W(7)
+    FRT_W(8)
+#undef FRT_W
+    return nullptr;
 }
 static MarchFn march_fn(int nb, int agg, int minb, int ext) {
     switch (ext) {

@@ -62,8 +62,10 @@ void set_free_error(const std::string &msg);
 cudaError_t launch_pixtab(int4 *tab, int L, cudaStream_t st);
 cudaError_t launch_init_cells(const SimDev *sims, int sim, Cells c, long long ncell, cudaStream_t st);
 cudaError_t launch_emit(const EmitArgs &a, int blocks, cudaStream_t st);
+// after a march: directions of children beyond the pixel table
+cudaError_t launch_far(const EmitArgs &a, int blocks, cudaStream_t st);
 // a queue's first n records to (join: from) one array of n words per word of the record
-cudaError_t launch_queue_words(const Queue &q, int nb, bool merged, long long n, uint32_t *words, bool join,
+cudaError_t launch_queue_words(const Queue &q, bool merged, long long n, uint32_t *words, bool join,
                                cudaStream_t st);
 using MarchFn = void (*)(MarchArgs);
 // the march variant with merged rays (nullptr if not built)

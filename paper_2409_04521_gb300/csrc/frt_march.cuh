@@ -50,7 +50,7 @@ __device__ __forceinline__ void flush_tallies(float &esc, float &out, unsigned &
 
 // The per-simulation constants the march needs, staged in shared memory.
 struct MarchSim {
-    int nx, ny, nz, step, l_src, l_max, active, l_merge, gen, pad0, pad1, pad2;
+    int nx, ny, nz, step, l_src, l_max, active, l_merge, gen, ring0, pad1, pad2;   // ring0: this step's ring slot
     long long coff;
     float eps;
     float sig_max;          // largest sigma_b / sigma_ref of the bins
@@ -174,6 +174,8 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
     // per-simulation tallies of this block (photons in 2^-32 fixed point,
     // counts as integers), then the staged constants
     extern __shared__ unsigned long long sh_acc[];
+    __shared__ unsigned char sh_parent[8][32];     // splitting lanes of each warp, in order
+    unsigned char *const parent = sh_parent[threadIdx.x >> 5];
     MarchSim *msim = reinterpret_cast<MarchSim *>(sh_acc + A.nsims * NACC);
     for (int i = threadIdx.x; i < A.nsims * NACC; i += blockDim.x) sh_acc[i] = 0ull;
     for (int i = threadIdx.x; i < A.nsims; i += blockDim.x) {
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
         MarchSim &m = msim[i];
         m.nx = S.nx; m.ny = S.ny; m.nz = S.nz; m.step = S.step; m.l_src = S.l_src; m.l_max = S.l_max;
         m.active = S.active; m.l_merge = S.l_merge; m.coff = S.cell_off; m.eps = S.eps_term;
-        m.gen = S.gen_mode; m.pad0 = m.pad1 = m.pad2 = 0;
+        m.gen = S.gen_mode; m.ring0 = S.step % A.em.ring_w; m.pad1 = m.pad2 = 0;
         for (int l = 0; l < MAXL; ++l) m.K[l] = S.K[l];
         m.sig_max = 0.0f;
         for (int b = 0; b < MAXB; ++b) {
@@ -194,7 +196,10 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
     const int lane = lane_id();
     if (C->err == 0) {
         const int par = C->par;
-        const Queue qi = A.q[par], qo = A.q[par ^ 1];
+        // (one base address a queue: an address an array took 28 registers)
+        const char *const qin = A.q[par].base;
+        char *const qout = A.q[par ^ 1].base;
+        const unsigned tile = A.q[0].tile;
         unsigned long long *out_cnt = (unsigned long long *)&C->cnt[par ^ 1];
         // queue slots stay below 2^31 (the engine's bound), so 32-bit indices
         const unsigned n = (unsigned)(C->cnt[par] + C->emit_total);
@@ -217,8 +222,9 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             uint32_t w[2 + NB];
             w[1] = DEAD_RAY;
             if (i < n) {
-                ra = __ldcs(qi.a + i);
-                load_tail<NB, true>(qi, i, w);
+                const char *t = qin + (size_t)(i >> 5) * tile;       // the warp's tile: i & 31 is the lane
+                ra = __ldcs(reinterpret_cast<const uint4 *>(t) + lane);
+                load_tail<NB, true>(t, lane, w);
             }
             const uint32_t e = ra.x, pl = w[1];
             const int bi = (int)ra.y, dx = (int)ra.z, dy = (int)ra.w, dz = (int)w[0];
@@ -231,9 +237,10 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             uint32_t ma = 0;
             float mthr = 0.0f;
             if (mrg) {
-                const uint4 rm = __ldcs(qi.m + i);
+                const char *t = qin + (size_t)(i >> 5) * tile + 128 * (6 + NB);
+                const uint4 rm = __ldcs(reinterpret_cast<const uint4 *>(t) + lane);
                 mx = (int)rm.x; my = (int)rm.y; mz = (int)rm.z; ma = rm.w;
-                mthr = __ldcs(qi.mthr + i);
+                mthr = __ldcs(reinterpret_cast<const float *>(t + 512) + lane);
             }
             int sim = 0;
             int4 ec = make_int4(0, 0, 0, 0);
@@ -428,52 +435,101 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                     slab_left = left - tot;
                 }
                 w_out += tot;
-                if (fits && nout > 0) {
-                    auto slot_of = [&](int k) -> unsigned {
-                        return k < left ? s0 + (unsigned)k : s1 + (unsigned)(k - left);
-                    };
-                    if (nout == 1) {
-                        const unsigned o = slot_of(k0);
-                        __stcs(qo.a + o, ra);
+                auto slot_of = [&](int k) -> unsigned {
+                    return k < left ? s0 + (unsigned)k : s1 + (unsigned)(k - left);
+                };
+                if (fits && nout == 1) {
+                    const unsigned o = slot_of(k0);
+                    char *const t = qout + (size_t)(o >> 5) * tile;
+                    __stcs(reinterpret_cast<uint4 *>(t) + (o & 31u), ra);
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) w[2 + b] = __float_as_uint(ph[b]);
-                        store_tail<NB, true>(qo, o, w);
-                        if (mrg) {
-                            __stcs(qo.m + o, make_uint4((uint32_t)mx, (uint32_t)my, (uint32_t)mz, ma));
-                            __stcs(qo.mthr + o, mthr);
-                        }
-                    } else {
-                        const int L = lev + m;
-                        const uint32_t pix0 = (pl & PIX_MASK) << (2 * m);
-                        // children keep their parent's sphere (Sec. 3.2): the
-                        // emitter's of the birth step, or the merge cell's
-                        int4 rows[3];
-                        if (mrg) {
+                    for (int b = 0; b < NB; ++b) w[2 + b] = __float_as_uint(ph[b]);
+                    store_tail<NB, true>(t, o & 31u, w);
+                    if (mrg) {
+                        char *const tm = t + 128 * (6 + NB);
+                        __stcs(reinterpret_cast<uint4 *>(tm) + (o & 31u),
+                               make_uint4((uint32_t)mx, (uint32_t)my, (uint32_t)mz, ma));
+                        __stcs(reinterpret_cast<float *>(tm + 512) + (o & 31u), mthr);
+                    }
+                }
+                // children: the warp makes the children of all its splitting
+                // lanes together, one child a lane, whose neighbours go to
+                // neighbouring slots; the splits of one depth m at a time
+                // (one depth in nearly every warp).  Each splitting lane
+                // writing its own four children was a fifth to a third of the
+                // march: half of the warps hold a few such lanes, and every
+                // lane of the warp waited through four of them.
+                unsigned split = __ballot_sync(FULL, fits && nout > 1);
+                while (split) {
+                    const int mm = __shfl_sync(FULL, m, __ffs(split) - 1);
+                    const unsigned grp = __ballot_sync(FULL, ((split >> lane) & 1u) && m == mm);
+                    split &= ~grp;
+                    __syncwarp();
+                    if ((grp >> lane) & 1u) parent[__popc(grp & ((1u << lane) - 1u))] = (unsigned char)lane;
+                    __syncwarp();
+                    // children keep their parent's sphere (Sec. 3.2): the
+                    // emitter's of the birth step, or the merge cell's
+                    int4 mrows[3];
+                    const bool anym = MRG && __any_sync(FULL, mrg && ((grp >> lane) & 1u));
+                    if (MRG) {
+                        mrows[0] = mrows[1] = mrows[2] = make_int4(0, 0, 0, 0);
+                        if (mrg && ((grp >> lane) & 1u)) {
                             const SimDev &SD = A.sims[sim];
-                            rotation_rows(SD.seed, (1LL << 31) + (long long)(e & ~MERGED_BIT), bi, SD.rotate, rows);
-                        } else {
-                            const int4 *rg = A.em.ring + ((long long)e * A.em.ring_w + (bi % A.em.ring_w)) * 3;
-                            rows[0] = rg[0]; rows[1] = rg[1]; rows[2] = rg[2];
+                            rotation_rows(SD.seed, (1LL << 31) + (long long)(e & ~MERGED_BIT), bi, SD.rotate, mrows);
                         }
-                        const bool vert = mrg && (ma >> 31);
-                        const float scale = pow2_neg(2 * m);
+                    }
+                    const float scale = pow2_neg(2 * mm);
+                    const unsigned all = (unsigned)__popc(grp) << (2 * mm);
+                    for (unsigned c0 = 0; c0 < all; c0 += 32) {
+                        const unsigned c = c0 + lane;
+                        const int src = parent[c < all ? c >> (2 * mm) : 0u];
+                        const unsigned sub = c & ((1u << (2 * mm)) - 1u);
+                        const uint32_t ppl = __shfl_sync(FULL, pl, src), pe = __shfl_sync(FULL, e, src);
+                        const int pbi = __shfl_sync(FULL, bi, src), psim = __shfl_sync(FULL, sim, src);
+                        const int pk = __shfl_sync(FULL, k0, src);
                         uint32_t cw[2 + NB];
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) cw[2 + b] = __float_as_uint(ph[b] * scale);
-                        for (int c = 0; c < nout; ++c) {
-                            const uint32_t pix = vert ? vertex_child(S.l_merge, pl & PIX_MASK, lev, m, (uint32_t)c)
-                                                      : pix0 + (uint32_t)c;
-                            const int4 vq = L <= A.ltab ? __ldg(&A.pixtab[level_offset(L) + pix]) : healpix_vq(L, pix);
-                            int32_t cx, cy, cz;
-                            rotate_dir(rows, vq, cx, cy, cz);
-                            const unsigned oc = slot_of(k0 + c);
+                        for (int b = 0; b < NB; ++b) cw[2 + b] = __float_as_uint(__shfl_sync(FULL, ph[b], src) * scale);
+                        int4 rows[3];
+                        uint4 pm = make_uint4(0u, 0u, 0u, 0u);
+                        float pthr = 0.0f;
+                        if (MRG && anym) {
+#pragma unroll
+                            for (int r = 0; r < 3; ++r)
+                                rows[r] = make_int4(__shfl_sync(FULL, mrows[r].x, src), __shfl_sync(FULL, mrows[r].y, src),
+                                                    __shfl_sync(FULL, mrows[r].z, src), 0);
+                            pm = make_uint4((uint32_t)__shfl_sync(FULL, mx, src), (uint32_t)__shfl_sync(FULL, my, src),
+                                            (uint32_t)__shfl_sync(FULL, mz, src), __shfl_sync(FULL, ma, src));
+                            pthr = __shfl_sync(FULL, mthr, src);
+                        }
+                        if (c < all) {
+                            const int plev = (int)(ppl >> LEVEL_SHIFT), L = plev + mm;
+                            const bool pmrg = MRG && (pe & MERGED_BIT);
+                            if (!pmrg) {
+                                // the birth step's slot of the ring: the age is less than its length
+                                int slot = msim[psim].ring0 - (msim[psim].step - pbi);
+                                if (slot < 0) slot += A.em.ring_w;
+                                const int4 *rg = A.em.ring + ((long long)pe * A.em.ring_w + slot) * 3;
+                                rows[0] = rg[0]; rows[1] = rg[1]; rows[2] = rg[2];
+                            }
+                            const uint32_t pix = pmrg && (pm.w >> 31)
+                                                     ? vertex_child(msim[psim].l_merge, ppl & PIX_MASK, plev, mm, sub)
+                                                     : ((ppl & PIX_MASK) << (2 * mm)) + sub;
+                            // (a level beyond the table: k_far fills the direction in)
+                            int32_t cx = DIR_FAR, cy = 0, cz = 0;
+                            if (L <= A.ltab) rotate_dir(rows, __ldg(&A.pixtab[level_offset(L) + pix]), cx, cy, cz);
+                            else atomicOr(&C->far, 1);
+                            const unsigned o = slot_of(pk + (int)sub);
                             cw[0] = (uint32_t)cz;
                             cw[1] = ((uint32_t)L << LEVEL_SHIFT) | pix;
-                            qo.a[oc] = make_uint4(e, (uint32_t)bi, (uint32_t)cx, (uint32_t)cy);
-                            store_tail<NB, false>(qo, oc, cw);
-                            if (mrg) {
-                                qo.m[oc] = make_uint4((uint32_t)mx, (uint32_t)my, (uint32_t)mz, ma & 0x7fffffffu);
-                                qo.mthr[oc] = mthr * scale;
+                            char *const t = qout + (size_t)(o >> 5) * tile;
+                            reinterpret_cast<uint4 *>(t)[o & 31u] = make_uint4(pe, (uint32_t)pbi, (uint32_t)cx, (uint32_t)cy);
+                            store_tail<NB, false>(t, o & 31u, cw);
+                            if (pmrg) {
+                                char *const tm = t + 128 * (6 + NB);
+                                pm.w &= 0x7fffffffu;
+                                reinterpret_cast<uint4 *>(tm)[o & 31u] = pm;
+                                reinterpret_cast<float *>(tm + 512)[o & 31u] = pthr * scale;
                             }
                         }
                     }
@@ -481,7 +537,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             }
             ++w_it;
         }
-        for (int k = lane; k < slab_left; k += 32) *pixel_word(qo, NB, slab + k) = DEAD_RAY;
+        for (int k = lane; k < slab_left; k += 32) *pixel_word(A.q[par ^ 1], slab + k) = DEAD_RAY;
         flush_tallies(t_esc, t_out, t_cnt, t_rout, t_sim, sh_acc);
     }
     __syncthreads();

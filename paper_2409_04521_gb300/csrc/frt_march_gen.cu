@@ -24,15 +24,18 @@ MarchFn march_fn_gen(int nb, int agg, int minb) {
     FRT_V(3)
     FRT_V(4)
 #undef FRT_V
-    if (agg != 0 || minb != 2) return nullptr;
-    switch (nb) {
-        case 2: return k_march<2, 0, 2, 3>;
-        case 5: return k_march<5, 0, 2, 3>;
-        case 6: return k_march<6, 0, 2, 3>;
-        case 7: return k_march<7, 0, 2, 3>;
-        case 8: return k_march<8, 0, 2, 3>;
-        default: return nullptr;
+#define FRT_W(NB)                                                                   \
+    if (nb == NB && agg == 0) {                                                    \
+        if (minb == 2) return k_march<NB, 0, 2, 3>;                                \
+        if (minb == 3) return k_march<NB, 0, 3, 3>;                                \
     }
+    FRT_W(2)
+    FRT_W(5)
+    FRT_W(6)
+    FRT_W(7)
+    FRT_W(8)
+#undef FRT_W
+    return nullptr;
 }
 
 }  // namespace frt

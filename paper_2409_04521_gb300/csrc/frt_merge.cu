@@ -65,15 +65,18 @@ MarchFn march_fn_merge(int nb, int agg, int minb) {
     FRT_V(3)
     FRT_V(4)
 #undef FRT_V
-    if (agg != 0 || minb != 2) return nullptr;
-    switch (nb) {
-        case 2: return k_march<2, 0, 2, 1>;
-        case 5: return k_march<5, 0, 2, 1>;
-        case 6: return k_march<6, 0, 2, 1>;
-        case 7: return k_march<7, 0, 2, 1>;
-        case 8: return k_march<8, 0, 2, 1>;
-        default: return nullptr;
+#define FRT_W(NB)                                                                   \
+    if (nb == NB && agg == 0) {                                                    \
+        if (minb == 2) return k_march<NB, 0, 2, 1>;                                \
+        if (minb == 3) return k_march<NB, 0, 3, 1>;                                \
     }
+    FRT_W(2)
+    FRT_W(5)
+    FRT_W(6)
+    FRT_W(7)
+    FRT_W(8)
+#undef FRT_W
+    return nullptr;
 }
 
 namespace {
@@ -118,7 +121,7 @@ __device__ __forceinline__ void hist_add(uint32_t *hist, long long bin) {
 
 // the simulation a queued ray belongs to
 __device__ __forceinline__ int ray_sim(const Queue &q, const Emitters &em, long long i, uint32_t e) {
-    return (e & MERGED_BIT) ? (int)((q.m[i].w >> 16) & 0x7fffu) : __ldg(&em.cell[e]).w;
+    return (e & MERGED_BIT) ? (int)((ray_merge(q, i)->w >> 16) & 0x7fffu) : __ldg(&em.cell[e]).w;
 }
 
 // whether a block of a pass with barriers runs: the control words are read
@@ -257,9 +260,9 @@ __global__ void __launch_bounds__(256) k_mhist1(MergeArgs A) {
         if (i < n) {
             // the ray's words together (a single simulation needs no
             // emitter lookup); bins past a member's own are zero
-            const uint32_t e = A.nsims > 1 ? q.a[i].x : 0u;
+            const uint32_t e = A.nsims > 1 ? ray_head(q, i)->x : 0u;
             uint32_t w[2 + MAXB];
-            load_tail_n<false>(q, A.nbq, (unsigned)i, w);
+            load_tail_n<false>(q, (unsigned)i, w);
             const uint32_t pl = w[1];
             int sim = -1;
             uint32_t key = 0;
@@ -534,10 +537,10 @@ __global__ void __launch_bounds__(256, 4) k_mgroup(MergeArgs A) {
             const uint32_t tref = sel[SEL_T];
             if (sel[SEL_STATE] == SEL_DONE && !(sel[SEL_EXEMPT] && key >= tref)) {
                 const SimDev &S = A.sims[sim];
-                const uint4 ra = q.a[i];
+                const uint4 ra = *ray_head(q, i);
                 const uint32_t e = ra.x;
                 const int bi = (int)ra.y, dx = (int)ra.z, dy = (int)ra.w;
-                const uint2 rt = A.nbq >= 2 ? *reinterpret_cast<const uint2 *>(q.t4[0] + i) : q.t2[i];
+                const uint2 rt = *reinterpret_cast<const uint2 *>(pixel_word(q, i) - 1);
                 const int dz = (int)rt.x;
                 const uint32_t pl = rt.y;
                 const int lev = (int)(pl >> LEVEL_SHIFT);
@@ -546,7 +549,7 @@ __global__ void __launch_bounds__(256, 4) k_mgroup(MergeArgs A) {
                 int dist;
                 if (e & MERGED_BIT) {
                     const long long k = S.step - bi;
-                    const uint4 rm = q.m[i];
+                    const uint4 rm = *ray_merge(q, i);
                     p[0] = (int)rm.x + k * dx; p[1] = (int)rm.y + k * dy; p[2] = (int)rm.z + k * dz;
                     dist = (int)(rm.w & 0xffffu) + (int)k;
                 } else {
@@ -639,20 +642,20 @@ __global__ void __launch_bounds__(256, 4) k_mweight(MergeArgs A) {
         if (slot >= 0) {
             sim = A.nsims > 1 ? A.w.tsim[qi] : 0;
             const SimDev &S = A.sims[sim];
-            const uint32_t e = q.a[qi].x;
+            const uint32_t e = ray_head(q, qi)->x;
             nbf = S.nb;
             uint32_t w[2 + MAXB];
-            load_tail_n<false>(q, A.nbq, qi, w);
+            load_tail_n<false>(q, qi, w);
 #pragma unroll
             for (int b = 0; b < MAXB; ++b)
                 if (b < nbf) f[b] = __uint_as_float(w[2 + b]);
             const int lev = (int)((pk.y >> 21) & 0xfu);
-            const float thr = (e & MERGED_BIT) ? q.mthr[qi]
+            const float thr = (e & MERGED_BIT) ? *ray_thr(q, qi)
                                                : S.eps_term * __ldg(&A.em.n0[e]) * pow2_neg(2 * (lev - S.l_src));
 #pragma unroll
             for (int b = 0; b <= MAXB; ++b)
                 if (b == nbf) f[b] = thr;
-            *pixel_word(q, A.nbq, qi) = DEAD_RAY;
+            *pixel_word(q, qi) = DEAD_RAY;
         }
         unsigned long long v[GSUMS] = {0, 0, 0, 0, 0, 0};
         if (slot >= 0) {
@@ -765,7 +768,7 @@ __global__ void __launch_bounds__(256, 4) k_memit(MergeArgs A) {
     const unsigned long long pre = A.w.bcnt[blockIdx.x];   // this block's place in the appended run
     const long long b0 = blockIdx.x * block_chunk(mbase);
     const uint32_t bl = A.w.bled[blockIdx.x];
-    const int ndir = A.w.ndir, gw = A.w.grp_w, nbq = A.nbq;
+    const int ndir = A.w.ndir, gw = A.w.grp_w;
     for (uint32_t j = threadIdx.x; j < bl; j += blockDim.x) {
         const uint32_t slot = A.w.lead_slot[b0 + j];
         const int sim = A.w.lead_sim[b0 + j];
@@ -799,11 +802,11 @@ __global__ void __launch_bounds__(256, 4) k_memit(MergeArgs A) {
         w[1] = ((uint32_t)L2 << LEVEL_SHIFT) | pm;
 #pragma unroll
         for (int b = 0; b < MAXB; ++b) w[2 + b] = __float_as_uint(b < S.nb ? gph[b] : 0.0f);
-        q.a[o] = make_uint4(MERGED_BIT | (uint32_t)local, (uint32_t)S.step, (uint32_t)dx, (uint32_t)dy);
-        store_tail_n(q, nbq, (unsigned)o, w);
-        q.m[o] = make_uint4((uint32_t)P[0], (uint32_t)P[1], (uint32_t)P[2],
+        *ray_head(q, o) = make_uint4(MERGED_BIT | (uint32_t)local, (uint32_t)S.step, (uint32_t)dx, (uint32_t)dy);
+        store_tail_n(q, (unsigned)o, w);
+        *ray_merge(q, o) = make_uint4((uint32_t)P[0], (uint32_t)P[1], (uint32_t)P[2],
                             (L2 > S.l_merge ? 0x80000000u : 0u) | ((uint32_t)sim << 16) | (uint32_t)Adist);
-        q.mthr[o] = gph[S.nb];
+        *ray_thr(q, o) = gph[S.nb];
         // the group is cleared for the next step
         float4 *gz = reinterpret_cast<float4 *>(gp);
         for (int b = 0; b < gw / 4; ++b) gz[b] = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -18,6 +18,7 @@ constexpr int MAXL = 13;                            // HEALPix levels 0..12
 constexpr int LEVEL_SHIFT = 28;                     // pixlev = level<<28 | pixel
 constexpr uint32_t PIX_MASK = (1u << LEVEL_SHIFT) - 1u;
 constexpr uint32_t DEAD_RAY = 0xffffffffu;         // unused queue slot (level 15 never occurs)
+constexpr int32_t DIR_FAR = (int32_t)0x80000000u;  // dx of a child whose direction is not known yet (k_far)
 constexpr int OUT_SLAB = 512;                       // queue slots a warp reserves at once
 constexpr uint32_t MERGED_BIT = 0x80000000u;        // emitter word of a merged ray: bit | local cell
 constexpr int HIST_BINS = 65536;                    // radix-select bins per pass (16 bits)
@@ -99,42 +100,55 @@ struct Ctl {
     int32_t n_ranges;        // active cell ranges
     long long ncell_active;  // cells in active simulations
     int32_t merged;          // a simulation merged rays this step
-    int32_t pad;
+    int32_t far;             // the march left children beyond the pixel table
     long long mbase;         // the march's output count: merged rays are appended from here
     long long pad2;
 };
 
 // Ray queue.  A record is 6 + nb words -- emitter, birth step, direction (dx,
-// dy, dz), level << 28 | NESTED pixel, photons per bin -- kept in arrays of
-// 16-, 8- and 4-byte pieces, so that a warp reads or writes a record in a few
-// coalesced vector accesses (three at four bins, where an array a word took
-// ten, with ten addresses):
-//   a   emitter id, birth step, dx, dy
-//   the tail words dz, pixel word, photons[0..nb): as many 16-byte pieces t4
-//   as they fill, then an 8-byte piece t2 and a 4-byte piece t1 for the rest
-// Merged rays only (Sec. 3.3; null when merging is not built in):
-//   m   position at the merge (2^-21 cell), vertex << 31 | simulation << 16 |
-//       distance travelled at the merge
-//   mthr  termination threshold, code photons
+// dy, dz), level << 28 | NESTED pixel, photons per bin -- in tiles of 32
+// records, one contiguous run of 128 (6 + nb) bytes that a warp reads with a
+// few coalesced vector accesses (three at four bins) from one address.  A
+// tile holds, 32 records each:
+//   16-byte pieces: emitter id, birth step, dx, dy
+//   the tail words dz, pixel word, photons[0..nb): as many 16-byte pieces as
+//   they fill, then 8-byte and 4-byte pieces for the rest
+// and in queues of engines built for merging (Sec. 3.3), for merged rays only:
+//   16-byte pieces: position at the merge (2^-21 cell), vertex << 31 |
+//   simulation << 16 | distance travelled at the merge
+//   4-byte pieces: termination threshold, code photons
 struct Queue {
-    uint4 *a;
-    uint4 *t4[2];
-    uint2 *t2;
-    uint32_t *t1;
-    uint4 *m;
-    float *mthr;
+    char *base;
+    uint32_t tile;           // bytes of a tile
+    int32_t nb;
 };
 
-// tail word w (0: dz, 1: pixel word, 2 + b: photons of bin b) of ray i
-__host__ __device__ inline uint32_t *tail_word(const Queue &q, int nb, int w, long long i) {
-    const int n4 = (2 + nb) >> 2;
-    if (w < 4 * n4) return reinterpret_cast<uint32_t *>(q.t4[w >> 2] + i) + (w & 3);
-    if (((2 + nb) & 2) && w < 4 * n4 + 2) return reinterpret_cast<uint32_t *>(q.t2 + i) + (w - 4 * n4);
-    return q.t1 + i;
+__host__ __device__ constexpr uint32_t tile_bytes(int nb, bool merged) { return 128u * (6 + nb + (merged ? 5 : 0)); }
+// byte offset in a tile of the piece of tail word w (0: dz, 1: pixel word,
+// 2 + b: photons of bin b), of the merge words and of the threshold; a
+// record's own piece is (i & 31) pieces further
+__host__ __device__ inline char *tile_of(const Queue &q, long long i) { return q.base + (i >> 5) * (long long)q.tile; }
+__host__ __device__ inline uint4 *ray_head(const Queue &q, long long i) {
+    return reinterpret_cast<uint4 *>(tile_of(q, i)) + (i & 31);
+}
+__host__ __device__ inline uint32_t *tail_word(const Queue &q, int w, long long i) {
+    const int T = 2 + q.nb, n4 = T >> 2;
+    char *t = tile_of(q, i) + 512;
+    const int r = (int)(i & 31);
+    if (w < 4 * n4) return reinterpret_cast<uint32_t *>(t + 512 * (w >> 2) + 16 * r) + (w & 3);
+    t += 512 * n4;
+    if ((T & 2) && w < 4 * n4 + 2) return reinterpret_cast<uint32_t *>(t + 8 * r) + (w - 4 * n4);
+    return reinterpret_cast<uint32_t *>(t + ((T & 2) ? 256 : 0) + 4 * r);
 }
 // the pixel word of ray i (DEAD_RAY marks an unused slot)
-__host__ __device__ inline uint32_t *pixel_word(const Queue &q, int nb, long long i) {
-    return nb >= 2 ? reinterpret_cast<uint32_t *>(q.t4[0] + i) + 1 : reinterpret_cast<uint32_t *>(q.t2 + i) + 1;
+__host__ __device__ inline uint32_t *pixel_word(const Queue &q, long long i) {
+    return reinterpret_cast<uint32_t *>(tile_of(q, i) + 512 + (i & 31) * (q.nb >= 2 ? 16 : 8)) + 1;
+}
+__host__ __device__ inline uint4 *ray_merge(const Queue &q, long long i) {
+    return reinterpret_cast<uint4 *>(tile_of(q, i) + 128 * (6 + q.nb)) + (i & 31);
+}
+__host__ __device__ inline float *ray_thr(const Queue &q, long long i) {
+    return reinterpret_cast<float *>(tile_of(q, i) + 128 * (6 + q.nb) + 512) + (i & 31);
 }
 
 struct Cells {

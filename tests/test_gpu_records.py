@@ -8,7 +8,7 @@ import pytest
 
 import paper_2409_04521_gb300 as F
 import workloads as W
-from parity_util import run_pair
+from parity_util import ray_table, run_pair
 
 pytestmark = pytest.mark.gpu
 
@@ -53,3 +53,24 @@ def test_checkpoint_keeps_one_array_a_word(nb):
     assert np.array_equal(t.save_state(), blob)
     s.close()
     t.close()
+
+
+def test_children_beyond_the_batch_pixel_table():
+    # the batch's table is sized by its own N_min; a member with a larger one
+    # splits deeper, past the table, and must get the directions it gets alone
+    p = W.batch_member(3, sizes=(16,), nsteps=9)
+    p = dc.replace(p, options=dc.replace(p.options, n_ray_min=200.0))
+    b = F.Batch(max_sims=2, max_grid=16, nbins=3, ray_capacity=1 << 22, cell_capacity=2 * 16 ** 3,
+                emitter_capacity=128, n_ray_min=3.0)
+    slot = b.add(p)
+    s = F.Simulation(p, ray_capacity=1 << 22)
+    for _ in range(p.nsteps):
+        b.step()
+        s.step(p.dt)
+    kb, db, Nb = ray_table(b.rays(slot))
+    ks, ds, Ns = ray_table(s.rays())
+    assert ks[:, 2].max() >= 7                            # table levels 0..6
+    assert np.array_equal(kb, ks) and np.array_equal(db, ds)
+    assert np.allclose(Nb, Ns, rtol=1e-5, atol=1e-9 * Ns.max())
+    b.close()
+    s.close()
