@@ -615,6 +615,35 @@ __device__ __forceinline__ void red_add_v4(float4 *addr, float a, float b, float
 }
 
 // ---------------------------------------------------------------------------
+// Bulk copies global -> shared with an mbarrier (sizes and addresses multiples
+// of 16 bytes).  One thread announces the bytes and starts the copy; every
+// reader waits for the barrier's phase.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void mbar_init(unsigned bar, unsigned arrivals) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(arrivals) : "memory");
+}
+__device__ __forceinline__ void bulk_load(unsigned dst, const void *src, unsigned bytes, unsigned bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+// false if the phase did not complete within the limit (a second or so)
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+    for (int k = 0; k < (1 << 20); ++k) {
+        unsigned done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
+// ---------------------------------------------------------------------------
 // Rate coefficients in single precision (temperature-dependent fits cited by
 // Sec. 4.1: Hui & Gnedin 1997 for case-B recombination, recombination cooling
 // and collisional ionisation; Cen 1992 for collisional excitation and

@@ -321,8 +321,8 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
     sm_count_ = std::max(sms, 1);
     const int ext = ext_variants();
     if (!march_variant_exists(cfg_.nb, march_agg_, march_minb_, ext)) { march_agg_ = 0; march_minb_ = 2; }
-    CK(march_prepare(cfg_.nb, march_agg_, march_minb_, ms, ext));
-    const int per_sm = march_max_blocks_per_sm(cfg_.nb, march_agg_, march_minb_, march_threads_, ms, ext);
+    CK(march_prepare(cfg_.nb, march_agg_, march_minb_, ms, ext, q_[0].tile));
+    const int per_sm = march_max_blocks_per_sm(cfg_.nb, march_agg_, march_minb_, march_threads_, ms, ext, q_[0].tile);
     if (per_sm < 1) return fail(FLEXRT_E_INVALID, "too many simulation slots for one march block");
     march_blocks_ = sm_count_ * std::max(per_sm, 1);
     chem_blocks_ = (int)std::max<long long>(1, std::min<long long>((nc + 255) / 256, (long long)sm_count_ * 8));
@@ -712,6 +712,7 @@ flexrt_status Engine::poll(bool wait) {
         latched_ = FLEXRT_E_CAPACITY;
         if (v & 1) err_ = "ray queue capacity exceeded; state kept at the last complete step";
         else if (v & 8) err_ = "merge group too heavy for exact weighted sums (more than 2^13 rays as bright as its brightest)";
+        else if (v & 16) err_ = "a march's copy of its rays did not complete (internal limit)";
         else if (v & 2) err_ = "ray older than the rotation ring (internal bound)";
         else err_ = "ray crossed more than four cells in one step (internal bound)";
     }
@@ -1105,8 +1106,8 @@ flexrt_status Engine::set_launch(int agg, int minb, int blocks_per_sm, int threa
     if (!march_variant_exists(cfg_.nb, agg, minb, ext_variants()) || blocks_per_sm < 0 || blocks_per_sm > 32 ||
         (threads != 128 && threads != 256) || slab < 32 || slab > 4096)
         return fail(FLEXRT_E_INVALID, "march kernel variant not built or launch shape out of range");
-    CK(march_prepare(cfg_.nb, agg, minb, (int)slots_.size(), ext_variants()));
-    const int lim = march_max_blocks_per_sm(cfg_.nb, agg, minb, threads, (int)slots_.size(), ext_variants());
+    CK(march_prepare(cfg_.nb, agg, minb, (int)slots_.size(), ext_variants(), q_[0].tile));
+    const int lim = march_max_blocks_per_sm(cfg_.nb, agg, minb, threads, (int)slots_.size(), ext_variants(), q_[0].tile);
     if (lim < 1) return fail(FLEXRT_E_INVALID, "variant cannot be resident");
     const int bps = blocks_per_sm == 0 ? lim : std::min(blocks_per_sm, lim);
     march_agg_ = agg;

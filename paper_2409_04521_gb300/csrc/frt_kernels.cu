@@ -716,10 +716,10 @@ static MarchFn march_fn(int nb, int agg, int minb, int ext) {
     }
 }
 bool march_variant_exists(int nb, int agg, int minb, int ext) { return march_fn(nb, agg, minb, ext) != nullptr; }
-cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext) {
+cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext, uint32_t tile) {
     MarchFn f = march_fn(nb, agg, minb, ext);
     if (!f) return cudaErrorInvalidValue;
-    const size_t sh = march_shared_bytes(nsims);
+    const size_t sh = march_shared_bytes(nsims, tile, 256);
     if (sh > 48 * 1024) return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
     return cudaSuccess;
 }
@@ -727,14 +727,14 @@ cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int bloc
                          int ext) {
     MarchFn f = march_fn(nb, agg, minb, ext);
     if (!f) return cudaErrorInvalidValue;
-    f<<<blocks, threads, march_shared_bytes(a.nsims), st>>>(a);
+    f<<<blocks, threads, march_shared_bytes(a.nsims, a.q[0].tile, threads), st>>>(a);
     return cudaGetLastError();
 }
-int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, int ext) {
+int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, int ext, uint32_t tile) {
     MarchFn f = march_fn(nb, agg, minb, ext);
     if (!f) return 0;
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, threads, march_shared_bytes(nsims));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, threads, march_shared_bytes(nsims, tile, threads));
     return n;
 }
 cudaError_t launch_chem(const ChemArgs &a, int blocks, cudaStream_t st) {

@@ -75,10 +75,10 @@ MarchFn march_fn_gen(int nb, int agg, int minb);
 // ext: 0 plain, 1 merged rays, 3 merged rays and Generalized mode
 bool march_variant_exists(int nb, int agg, int minb, int ext);
 // opt the variant into the dynamic shared memory `nsims` slots need
-cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext);
+cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext, uint32_t tile);
 cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int blocks, int threads, cudaStream_t st,
                          int ext);
-int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, int ext);
+int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, int ext, uint32_t tile);
 cudaError_t launch_chem(const ChemArgs &a, int blocks, cudaStream_t st);
 cudaError_t launch_end(Ctl *c, SimDev *sims, SimAcc *acc, int nsims, cudaStream_t st);
 // between passes of the iteration: drop the march's output and the step's tallies (not emission)

@@ -58,8 +58,13 @@ struct MarchSim {
     float sig[MAXB], sige[MAXB], eh[MAXB];
 };
 
-__host__ __device__ constexpr size_t march_shared_bytes(int nsims) {
-    return (size_t)nsims * (NACC * sizeof(unsigned long long) + sizeof(MarchSim));
+// shared memory of a march block: tallies and constants per simulation, then
+// two tiles of ray records per warp
+__host__ __device__ constexpr size_t march_tiles_offset(int nsims) {
+    return ((size_t)nsims * (NACC * sizeof(unsigned long long) + sizeof(MarchSim)) + 127) & ~(size_t)127;
+}
+__host__ __device__ constexpr size_t march_shared_bytes(int nsims, uint32_t tile, int threads) {
+    return march_tiles_offset(nsims) + (size_t)(threads / 32) * 2 * tile;
 }
 
 // (1 - e^-t)/t for 0 <= t < 1/8, from -t: its Taylor series through t^4 (the
@@ -173,7 +178,8 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
     constexpr bool MRG = (EXT & 1) != 0, GEN = (EXT & 2) != 0;
     // per-simulation tallies of this block (photons in 2^-32 fixed point,
     // counts as integers), then the staged constants
-    extern __shared__ unsigned long long sh_acc[];
+    extern __shared__ __align__(128) unsigned long long sh_acc[];
+    __shared__ __align__(8) unsigned long long sh_bar[8][2];
     __shared__ unsigned char sh_parent[8][32];     // splitting lanes of each warp, in order
     unsigned char *const parent = sh_parent[threadIdx.x >> 5];
     MarchSim *msim = reinterpret_cast<MarchSim *>(sh_acc + A.nsims * NACC);
@@ -191,15 +197,22 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             if (b < S.nb) m.sig_max = fmaxf(m.sig_max, S.sig[b]);
         }
     }
+    const int lane = lane_id();
+    const unsigned tile = A.q[0].tile;
+    // this warp's two tiles and their barriers (one arrival each: lane 0's)
+    char *const tiles = reinterpret_cast<char *>(sh_acc) + march_tiles_offset(A.nsims) + (threadIdx.x >> 5) * 2 * tile;
+    const unsigned tiles_s = smem_addr(tiles), bars_s = smem_addr(sh_bar[threadIdx.x >> 5]);
+    if (lane == 0) {
+        mbar_init(bars_s, 1);
+        mbar_init(bars_s + 8, 1);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
     __syncthreads();
     Ctl *C = A.ctl;
-    const int lane = lane_id();
     if (C->err == 0) {
         const int par = C->par;
-        // (one base address a queue: an address an array took 28 registers)
         const char *const qin = A.q[par].base;
         char *const qout = A.q[par ^ 1].base;
-        const unsigned tile = A.q[0].tile;
         unsigned long long *out_cnt = (unsigned long long *)&C->cnt[par ^ 1];
         // queue slots stay below 2^31 (the engine's bound), so 32-bit indices
         const unsigned n = (unsigned)(C->cnt[par] + C->emit_total);
@@ -215,37 +228,52 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
         float t_esc = 0.0f, t_out = 0.0f;
         unsigned t_cnt = 0u, t_rout = 0u;
         int t_sim = -1, t_n = 0;
-        for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < nr; i += stride) {
-            // the ray's words: every piece at once, the pixel word among them
-            // (a dead slot's other words are old ones, and are not used)
-            uint4 ra = make_uint4(0u, 0u, 0u, 0u);
-            uint32_t w[2 + NB];
-            w[1] = DEAD_RAY;
-            if (i < n) {
-                const char *t = qin + (size_t)(i >> 5) * tile;       // the warp's tile: i & 31 is the lane
-                ra = __ldcs(reinterpret_cast<const uint4 *>(t) + lane);
-                load_tail<NB, true>(t, lane, w);
+        unsigned i = blockIdx.x * blockDim.x + threadIdx.x;       // i & 31 is the lane: a warp marches one tile
+        auto fetch = [&](unsigned j, unsigned b) {
+            bulk_load(tiles_s + b * tile, qin + (size_t)(j >> 5) * tile, tile, bars_s + 8 * b);
+        };
+        if (lane == 0) {
+            if (i < nr) fetch(i, 0);
+            if (i < nr && stride < nr - i) fetch(i + stride, 1);
+        }
+        for (; i < nr; i += stride) {
+            // the tile's records, fetched two iterations ago (the copy hides
+            // behind a whole iteration).  Words are read from shared memory
+            // when they are needed, the unchanged ones again at the end: held
+            // in registers they would spill (a dead slot's words are not used)
+            const unsigned buf = w_it & 1;
+            const char *const rec = tiles + buf * tile;
+            if (!__all_sync(FULL, mbar_wait(bars_s + 8 * buf, (w_it >> 1) & 1))) {
+                // never in a working machine: report, let the other tile's copy end, stop
+                if (lane == 0) {
+                    atomicOr(&C->err, 16);
+                    if (i + stride < nr) mbar_wait(bars_s + 8 * (buf ^ 1), ((w_it + 1) >> 1) & 1);
+                }
+                break;
             }
-            const uint32_t e = ra.x, pl = w[1];
-            const int bi = (int)ra.y, dx = (int)ra.z, dy = (int)ra.w, dz = (int)w[0];
-            float ph[NB];
-#pragma unroll
-            for (int b = 0; b < NB; ++b) ph[b] = __uint_as_float(w[2 + b]);
-            bool valid = pl != DEAD_RAY;
-            const bool mrg = MRG && valid && (e & MERGED_BIT);
-            int mx = 0, my = 0, mz = 0;
-            uint32_t ma = 0;
-            float mthr = 0.0f;
-            if (mrg) {
-                const char *t = qin + (size_t)(i >> 5) * tile + 128 * (6 + NB);
-                const uint4 rm = __ldcs(reinterpret_cast<const uint4 *>(t) + lane);
-                mx = (int)rm.x; my = (int)rm.y; mz = (int)rm.z; ma = rm.w;
-                mthr = __ldcs(reinterpret_cast<const float *>(t + 512) + lane);
-            }
-            int sim = 0;
+            const uint4 *const heads = reinterpret_cast<const uint4 *>(rec);
+            const uint2 *const tails = reinterpret_cast<const uint2 *>(rec + 512);
+            constexpr int TW = NB >= 2 ? 2 : 1;                   // a record's dz and pixel word, in uint2 strides
+            const uint4 *const merged = reinterpret_cast<const uint4 *>(rec + 128 * (6 + NB));
+            const float *const mthrs = reinterpret_cast<const float *>(rec + 128 * (6 + NB) + 512);
+            bool valid = false, mrg = false;
+            int sim = 0, age = 0;
+            // (1) integer walk of this step
+            int key[4];
+            float ds[4];
+            bool esc = false;
+            {
+            const uint4 ra = heads[lane];
+            const uint2 rt = tails[lane * TW];
+            const uint32_t e = ra.x;
+            const int bi = (int)ra.y, dx = (int)ra.z, dy = (int)ra.w, dz = (int)rt.x;
+            valid = i < n && rt.y != DEAD_RAY;
+            mrg = MRG && valid && (e & MERGED_BIT);
+            uint4 rm = make_uint4(0u, 0u, 0u, 0u);
+            if (mrg) rm = merged[lane];
             int4 ec = make_int4(0, 0, 0, 0);
             if (mrg) {
-                sim = (int)((ma >> 16) & 0x7fffu);
+                sim = (int)((rm.w >> 16) & 0x7fffu);
             } else if (valid) {
                 ec = __ldg(&A.em.cell[e]);
                 sim = ec.w;
@@ -256,39 +284,41 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             // `since` steps from its merge position and had travelled its
             // constituents' mean distance when it was made.
             const int since = S.step - bi - 1;
-            const int age = mrg ? (int)(ma & 0xffffu) + since : S.step - bi;
+            age = mrg ? (int)(rm.w & 0xffffu) + since : S.step - bi;
             if (valid && (mrg ? since < 0 : (age < 0 || age >= A.em.ring_w))) {
                 atomicOr(&C->err, 2);
                 valid = false;
             }
-
-            // (1) integer walk of this step
-            int key[4];
-            float ds[4];
-            bool esc = false;
-            {
-                // a queued ray is inside the box at the start of its step, so
-                // its position (at most 1000 cells of 2^21) fits 32 bits
-                int px, py, pz;
-                if (mrg) {
-                    px = mx + since * dx;
-                    py = my + since * dy;
-                    pz = mz + since * dz;
-                } else {
-                    px = ((2 * ec.x + 1) << (FRAC_BITS - 1)) + age * dx;
-                    py = ((2 * ec.y + 1) << (FRAC_BITS - 1)) + age * dy;
-                    pz = ((2 * ec.z + 1) << (FRAC_BITS - 1)) + age * dz;
-                }
-                // slots may be empty: every later phase visits the four slots
-                // in order and skips the empty ones (negative keys)
-                walk_step(valid, px, py, pz, dx, dy, dz, S.nx, S.ny, S.nz, (int)S.coff, key, ds, esc);
+            // a queued ray is inside the box at the start of its step, so
+            // its position (at most 1000 cells of 2^21) fits 32 bits
+            int px, py, pz;
+            if (mrg) {
+                px = (int)rm.x + since * dx;
+                py = (int)rm.y + since * dy;
+                pz = (int)rm.z + since * dz;
+            } else {
+                px = ((2 * ec.x + 1) << (FRAC_BITS - 1)) + age * dx;
+                py = ((2 * ec.y + 1) << (FRAC_BITS - 1)) + age * dy;
+                pz = ((2 * ec.z + 1) << (FRAC_BITS - 1)) + age * dz;
             }
+            // slots may be empty: every later phase visits the four slots
+            // in order and skips the empty ones (negative keys)
+            walk_step(valid, px, py, pz, dx, dy, dz, S.nx, S.ny, S.nz, (int)S.coff, key, ds, esc);
+            }
+            const MarchSim &S = msim[sim];
             int nseg = 4 + (key[0] >> 31) + (key[1] >> 31) + (key[2] >> 31) + (key[3] >> 31);
             // (2) opacities of the crossed cells (Generalized mode: also the
             // ionised fraction and the screen's share)
             float2 kc[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) kc[j] = key[j] >= 0 ? __ldg(&A.cells.kap[key[j]]) : make_float2(0.f, 0.f);
+            float ph[NB];
+            {
+                uint32_t w[2 + NB];
+                load_tail<NB, false>(rec, lane, w);
+#pragma unroll
+                for (int b = 0; b < NB; ++b) ph[b] = __uint_as_float(w[2 + b]);
+            }
             const bool gen = GEN && valid && S.gen;
             float xg[4], rg[4];
 #pragma unroll
@@ -351,10 +381,10 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
 #pragma unroll
             for (int b = 0; b < NB; ++b) s_end += ph[b];
             int nout = 0, m = 0;
-            const int lev = (int)(pl >> LEVEL_SHIFT);
             if (GEN && screened) esc = false;
             if (valid && !esc && !(GEN && screened)) {
-                const float thr = mrg ? mthr : S.eps * __ldg(&A.em.n0[e]) * pow2_neg(2 * (lev - S.l_src));
+                const int lev = (int)(tails[lane * TW].y >> LEVEL_SHIFT);
+                const float thr = mrg ? mthrs[lane] : S.eps * __ldg(&A.em.n0[heads[lane].x]) * pow2_neg(2 * (lev - S.l_src));
                 if (s_end < thr) {
                     // termination: the ray's last photons stay in its last cell
                     float g = 0.f, h = 0.f;
@@ -441,15 +471,17 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                 if (fits && nout == 1) {
                     const unsigned o = slot_of(k0);
                     char *const t = qout + (size_t)(o >> 5) * tile;
-                    __stcs(reinterpret_cast<uint4 *>(t) + (o & 31u), ra);
+                    __stcs(reinterpret_cast<uint4 *>(t) + (o & 31u), heads[lane]);
+                    const uint2 rt = tails[lane * TW];
+                    uint32_t w[2 + NB];
+                    w[0] = rt.x; w[1] = rt.y;
 #pragma unroll
                     for (int b = 0; b < NB; ++b) w[2 + b] = __float_as_uint(ph[b]);
                     store_tail<NB, true>(t, o & 31u, w);
                     if (mrg) {
                         char *const tm = t + 128 * (6 + NB);
-                        __stcs(reinterpret_cast<uint4 *>(tm) + (o & 31u),
-                               make_uint4((uint32_t)mx, (uint32_t)my, (uint32_t)mz, ma));
-                        __stcs(reinterpret_cast<float *>(tm + 512) + (o & 31u), mthr);
+                        __stcs(reinterpret_cast<uint4 *>(tm) + (o & 31u), merged[lane]);
+                        __stcs(reinterpret_cast<float *>(tm + 512) + (o & 31u), mthrs[lane]);
                     }
                 }
                 // children: the warp makes the children of all its splitting
@@ -468,14 +500,21 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                     if ((grp >> lane) & 1u) parent[__popc(grp & ((1u << lane) - 1u))] = (unsigned char)lane;
                     __syncwarp();
                     // children keep their parent's sphere (Sec. 3.2): the
-                    // emitter's of the birth step, or the merge cell's
-                    int4 mrows[3];
-                    const bool anym = MRG && __any_sync(FULL, mrg && ((grp >> lane) & 1u));
-                    if (MRG) {
-                        mrows[0] = mrows[1] = mrows[2] = make_int4(0, 0, 0, 0);
-                        if (mrg && ((grp >> lane) & 1u)) {
+                    // emitter's of the birth step (whose slot of the ring the
+                    // age gives: it is less than the ring's length), or the
+                    // merge cell's; each parent's lane gets the rows
+                    int4 prow[3];
+                    prow[0] = prow[1] = prow[2] = make_int4(0, 0, 0, 0);
+                    if ((grp >> lane) & 1u) {
+                        const uint4 ra = heads[lane];
+                        if (mrg) {
                             const SimDev &SD = A.sims[sim];
-                            rotation_rows(SD.seed, (1LL << 31) + (long long)(e & ~MERGED_BIT), bi, SD.rotate, mrows);
+                            rotation_rows(SD.seed, (1LL << 31) + (long long)(ra.x & ~MERGED_BIT), (int)ra.y, SD.rotate, prow);
+                        } else {
+                            int slot = S.ring0 - age;
+                            if (slot < 0) slot += A.em.ring_w;
+                            const int4 *rg = A.em.ring + ((long long)ra.x * A.em.ring_w + slot) * 3;
+                            prow[0] = rg[0]; prow[1] = rg[1]; prow[2] = rg[2];
                         }
                     }
                     const float scale = pow2_neg(2 * mm);
@@ -484,34 +523,22 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                         const unsigned c = c0 + lane;
                         const int src = parent[c < all ? c >> (2 * mm) : 0u];
                         const unsigned sub = c & ((1u << (2 * mm)) - 1u);
-                        const uint32_t ppl = __shfl_sync(FULL, pl, src), pe = __shfl_sync(FULL, e, src);
-                        const int pbi = __shfl_sync(FULL, bi, src), psim = __shfl_sync(FULL, sim, src);
-                        const int pk = __shfl_sync(FULL, k0, src);
+                        const uint4 pa = heads[src];
+                        const uint32_t ppl = tails[src * TW].y;
+                        const int psim = __shfl_sync(FULL, sim, src), pk = __shfl_sync(FULL, k0, src);
                         uint32_t cw[2 + NB];
 #pragma unroll
                         for (int b = 0; b < NB; ++b) cw[2 + b] = __float_as_uint(__shfl_sync(FULL, ph[b], src) * scale);
                         int4 rows[3];
-                        uint4 pm = make_uint4(0u, 0u, 0u, 0u);
-                        float pthr = 0.0f;
-                        if (MRG && anym) {
 #pragma unroll
-                            for (int r = 0; r < 3; ++r)
-                                rows[r] = make_int4(__shfl_sync(FULL, mrows[r].x, src), __shfl_sync(FULL, mrows[r].y, src),
-                                                    __shfl_sync(FULL, mrows[r].z, src), 0);
-                            pm = make_uint4((uint32_t)__shfl_sync(FULL, mx, src), (uint32_t)__shfl_sync(FULL, my, src),
-                                            (uint32_t)__shfl_sync(FULL, mz, src), __shfl_sync(FULL, ma, src));
-                            pthr = __shfl_sync(FULL, mthr, src);
-                        }
+                        for (int r = 0; r < 3; ++r)
+                            rows[r] = make_int4(__shfl_sync(FULL, prow[r].x, src), __shfl_sync(FULL, prow[r].y, src),
+                                                __shfl_sync(FULL, prow[r].z, src), 0);
                         if (c < all) {
                             const int plev = (int)(ppl >> LEVEL_SHIFT), L = plev + mm;
-                            const bool pmrg = MRG && (pe & MERGED_BIT);
-                            if (!pmrg) {
-                                // the birth step's slot of the ring: the age is less than its length
-                                int slot = msim[psim].ring0 - (msim[psim].step - pbi);
-                                if (slot < 0) slot += A.em.ring_w;
-                                const int4 *rg = A.em.ring + ((long long)pe * A.em.ring_w + slot) * 3;
-                                rows[0] = rg[0]; rows[1] = rg[1]; rows[2] = rg[2];
-                            }
+                            const bool pmrg = MRG && (pa.x & MERGED_BIT);
+                            uint4 pm = make_uint4(0u, 0u, 0u, 0u);
+                            if (pmrg) pm = merged[src];
                             const uint32_t pix = pmrg && (pm.w >> 31)
                                                      ? vertex_child(msim[psim].l_merge, ppl & PIX_MASK, plev, mm, sub)
                                                      : ((ppl & PIX_MASK) << (2 * mm)) + sub;
@@ -523,18 +550,21 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                             cw[0] = (uint32_t)cz;
                             cw[1] = ((uint32_t)L << LEVEL_SHIFT) | pix;
                             char *const t = qout + (size_t)(o >> 5) * tile;
-                            reinterpret_cast<uint4 *>(t)[o & 31u] = make_uint4(pe, (uint32_t)pbi, (uint32_t)cx, (uint32_t)cy);
+                            reinterpret_cast<uint4 *>(t)[o & 31u] = make_uint4(pa.x, pa.y, (uint32_t)cx, (uint32_t)cy);
                             store_tail<NB, false>(t, o & 31u, cw);
                             if (pmrg) {
                                 char *const tm = t + 128 * (6 + NB);
                                 pm.w &= 0x7fffffffu;
                                 reinterpret_cast<uint4 *>(tm)[o & 31u] = pm;
-                                reinterpret_cast<float *>(tm + 512)[o & 31u] = pthr * scale;
+                                reinterpret_cast<float *>(tm + 512)[o & 31u] = mthrs[src] * scale;
                             }
                         }
                     }
                 }
             }
+            // every lane is done with the tile: fetch the one after next into it
+            __syncwarp();
+            if (lane == 0 && 2u * stride < nr - i) fetch(i + 2u * stride, buf);
             ++w_it;
         }
         for (int k = lane; k < slab_left; k += 32) *pixel_word(A.q[par ^ 1], slab + k) = DEAD_RAY;
