@@ -740,7 +740,17 @@ flexrt_status Engine::launch_step() {
 flexrt_status Engine::launch_stage(int stage) {
     const int ms = (int)slots_.size();
     EmitArgs ea{ctl_, sims_, acc_, {q_[0], q_[1]}, qcap_, em_, pixtab_, ltab_, cfg_.nb};
-    MarchArgs ma{ctl_, sims_, acc_, ms, {q_[0], q_[1]}, qcap_, em_, cells_, pixtab_, ltab_, march_slab_};
+    MarchArgs ma{ctl_, sims_, acc_, ms, {q_[0], q_[1]}, qcap_, em_, cells_, pixtab_, ltab_, march_slab_, {}};
+    if (one_sim()) {
+        const SimDev &h = slots_[0].h;
+        MarchSim &o = ma.one;
+        o.nx = h.nx; o.ny = h.ny; o.nz = h.nz; o.l_src = h.l_src; o.l_max = h.l_max; o.active = h.active;
+        o.l_merge = h.l_merge; o.gen = h.gen_mode; o.coff = h.cell_off; o.eps = h.eps_term;
+        for (int b = 0; b < MAXB; ++b) {
+            o.sig[b] = h.sig[b]; o.sige[b] = h.sige[b]; o.eh[b] = h.eh[b];
+            if (b < h.nb) o.sig_max = std::max(o.sig_max, h.sig[b]);
+        }
+    }
     ChemArgs ca{ctl_, sims_, acc_, ms, cells_, rg_, 1};
     const bool prof = profiling_ && !cfg_.use_graph;
     cudaEvent_t e0 = nullptr;

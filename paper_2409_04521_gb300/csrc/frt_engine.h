@@ -104,8 +104,11 @@ class Engine {
                               double *thr, int64_t *n);
     bool merge_built() const { return cfg_.merge_l_max >= 0; }
     // the march variants: 0 plain, 1 with merged rays, 3 with merged rays
-    // and the moving screen (engines that may run Generalized members)
-    int ext_variants() const { return cfg_.gen_capable ? 3 : (merge_built() ? 1 : 0); }
+    // and the moving screen (engines that may run Generalized members); plus 4
+    int ext_variants() const { return (cfg_.gen_capable ? 3 : (merge_built() ? 1 : 0)) | (one_sim() ? 4 : 0); }
+    // one simulation, steps launched directly (a graph would keep the
+    // constants of a member replaced since)
+    bool one_sim() const { return cfg_.max_sims == 1 && !cfg_.use_graph; }
     flexrt_status ionized_volume(int slot, double *x_ion);
     // checkpoint of a single-simulation engine (slot 0): bytes needed, save, load
     flexrt_status save_state(int slot, void *buf, int64_t cap, int64_t *bytes);

@@ -671,45 +671,19 @@ cudaError_t launch_queue_words(const Queue &q, bool merged, long long n, uint32_
     k_queue_words<<<blocks, 256, 0, st>>>(q, merged ? 1 : 0, n, words, join ? 1 : 0);
     return cudaGetLastError();
 }
-// Kernel variants: every bin count with the default (AGG 0, 2 blocks/SM);
-// the bin counts of the standard spectra (1, 3, 4) with every aggregation
-// and register budget, for the autotuner.  The variants with merged rays
-// are built in frt_merge.cu, those that also run Generalized members in
-// frt_march_gen.cu.
-static MarchFn march_fn_plain(int nb, int agg, int minb) {
-#define FRT_V(NB)                                                                   \
-    if (nb == NB) {                                                                \
-        if (agg == 0 && minb == 2) return k_march<NB, 0, 2, 0>;                    \
-        if (agg == 0 && minb == 3) return k_march<NB, 0, 3, 0>;                    \
-        if (agg == 0 && minb == 4) return k_march<NB, 0, 4, 0>;                    \
-        if (agg == 1 && minb == 2) return k_march<NB, 1, 2, 0>;                    \
-        if (agg == 1 && minb == 3) return k_march<NB, 1, 3, 0>;                    \
-        if (agg == 1 && minb == 4) return k_march<NB, 1, 4, 0>;                    \
-        if (agg == 2 && minb == 2) return k_march<NB, 2, 2, 0>;                    \
-        if (agg == 2 && minb == 3) return k_march<NB, 2, 3, 0>;                    \
-        if (agg == 2 && minb == 4) return k_march<NB, 2, 4, 0>;                    \
-        return nullptr;                                                            \
-    }
-    FRT_V(1)
-    FRT_V(3)
-    FRT_V(4)
-#undef FRT_V
-#define FRT_W(NB)                                                                   \
-    if (nb == NB && agg == 0) {                                                    \
-        if (minb == 2) return k_march<NB, 0, 2, 0>;                                \
-        if (minb == 3) return k_march<NB, 0, 3, 0>;                                \
-    }
-    FRT_W(2)
-    FRT_W(5)
-    FRT_W(6)
-    FRT_W(7)
-    FRT_W(8)
-#undef FRT_W
-    return nullptr;
-}
+// The plain variants are built here, those with merged rays in frt_merge.cu,
+// the others in frt_march_gen.cu and frt_march_one*.cu.
 static MarchFn march_fn(int nb, int agg, int minb, int ext) {
-    switch (ext) {
-        case 0: return march_fn_plain(nb, agg, minb);
+    if (agg == 0) {
+        switch (ext) {
+            case 4: return march_fn_one(nb, agg, minb);
+            case 5: return march_fn_one_merge(nb, agg, minb);
+            case 7: return march_fn_one_gen(nb, agg, minb);
+            default: break;
+        }
+    }
+    switch (ext & 3) {
+        case 0: return march_pick<0, false>(nb, agg, minb);
         case 1: return march_fn_merge(nb, agg, minb);
         case 3: return march_fn_gen(nb, agg, minb);
         default: return nullptr;

@@ -17,6 +17,17 @@ struct EmitArgs {
     int nb;
 };
 
+// The per-simulation constants the march needs, staged in shared
+// memory; an engine with one simulation passes them with the launch.
+struct MarchSim {
+    int nx, ny, nz, step, l_src, l_max, active, l_merge, gen, ring0, pad1, pad2;   // ring0: this step's ring slot
+    long long coff;
+    float eps;
+    float sig_max;          // largest sigma_b / sigma_ref of the bins
+    int K[MAXL];
+    float sig[MAXB], sige[MAXB], eh[MAXB];
+};
+
 struct MarchArgs {
     Ctl *ctl;
     const SimDev *sims;
@@ -29,6 +40,7 @@ struct MarchArgs {
     const int4 *pixtab;
     int ltab;
     int slab;                // output slots a warp reserves at once (run length, 32..4096)
+    MarchSim one;            // the only simulation's constants (variants with ext bit 2; its step is the device's)
 };
 
 struct MergeArgs {
@@ -67,12 +79,18 @@ cudaError_t launch_far(const EmitArgs &a, int blocks, cudaStream_t st);
 // a queue's first n records to (join: from) one array of n words per word of the record
 cudaError_t launch_queue_words(const Queue &q, bool merged, long long n, uint32_t *words, bool join,
                                cudaStream_t st);
-using MarchFn = void (*)(MarchArgs);
-// the march variant with merged rays (nullptr if not built)
+using MarchFn = void (*)(const MarchArgs);
+// the march variants (nullptr if not built): with merged rays, with merged
+// rays and Generalized Opacity mode, and all three for engines with one
+// simulation
 MarchFn march_fn_merge(int nb, int agg, int minb);
-// the variant with merged rays and Generalized Opacity mode (nullptr if not built)
 MarchFn march_fn_gen(int nb, int agg, int minb);
-// ext: 0 plain, 1 merged rays, 3 merged rays and Generalized mode
+MarchFn march_fn_one(int nb, int agg, int minb);
+MarchFn march_fn_one_merge(int nb, int agg, int minb);
+MarchFn march_fn_one_gen(int nb, int agg, int minb);
+// ext: 0 plain, 1 merged rays, 3 merged rays and Generalized mode; plus 4:
+// one simulation, launched directly (its variants exist without aggregation;
+// with it the general one runs)
 bool march_variant_exists(int nb, int agg, int minb, int ext);
 // opt the variant into the dynamic shared memory `nsims` slots need
 cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext, uint32_t tile);

@@ -48,23 +48,29 @@ __device__ __forceinline__ void flush_tallies(float &esc, float &out, unsigned &
     tsim = -1;
 }
 
-// The per-simulation constants the march needs, staged in shared memory.
-struct MarchSim {
-    int nx, ny, nz, step, l_src, l_max, active, l_merge, gen, ring0, pad1, pad2;   // ring0: this step's ring slot
-    long long coff;
-    float eps;
-    float sig_max;          // largest sigma_b / sigma_ref of the bins
-    int K[MAXL];
-    float sig[MAXB], sige[MAXB], eh[MAXB];
-};
+// The same for the only simulation (rays out are the warp's output count).
+__device__ __forceinline__ void flush_one(float &esc, float &out, unsigned &cnt, unsigned long long *sh_acc) {
+    float v[2] = {esc, out};
+    warp_sum<2>(v);
+    const unsigned seg = __reduce_add_sync(FULL, cnt & 0xffffu), rays = __reduce_add_sync(FULL, cnt >> 16);
+    if (lane_id() == 0) {
+        atomicAdd(sh_acc + 1, fixed32(v[0]));
+        atomicAdd(sh_acc + 2, fixed32(v[1]));
+        atomicAdd(sh_acc + 3, (unsigned long long)seg);
+        atomicAdd(sh_acc + 4, (unsigned long long)rays);
+    }
+    esc = out = 0.0f;
+    cnt = 0u;
+}
 
 // shared memory of a march block: tallies and constants per simulation, then
-// two tiles of ray records per warp
+// two tiles of ray records and the splitting lanes' rotation rows per warp
 __host__ __device__ constexpr size_t march_tiles_offset(int nsims) {
     return ((size_t)nsims * (NACC * sizeof(unsigned long long) + sizeof(MarchSim)) + 127) & ~(size_t)127;
 }
+constexpr int ROW_BYTES = 3 * 32 * 16;
 __host__ __device__ constexpr size_t march_shared_bytes(int nsims, uint32_t tile, int threads) {
-    return march_tiles_offset(nsims) + (size_t)(threads / 32) * 2 * tile;
+    return march_tiles_offset(nsims) + (size_t)(threads / 32) * (2 * tile + ROW_BYTES);
 }
 
 // (1 - e^-t)/t for 0 <= t < 1/8, from -t: its Taylor series through t^4 (the
@@ -173,8 +179,13 @@ __device__ __forceinline__ void seg_attenuate(float2 k, float dse, const float *
 // (Eq. 18-19).  A merging engine without Generalized members runs EXT = 1
 // (fewer registers: 10% less march time on the merging workloads than with
 // both), an engine that may run Generalized members EXT = 3.
-template <int NB, int AGG, int MINB, int EXT>
-__global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
+// ONE: an engine with one simulation whose steps are launched directly: its
+// constants come with the launch (A.one: the instructions take them from
+// constant memory, where a load of each from shared memory a ray and segment
+// was a fifth of the load-store unit's work, the march's busiest) and its
+// tallies need no simulation index.
+template <int NB, int AGG, int MINB, int EXT, bool ONE>
+__global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ MarchArgs A) {
     constexpr bool MRG = (EXT & 1) != 0, GEN = (EXT & 2) != 0;
     // per-simulation tallies of this block (photons in 2^-32 fixed point,
     // counts as integers), then the staged constants
@@ -200,7 +211,9 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
     const int lane = lane_id();
     const unsigned tile = A.q[0].tile;
     // this warp's two tiles and their barriers (one arrival each: lane 0's)
-    char *const tiles = reinterpret_cast<char *>(sh_acc) + march_tiles_offset(A.nsims) + (threadIdx.x >> 5) * 2 * tile;
+    char *const tiles = reinterpret_cast<char *>(sh_acc) + march_tiles_offset(A.nsims) +
+                        (threadIdx.x >> 5) * (2 * tile + ROW_BYTES);
+    int4 *const rowbuf = reinterpret_cast<int4 *>(tiles + 2 * tile);
     const unsigned tiles_s = smem_addr(tiles), bars_s = smem_addr(sh_bar[threadIdx.x >> 5]);
     if (lane == 0) {
         mbar_init(bars_s, 1);
@@ -211,13 +224,18 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
     Ctl *C = A.ctl;
     if (C->err == 0) {
         const int par = C->par;
+        const int step0 = ONE ? msim[0].step : 0;
         const char *const qin = A.q[par].base;
         char *const qout = A.q[par ^ 1].base;
-        unsigned long long *out_cnt = (unsigned long long *)&C->cnt[par ^ 1];
         // queue slots stay below 2^31 (the engine's bound), so 32-bit indices
         const unsigned n = (unsigned)(C->cnt[par] + C->emit_total);
-        const unsigned nr = (n + 31u) & ~31u;
-        const unsigned stride = gridDim.x * blockDim.x;
+        const unsigned ntile = (n + 31u) >> 5;
+        // the tile of this warp's iteration k: the warps take the tiles in turn.
+        // (Runs of 8 or 32 tiles a warp keep the shells of a source and step
+        // together, 2.7 of them in a tile instead of 8.2, and are 2 to 6%
+        // slower: more lanes of a reduction then hit one cell.)
+        const unsigned warps = gridDim.x * (blockDim.x >> 5), warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+        auto tile_at = [&](unsigned k) { return k * warps + warp; };
         // warp-private run of output slots [slab, slab + slab_left), and this
         // warp's outputs and iterations so far (its output rate)
         unsigned slab = 0;
@@ -227,27 +245,27 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
         // escaped and surviving photons, segments | rays in << 16, rays out
         float t_esc = 0.0f, t_out = 0.0f;
         unsigned t_cnt = 0u, t_rout = 0u;
-        int t_sim = -1, t_n = 0;
-        unsigned i = blockIdx.x * blockDim.x + threadIdx.x;       // i & 31 is the lane: a warp marches one tile
-        auto fetch = [&](unsigned j, unsigned b) {
-            bulk_load(tiles_s + b * tile, qin + (size_t)(j >> 5) * tile, tile, bars_s + 8 * b);
+        int t_sim = -1;
+        auto fetch = [&](unsigned k) {                  // iteration k's tile into buffer k & 1
+            const unsigned j = tile_at(k);
+            if (j < ntile) bulk_load(tiles_s + (k & 1u) * tile, qin + (size_t)j * tile, tile, bars_s + 8 * (k & 1u));
         };
         if (lane == 0) {
-            if (i < nr) fetch(i, 0);
-            if (i < nr && stride < nr - i) fetch(i + stride, 1);
+            fetch(0);
+            fetch(1);
         }
-        for (; i < nr; i += stride) {
+        for (unsigned tl; (tl = tile_at(w_it)) < ntile;) {
             // the tile's records, fetched two iterations ago (the copy hides
             // behind a whole iteration).  Words are read from shared memory
             // when they are needed, the unchanged ones again at the end: held
             // in registers they would spill (a dead slot's words are not used)
             const unsigned buf = w_it & 1;
-            const char *const rec = tiles + buf * tile;
+            char *const rec = tiles + buf * tile;
             if (!__all_sync(FULL, mbar_wait(bars_s + 8 * buf, (w_it >> 1) & 1))) {
                 // never in a working machine: report, let the other tile's copy end, stop
                 if (lane == 0) {
                     atomicOr(&C->err, 16);
-                    if (i + stride < nr) mbar_wait(bars_s + 8 * (buf ^ 1), ((w_it + 1) >> 1) & 1);
+                    if (tile_at(w_it + 1) < ntile) mbar_wait(bars_s + 8 * (buf ^ 1), ((w_it + 1) >> 1) & 1);
                 }
                 break;
             }
@@ -257,7 +275,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             const uint4 *const merged = reinterpret_cast<const uint4 *>(rec + 128 * (6 + NB));
             const float *const mthrs = reinterpret_cast<const float *>(rec + 128 * (6 + NB) + 512);
             bool valid = false, mrg = false;
-            int sim = 0, age = 0;
+            int sim = 0;
             // (1) integer walk of this step
             int key[4];
             float ds[4];
@@ -267,24 +285,25 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             const uint2 rt = tails[lane * TW];
             const uint32_t e = ra.x;
             const int bi = (int)ra.y, dx = (int)ra.z, dy = (int)ra.w, dz = (int)rt.x;
-            valid = i < n && rt.y != DEAD_RAY;
+            valid = 32u * tl + lane < n && rt.y != DEAD_RAY;
             mrg = MRG && valid && (e & MERGED_BIT);
             uint4 rm = make_uint4(0u, 0u, 0u, 0u);
             if (mrg) rm = merged[lane];
             int4 ec = make_int4(0, 0, 0, 0);
             if (mrg) {
-                sim = (int)((rm.w >> 16) & 0x7fffu);
+                if (!ONE) sim = (int)((rm.w >> 16) & 0x7fffu);
             } else if (valid) {
                 ec = __ldg(&A.em.cell[e]);
-                sim = ec.w;
+                if (!ONE) sim = ec.w;
             }
-            const MarchSim &S = msim[sim];
+            const MarchSim &S = ONE ? A.one : msim[sim];
+            const int step = ONE ? step0 : S.step;
             if (!S.active) valid = false;
             // age: cells travelled before this step.  A merged ray has moved
             // `since` steps from its merge position and had travelled its
             // constituents' mean distance when it was made.
-            const int since = S.step - bi - 1;
-            age = mrg ? (int)(rm.w & 0xffffu) + since : S.step - bi;
+            const int since = step - bi - 1;
+            const int age = mrg ? (int)(rm.w & 0xffffu) + since : step - bi;
             if (valid && (mrg ? since < 0 : (age < 0 || age >= A.em.ring_w))) {
                 atomicOr(&C->err, 2);
                 valid = false;
@@ -305,7 +324,8 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             // in order and skips the empty ones (negative keys)
             walk_step(valid, px, py, pz, dx, dy, dz, S.nx, S.ny, S.nz, (int)S.coff, key, ds, esc);
             }
-            const MarchSim &S = msim[sim];
+            const MarchSim &S = ONE ? A.one : msim[sim];
+            const int step = ONE ? step0 : S.step;
             int nseg = 4 + (key[0] >> 31) + (key[1] >> 31) + (key[2] >> 31) + (key[3] >> 31);
             // (2) opacities of the crossed cells (Generalized mode: also the
             // ionised fraction and the screen's share)
@@ -399,7 +419,10 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                     }
                     red_add_v4(A.cells.dep + last, s_end, g, h, 0.0f);
                 } else {
-                    while (lev + m < S.l_max && age + 1 >= S.K[lev + m]) ++m;
+                    const int age = mrg ? (int)(merged[lane].w & 0xffffu) + step - (int)heads[lane].y - 1
+                                        : step - (int)heads[lane].y;
+                    const int *const K = msim[sim].K;
+                    while (lev + m < S.l_max && age + 1 >= K[lev + m]) ++m;
                     nout = 1 << (2 * m);
                 }
             }
@@ -407,19 +430,20 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             // simulation for up to sixteen iterations, then the warp reduces them
             // into the block's fixed-point totals
             {
-                const bool clash = valid && t_sim >= 0 && t_sim != sim;
-                if (__any_sync(FULL, clash) || t_n == 16) {
-                    flush_tallies(t_esc, t_out, t_cnt, t_rout, t_sim, sh_acc);
-                    t_n = 0;
+                const bool clash = !ONE && valid && t_sim >= 0 && t_sim != sim;
+                if ((w_it & 15) == 15 || (!ONE && __any_sync(FULL, clash))) {
+                    if (ONE) flush_one(t_esc, t_out, t_cnt, sh_acc);
+                    else flush_tallies(t_esc, t_out, t_cnt, t_rout, t_sim, sh_acc);
                 }
                 if (valid) {
                     if (esc) t_esc += s_end;
                     if (nout) t_out += s_end;
                     t_cnt += (unsigned)nseg + (1u << 16);
-                    t_rout += (unsigned)nout;
-                    t_sim = sim;
+                    if (!ONE) {
+                        t_rout += (unsigned)nout;
+                        t_sim = sim;
+                    }
                 }
-                ++t_n;
             }
             // compacted output into the warp's run of slots: the remainder of
             // the current run first, then a new run reserved with one atomic
@@ -442,13 +466,13 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                     // rate (at most 16 iterations ahead and OUT_SLAB slots), so the
                     // unused tail stays small whatever the queue's dead fraction
                     const int need = tot - left;
-                    const unsigned iters_left = (nr - i + stride - 1u) / stride;
+                    const unsigned iters_left = (ntile - tl + warps - 1u) / warps;
                     const int ahead = iters_left < 16u ? (int)iters_left : 16;
                     const int rate = (w_out + tot + w_it) / (w_it + 1);
                     const int guess = rate * ahead < A.slab ? rate * ahead : A.slab;
                     const int want = need > guess ? need : guess;
                     unsigned long long nb64 = 0;
-                    if (lane == 0) nb64 = atomicAdd(out_cnt, (unsigned long long)want);
+                    if (lane == 0) nb64 = atomicAdd((unsigned long long *)&C->cnt[par ^ 1], (unsigned long long)want);
                     nb64 = __shfl_sync(FULL, nb64, 0);
                     const unsigned nbase = (unsigned)nb64;
                     if ((long long)(nb64 + want) > A.cap) {
@@ -497,56 +521,62 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                     const unsigned grp = __ballot_sync(FULL, ((split >> lane) & 1u) && m == mm);
                     split &= ~grp;
                     __syncwarp();
-                    if ((grp >> lane) & 1u) parent[__popc(grp & ((1u << lane) - 1u))] = (unsigned char)lane;
-                    __syncwarp();
                     // children keep their parent's sphere (Sec. 3.2): the
                     // emitter's of the birth step (whose slot of the ring the
                     // age gives: it is less than the ring's length), or the
-                    // merge cell's; each parent's lane gets the rows
-                    int4 prow[3];
-                    prow[0] = prow[1] = prow[2] = make_int4(0, 0, 0, 0);
+                    // merge cell's.  Each parent's lane gets the rows and
+                    // hands them over in shared memory, with its photons in
+                    // its record of the tile (nobody reads it afterwards)
                     if ((grp >> lane) & 1u) {
+                        parent[__popc(grp & ((1u << lane) - 1u))] = (unsigned char)lane;
                         const uint4 ra = heads[lane];
+                        int4 row[3];
                         if (mrg) {
                             const SimDev &SD = A.sims[sim];
-                            rotation_rows(SD.seed, (1LL << 31) + (long long)(ra.x & ~MERGED_BIT), (int)ra.y, SD.rotate, prow);
+                            rotation_rows(SD.seed, (1LL << 31) + (long long)(ra.x & ~MERGED_BIT), (int)ra.y, SD.rotate, row);
                         } else {
-                            int slot = S.ring0 - age;
+                            int slot = msim[sim].ring0 - (step - (int)ra.y);
                             if (slot < 0) slot += A.em.ring_w;
                             const int4 *rg = A.em.ring + ((long long)ra.x * A.em.ring_w + slot) * 3;
-                            prow[0] = rg[0]; prow[1] = rg[1]; prow[2] = rg[2];
+                            row[0] = rg[0]; row[1] = rg[1]; row[2] = rg[2];
                         }
+                        row[0].w = k0;
+                        row[1].w = sim;
+                        rowbuf[lane] = row[0];
+                        rowbuf[32 + lane] = row[1];
+                        rowbuf[64 + lane] = row[2];
+                        const float scale = pow2_neg(2 * mm);
+                        const uint2 rt = tails[lane * TW];
+                        uint32_t w[2 + NB];
+                        w[0] = rt.x; w[1] = rt.y;
+#pragma unroll
+                        for (int b = 0; b < NB; ++b) w[2 + b] = __float_as_uint(ph[b] * scale);
+                        store_tail<NB, false>(rec, lane, w);
                     }
-                    const float scale = pow2_neg(2 * mm);
+                    __syncwarp();
                     const unsigned all = (unsigned)__popc(grp) << (2 * mm);
-                    for (unsigned c0 = 0; c0 < all; c0 += 32) {
-                        const unsigned c = c0 + lane;
-                        const int src = parent[c < all ? c >> (2 * mm) : 0u];
+                    for (unsigned c = lane; c < all; c += 32) {
+                        const int src = parent[c >> (2 * mm)];
                         const unsigned sub = c & ((1u << (2 * mm)) - 1u);
                         const uint4 pa = heads[src];
-                        const uint32_t ppl = tails[src * TW].y;
-                        const int psim = __shfl_sync(FULL, sim, src), pk = __shfl_sync(FULL, k0, src);
                         uint32_t cw[2 + NB];
-#pragma unroll
-                        for (int b = 0; b < NB; ++b) cw[2 + b] = __float_as_uint(__shfl_sync(FULL, ph[b], src) * scale);
-                        int4 rows[3];
-#pragma unroll
-                        for (int r = 0; r < 3; ++r)
-                            rows[r] = make_int4(__shfl_sync(FULL, prow[r].x, src), __shfl_sync(FULL, prow[r].y, src),
-                                                __shfl_sync(FULL, prow[r].z, src), 0);
-                        if (c < all) {
+                        load_tail<NB, false>(rec, src, cw);
+                        const int4 rows[3] = {rowbuf[src], rowbuf[32 + src], rowbuf[64 + src]};
+                        const uint32_t ppl = cw[1];
+                        const int psim = rows[1].w;
+                        {
                             const int plev = (int)(ppl >> LEVEL_SHIFT), L = plev + mm;
                             const bool pmrg = MRG && (pa.x & MERGED_BIT);
                             uint4 pm = make_uint4(0u, 0u, 0u, 0u);
                             if (pmrg) pm = merged[src];
                             const uint32_t pix = pmrg && (pm.w >> 31)
-                                                     ? vertex_child(msim[psim].l_merge, ppl & PIX_MASK, plev, mm, sub)
+                                                     ? vertex_child(ONE ? A.one.l_merge : msim[psim].l_merge, ppl & PIX_MASK, plev, mm, sub)
                                                      : ((ppl & PIX_MASK) << (2 * mm)) + sub;
                             // (a level beyond the table: k_far fills the direction in)
                             int32_t cx = DIR_FAR, cy = 0, cz = 0;
                             if (L <= A.ltab) rotate_dir(rows, __ldg(&A.pixtab[level_offset(L) + pix]), cx, cy, cz);
                             else atomicOr(&C->far, 1);
-                            const unsigned o = slot_of(pk + (int)sub);
+                            const unsigned o = slot_of(rows[0].w + (int)sub);
                             cw[0] = (uint32_t)cz;
                             cw[1] = ((uint32_t)L << LEVEL_SHIFT) | pix;
                             char *const t = qout + (size_t)(o >> 5) * tile;
@@ -556,7 +586,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
                                 char *const tm = t + 128 * (6 + NB);
                                 pm.w &= 0x7fffffffu;
                                 reinterpret_cast<uint4 *>(tm)[o & 31u] = pm;
-                                reinterpret_cast<float *>(tm + 512)[o & 31u] = mthrs[src] * scale;
+                                reinterpret_cast<float *>(tm + 512)[o & 31u] = mthrs[src] * pow2_neg(2 * mm);
                             }
                         }
                     }
@@ -564,11 +594,16 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             }
             // every lane is done with the tile: fetch the one after next into it
             __syncwarp();
-            if (lane == 0 && 2u * stride < nr - i) fetch(i + 2u * stride, buf);
+            if (lane == 0) fetch(w_it + 2);
             ++w_it;
         }
         for (int k = lane; k < slab_left; k += 32) *pixel_word(A.q[par ^ 1], slab + k) = DEAD_RAY;
-        flush_tallies(t_esc, t_out, t_cnt, t_rout, t_sim, sh_acc);
+        if (ONE) {
+            flush_one(t_esc, t_out, t_cnt, sh_acc);
+            if (lane == 0 && w_out) atomicAdd(sh_acc + 5, (unsigned long long)w_out);    // rays out
+        } else {
+            flush_tallies(t_esc, t_out, t_cnt, t_rout, t_sim, sh_acc);
+        }
     }
     __syncthreads();
     for (int i = threadIdx.x; i < A.nsims * NACC; i += blockDim.x) {
@@ -587,6 +622,43 @@ __global__ void __launch_bounds__(256, MINB) k_march(MarchArgs A) {
             }
             atomicAdd(dst, v);
         }
+    }
+}
+
+// Kernel variants: every bin count with two and three blocks per SM (three:
+// a quarter less time than two at six bins; four spill at every bin count and
+// lose to three: 161 against 147 ms of march on the 128^3 workload); the bin
+// counts of the standard spectra (1, 3, 4) also with four, and with every
+// aggregation, for the autotuner.
+template <int NB, int EXT, bool ONE>
+MarchFn march_pick_nb(int agg, int minb) {
+    if (agg == 0 && minb == 2) return k_march<NB, 0, 2, EXT, ONE>;
+    if (agg == 0 && minb == 3) return k_march<NB, 0, 3, EXT, ONE>;
+    if constexpr (NB == 1 || NB == 3 || NB == 4) {
+        if (agg == 0 && minb == 4) return k_march<NB, 0, 4, EXT, ONE>;
+        if constexpr (!ONE) {
+            if (agg == 1 && minb == 2) return k_march<NB, 1, 2, EXT, false>;
+            if (agg == 1 && minb == 3) return k_march<NB, 1, 3, EXT, false>;
+            if (agg == 1 && minb == 4) return k_march<NB, 1, 4, EXT, false>;
+            if (agg == 2 && minb == 2) return k_march<NB, 2, 2, EXT, false>;
+            if (agg == 2 && minb == 3) return k_march<NB, 2, 3, EXT, false>;
+            if (agg == 2 && minb == 4) return k_march<NB, 2, 4, EXT, false>;
+        }
+    }
+    return nullptr;
+}
+template <int EXT, bool ONE>
+MarchFn march_pick(int nb, int agg, int minb) {
+    switch (nb) {
+        case 1: return march_pick_nb<1, EXT, ONE>(agg, minb);
+        case 2: return march_pick_nb<2, EXT, ONE>(agg, minb);
+        case 3: return march_pick_nb<3, EXT, ONE>(agg, minb);
+        case 4: return march_pick_nb<4, EXT, ONE>(agg, minb);
+        case 5: return march_pick_nb<5, EXT, ONE>(agg, minb);
+        case 6: return march_pick_nb<6, EXT, ONE>(agg, minb);
+        case 7: return march_pick_nb<7, EXT, ONE>(agg, minb);
+        case 8: return march_pick_nb<8, EXT, ONE>(agg, minb);
+        default: return nullptr;
     }
 }
 

@@ -47,37 +47,7 @@ namespace frt {
 // ---------------------------------------------------------------------------
 // march variants with merged rays (engines without Generalized members)
 // ---------------------------------------------------------------------------
-MarchFn march_fn_merge(int nb, int agg, int minb) {
-#define FRT_V(NB)                                                                   \
-    if (nb == NB) {                                                                \
-        if (agg == 0 && minb == 2) return k_march<NB, 0, 2, 1>;                    \
-        if (agg == 0 && minb == 3) return k_march<NB, 0, 3, 1>;                    \
-        if (agg == 0 && minb == 4) return k_march<NB, 0, 4, 1>;                    \
-        if (agg == 1 && minb == 2) return k_march<NB, 1, 2, 1>;                    \
-        if (agg == 1 && minb == 3) return k_march<NB, 1, 3, 1>;                    \
-        if (agg == 1 && minb == 4) return k_march<NB, 1, 4, 1>;                    \
-        if (agg == 2 && minb == 2) return k_march<NB, 2, 2, 1>;                    \
-        if (agg == 2 && minb == 3) return k_march<NB, 2, 3, 1>;                    \
-        if (agg == 2 && minb == 4) return k_march<NB, 2, 4, 1>;                    \
-        return nullptr;                                                            \
-    }
-    FRT_V(1)
-    FRT_V(3)
-    FRT_V(4)
-#undef FRT_V
-#define FRT_W(NB)                                                                   \
-    if (nb == NB && agg == 0) {                                                    \
-        if (minb == 2) return k_march<NB, 0, 2, 1>;                                \
-        if (minb == 3) return k_march<NB, 0, 3, 1>;                                \
-    }
-    FRT_W(2)
-    FRT_W(5)
-    FRT_W(6)
-    FRT_W(7)
-    FRT_W(8)
-#undef FRT_W
-    return nullptr;
-}
+MarchFn march_fn_merge(int nb, int agg, int minb) { return march_pick<1, false>(nb, agg, minb); }
 
 namespace {
 
