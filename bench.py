@@ -407,8 +407,9 @@ def impl_gpu(args, dist):
         batch = run_batch(args)
         serve_line = run_serve(args)
 
-    launches_per_sim = 1 + prob.nsteps * (3 + (1 if len(prob.source_ndot) else 0)
-                                          + 3 * (prob.options.gamma_iters - 1))
+    # reset and the cells' initialisation, then emission, march and chemistry
+    # a step (march and chemistry once more for each further pass)
+    launches_per_sim = 2 + prob.nsteps * (3 + 2 * (prob.options.gamma_iters - 1))
     if dist.rank == 0:
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": dist.ws, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": t_max / args.steps, "higher_is_better": True,
@@ -674,12 +675,12 @@ def impl_merge(args, dist):
                 "config": {"workload": "merge: " + WORKLOAD_DESC + "; ray merging as Sec. 7.1",
                            "cases": [c[0] for c in cases], "timed_case": best},
                 "results": results, "clocks": clk,
-                # per simulation: the cells' initialisation, then per RT step emission,
-                # march, chemistry and the budget's commit plus the merge's eleven
-                # launches (rotations, content histogram, two radix-select passes of
+                # per simulation: reset and the cells' initialisation, then per RT step
+                # emission, march, directions beyond the pixel table and chemistry plus
+                # the merge's eleven launches (rotations, content histogram, two radix-select passes of
                 # copy reduction and search, lower-bits histogram, group, weight,
                 # placement scan, emit)
-                "gpu_launches": args.steps * (1 + base.nsteps * (4 + 11))}
+                "gpu_launches": args.steps * (2 + base.nsteps * (4 + 11))}
         print(json.dumps(line), flush=True)
 
 

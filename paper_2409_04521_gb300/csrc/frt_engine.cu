@@ -178,12 +178,11 @@ Engine::~Engine() {
     // every device allocation of the engine, whether or not init completed
     for (auto &kv : alloc_sizes_) cudaFree(kv.first);
     alloc_sizes_.clear();
-    if (h_err_) cudaFreeHost(h_err_);
+    if (h_status_) cudaFreeHost(h_status_);
     if (h_stage_) cudaFreeHost(h_stage_);
     if (h_nh_) cudaFreeHost(h_nh_);
     if (h_fields_) cudaFreeHost(h_fields_);
     if (ev_nh_) cudaEventDestroy(ev_nh_);
-    if (ev_err_) cudaEventDestroy(ev_err_);
     if (ev_stage_) cudaEventDestroy(ev_stage_);
     for (auto e : ev_pool_) cudaEventDestroy(e);
     for (auto &v : ev_k_)
@@ -291,7 +290,8 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
         CK(cudaEventCreateWithFlags(&mside_.fork, cudaEventDisableTiming));
         CK(cudaEventCreateWithFlags(&mside_.join, cudaEventDisableTiming));
     }
-    if (cudaMallocHost(&h_err_, 64) != cudaSuccess) return fail(FLEXRT_E_OOM, "pinned allocation failed");
+    if (cudaMallocHost(&h_status_, 64) != cudaSuccess) return fail(FLEXRT_E_OOM, "pinned allocation failed");
+    std::memset(h_status_, 0, 64);
     if (ms > 1) {
         // members are admitted while others step: their densities go up
         // through pinned staging, so that admission does not wait for the GPU
@@ -301,7 +301,6 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
     }
     if (cudaMallocHost(&h_stage_, (size_t)(ms + 1) * 6 * sizeof(double)) != cudaSuccess)
         return fail(FLEXRT_E_OOM, "pinned allocation failed");
-    CK(cudaEventCreateWithFlags(&ev_err_, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_stage_, cudaEventDisableTiming));
     cell_alloc_.reset(nc);
     em_cap_ = 0;
@@ -361,7 +360,7 @@ flexrt_status Engine::grow_emitters(int need) {
     em_ = ne;
     em_cap_ = cap;
     emit_blocks_ = std::max(1, std::min((em_cap_ + 127) / 128, 1024));
-    graph_dirty_ = true;
+    graph_stale();
     return FLEXRT_OK;
 }
 
@@ -521,9 +520,10 @@ flexrt_status Engine::add_sim(const SimDev &proto, const double *n_H, int *slot_
         while (L < proto.l_max && (proto.merge || proto.K[L] <= em_.ring_w)) ++L;
         if (L > ltab_ && !far_possible_) {
             far_possible_ = true;
-            graph_dirty_ = true;
+            graph_stale();
         }
     }
+    if (one_sim()) graph_stale();                // its constants are launch arguments
     Slot &sl = slots_[s];
     sl = Slot();
     sl.used = true;
@@ -695,19 +695,17 @@ flexrt_status Engine::set_dt(int s, double dt) {
     return FLEXRT_OK;
 }
 
-flexrt_status Engine::poll(bool wait) {
+// the outcome of the last step the GPU has ended, if it is a new one (the
+// GPU writes the four words as one 16-byte store; after a stream
+// synchronisation this is the last step enqueued)
+flexrt_status Engine::poll() {
     if (latched_ != FLEXRT_OK) return latched_;
-    if (!err_pending_) return FLEXRT_OK;
-    if (wait) {
-        cudaError_t e = cudaEventSynchronize(ev_err_);
-        if (e != cudaSuccess) return cuda(e, "step");
-    } else if (cudaEventQuery(ev_err_) != cudaSuccess) {
-        return FLEXRT_OK;
-    }
-    err_pending_ = false;
-    static_assert(offsetof(Ctl, par) == 16 && offsetof(Ctl, err) == 20, "ctl layout");
-    const int32_t v = h_err_[5];
-    q_used_ = reinterpret_cast<const long long *>(h_err_)[h_err_[4] & 1];
+    const uint32_t seq = __atomic_load_n(h_status_ + 3, __ATOMIC_ACQUIRE);
+    if (seq == seq_seen_) return FLEXRT_OK;
+    seq_seen_ = seq;
+    const uint32_t v = __atomic_load_n(h_status_ + 2, __ATOMIC_RELAXED);
+    q_used_ = (long long)__atomic_load_n(h_status_, __ATOMIC_RELAXED) |
+              (long long)__atomic_load_n(h_status_ + 1, __ATOMIC_RELAXED) << 32;
     if (v) {
         latched_ = FLEXRT_E_CAPACITY;
         if (v & 1) err_ = "ray queue capacity exceeded; state kept at the last complete step";
@@ -751,8 +749,8 @@ flexrt_status Engine::launch_stage(int stage) {
             if (b < h.nb) o.sig_max = std::max(o.sig_max, h.sig[b]);
         }
     }
-    ChemArgs ca{ctl_, sims_, acc_, ms, cells_, rg_, 1};
-    const bool prof = profiling_ && !cfg_.use_graph;
+    ChemArgs ca{ctl_, sims_, acc_, ms, cells_, rg_, 1, reinterpret_cast<uint4 *>(h_status_)};
+    const bool prof = profiling_ && !cfg_.use_graph;      // (a profiled single simulation is never replayed)
     cudaEvent_t e0 = nullptr;
     auto tic = [&]() {
         if (prof) { e0 = take_event(ev_pool_); cudaEventRecord(e0, st_); }
@@ -779,7 +777,6 @@ flexrt_status Engine::launch_stage(int stage) {
             tic();
             CK(launch_chem(ct, chem_blocks_, st_));
             toc(2);
-            CK(launch_iter_reset(ctl_, acc_, ms, st_));
     }
         tic();
         CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, st_, ext_variants()));
@@ -796,7 +793,6 @@ flexrt_status Engine::launch_stage(int stage) {
     tic();
     CK(launch_chem(ca, chem_blocks_, st_));
     toc(2);
-    CK(launch_end(ctl_, sims_, acc_, ms, st_));
     return FLEXRT_OK;
 }
 
@@ -809,35 +805,47 @@ void Engine::free_retired() {
     }
 }
 
+bool Engine::graph_now() {
+    if (cfg_.use_graph) return true;
+    if (!one_sim() || profiling_ || graph_off_) return false;
+    if (graph_dirty_ && direct_steps_ < GRAPH_AFTER) { ++direct_steps_; return false; }
+    // a caller that captures the stream itself gets the kernels
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    return cudaStreamIsCapturing(st_, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+}
+
+flexrt_status Engine::run_graph() {
+    if (graph_dirty_) {
+        CK(cudaStreamSynchronize(st_));
+        if (graph_) { cudaGraphExecDestroy(graph_); graph_ = nullptr; }
+        cudaGraph_t g = nullptr;
+        cudaError_t e = cudaStreamBeginCapture(st_, cudaStreamCaptureModeThreadLocal);
+        if (e != cudaSuccess && !cfg_.use_graph) {
+            cudaGetLastError();                  // a stream that cannot be captured: direct launches
+            graph_off_ = true;
+            return launch_step();
+        }
+        CK(e);
+        flexrt_status r = launch_step();
+        e = cudaStreamEndCapture(st_, &g);
+        if (r != FLEXRT_OK) { if (g) cudaGraphDestroy(g); return r; }
+        if (e != cudaSuccess) return cuda(e, "graph capture");
+        e = cudaGraphInstantiate(&graph_, g, 0);
+        cudaGraphDestroy(g);
+        if (e != cudaSuccess) return cuda(e, "graph instantiate");
+        graph_dirty_ = false;
+    }
+    CK(cudaGraphLaunch(graph_, st_));
+    return FLEXRT_OK;
+}
+
 flexrt_status Engine::step() {
     if (mid_step_) return fail(FLEXRT_E_STATE, "finish the staged step first");
-    flexrt_status s = poll(false);
+    flexrt_status s = poll();
     if (s != FLEXRT_OK) return s;
     free_retired();
-    if (cfg_.use_graph) {
-        if (graph_dirty_) {
-            if (graph_) { cudaGraphExecDestroy(graph_); graph_ = nullptr; }
-            CK(cudaStreamSynchronize(st_));
-            cudaGraph_t g = nullptr;
-            CK(cudaStreamBeginCapture(st_, cudaStreamCaptureModeThreadLocal));
-            flexrt_status r = launch_step();
-            cudaError_t ee = cudaStreamEndCapture(st_, &g);
-            if (r != FLEXRT_OK) { if (g) cudaGraphDestroy(g); return r; }
-            if (ee != cudaSuccess) return cuda(ee, "graph capture");
-            ee = cudaGraphInstantiate(&graph_, g, 0);
-            cudaGraphDestroy(g);
-            if (ee != cudaSuccess) return cuda(ee, "graph instantiate");
-            graph_dirty_ = false;
-        }
-        CK(cudaGraphLaunch(graph_, st_));
-    } else {
-        flexrt_status r = launch_step();
-        if (r != FLEXRT_OK) return r;
-    }
-    // queue counts, parity and error word of the step, read when it completes
-    CK(cudaMemcpyAsync(h_err_, ctl_, offsetof(Ctl, err) + sizeof(int32_t), cudaMemcpyDeviceToHost, st_));
-    CK(cudaEventRecord(ev_err_, st_));
-    err_pending_ = true;
+    s = graph_now() ? run_graph() : launch_step();
+    if (s != FLEXRT_OK) return s;
     ++steps_taken_;
     for (auto &sl : slots_)
         if (sl.active) ++sl.h.step;
@@ -851,7 +859,7 @@ flexrt_status Engine::step_stage(int stage) {
     if (cfg_.use_graph || slots_.size() != 1) return fail(FLEXRT_E_STATE, "staged steps are for single simulations");
     if (stage == 1) {
         if (mid_step_) return fail(FLEXRT_E_STATE, "a staged step is already open");
-        flexrt_status s = poll(false);
+        flexrt_status s = poll();
         if (s != FLEXRT_OK) return s;
         s = launch_stage(1);
         if (s != FLEXRT_OK) return s;
@@ -862,10 +870,6 @@ flexrt_status Engine::step_stage(int stage) {
     mid_step_ = false;
     flexrt_status s = launch_stage(2);
     if (s != FLEXRT_OK) return s;
-    // queue counts, parity and error word of the step, read when it completes
-    CK(cudaMemcpyAsync(h_err_, ctl_, offsetof(Ctl, err) + sizeof(int32_t), cudaMemcpyDeviceToHost, st_));
-    CK(cudaEventRecord(ev_err_, st_));
-    err_pending_ = true;
     ++steps_taken_;
     for (auto &sl : slots_)
         if (sl.active) ++sl.h.step;
@@ -874,12 +878,13 @@ flexrt_status Engine::step_stage(int stage) {
 
 flexrt_status Engine::sync() {
     CK(cudaStreamSynchronize(st_));
-    return poll(true);
+    return poll();
 }
 
 flexrt_status Engine::retire(int s) {
     if (s < 0 || s >= (int)slots_.size() || !slots_[s].active) return fail(FLEXRT_E_INVALID, "bad slot");
     Slot &sl = slots_[s];
+    if (one_sim()) graph_stale();
     sl.active = false;
     sl.h.active = 0;
     const int32_t zero = 0;
@@ -893,28 +898,23 @@ flexrt_status Engine::retire(int s) {
 
 flexrt_status Engine::reset_all() {
     CK(cudaStreamSynchronize(st_));
+    const bool failed = latched_ != FLEXRT_OK || h_status_[2] != 0 || mid_step_;
     latched_ = FLEXRT_OK;
-    err_pending_ = false;
-    int32_t derr = 0;
-    CK(cudaMemcpy(&derr, &ctl_->err, sizeof(derr), cudaMemcpyDeviceToHost));
-    if (derr && mwmem_) {
+    seq_seen_ = h_status_[3];                    // what ended before is not reported any more
+    if (failed && mwmem_) {
         // a step that failed may have stopped inside the merge, with groups
         // not cleared: clear the whole merge scratch
         auto it = alloc_sizes_.find(mwmem_);
-        if (it != alloc_sizes_.end()) CK(cudaMemset(mwmem_, 0, it->second));
+        if (it != alloc_sizes_.end()) CK(cudaMemsetAsync(mwmem_, 0, it->second, st_));
     }
-    CK(cudaMemset(ctl_, 0, offsetof(Ctl, emit_total)));   // counts, parity, error
+    // the rest in stream order, ahead of the steps that follow
+    CK(launch_reset(ctl_, sims_, acc_, (int)slots_.size(), st_));
     for (int s = 0; s < (int)slots_.size(); ++s) {
         Slot &sl = slots_[s];
         if (!sl.active) continue;
         sl.h.step = 0;
-        const int32_t zero = 0;
-        CK(cudaMemcpy((char *)(sims_ + s) + offsetof(SimDev, step), &zero, sizeof(zero), cudaMemcpyHostToDevice));
-        // keep the monotonic marched-ray counter (last field) for profiling windows
-        CK(cudaMemset(acc_ + s, 0, offsetof(SimAcc, rays_in_total)));
         CK(launch_init_cells(sims_, s, cells_, sl.h.ncell, st_));
     }
-    CK(cudaStreamSynchronize(st_));
     return FLEXRT_OK;
 }
 
@@ -964,7 +964,7 @@ flexrt_status Engine::fields(int s, flexrt_fields *f) {
     if (f->T) CK(cudaMemcpyAsync(hT, cells_.T + c0, n * sizeof(float), cudaMemcpyDeviceToHost, st_));
     if (f->gamma_HI) CK(cudaMemcpyAsync(hg, cells_.gamma + c0, n * sizeof(float), cudaMemcpyDeviceToHost, st_));
     CK(cudaStreamSynchronize(st_));
-    poll(true);                                   // latch a failed step's error (the state is kept)
+    poll();                                   // latch a failed step's error (the state is kept)
     host_parallel(n, [&](size_t i0, size_t i1) {
         if (f->n_HI)
             for (size_t i = i0; i < i1; ++i) f->n_HI[i] = hn[i] * hy[i];
@@ -1103,7 +1103,7 @@ flexrt_status Engine::ionized_volume(int s, double *x_ion) {
     const Slot *sl = slot(s);
     if (!sl || !x_ion) return fail(FLEXRT_E_INVALID, "bad slot or buffer");
     CK(cudaStreamSynchronize(st_));
-    poll(true);
+    poll();
     std::vector<double> v((size_t)sl->h.ncell);
     CK(cudaMemcpy(v.data(), cells_.xion + sl->cell0, v.size() * sizeof(double), cudaMemcpyDeviceToHost));
     for (size_t i = 0; i < v.size(); ++i) x_ion[i] = sl->h.gen_mode ? (double)v[i] : 0.0;
@@ -1125,7 +1125,7 @@ flexrt_status Engine::set_launch(int agg, int minb, int blocks_per_sm, int threa
     march_threads_ = threads;
     march_slab_ = slab;
     march_blocks_ = sm_count_ * bps;
-    graph_dirty_ = true;
+    graph_stale();
     return FLEXRT_OK;
 }
 
@@ -1170,7 +1170,7 @@ int Engine::free_slots() const {
 flexrt_status Engine::queue_used(long long *n) {
     // the count after the last step seen complete (without waiting for the
     // GPU); exact after sync()
-    flexrt_status r = poll(false);
+    flexrt_status r = poll();
     *n = q_used_;
     return r;
 }
@@ -1204,7 +1204,7 @@ flexrt_status Engine::save_state(int s, void *buf, int64_t cap, int64_t *bytes) 
     if (!sl || !bytes || slots_.size() != 1) return fail(FLEXRT_E_INVALID, "checkpoints are for single simulations");
     if (mid_step_) return fail(FLEXRT_E_STATE, "finish the staged step first");
     CK(cudaStreamSynchronize(st_));
-    flexrt_status ps = poll(true);
+    flexrt_status ps = poll();
     if (ps != FLEXRT_OK) return ps;
     Ctl hc;
     CK(cudaMemcpy(&hc, ctl_, sizeof(hc), cudaMemcpyDeviceToHost));
@@ -1292,7 +1292,7 @@ flexrt_status Engine::load_state(int s, const void *buf, int64_t bytes) {
     sl->h.step = (int32_t)h.step;
     CK(cudaMemcpy((char *)(sims_ + s) + offsetof(SimDev, step), &sl->h.step, sizeof(int32_t), cudaMemcpyHostToDevice));
     latched_ = FLEXRT_OK;
-    err_pending_ = false;
+    seq_seen_ = h_status_[3];
     if (h.dt > 0.0) {
         flexrt_status r = set_dt(s, h.dt);
         if (r != FLEXRT_OK) return r;

@@ -134,7 +134,7 @@ class Engine {
     void dev_free(void *p);
     flexrt_status grow_emitters(int need);
     flexrt_status upload_lists();             // active emitters, cell ranges, counters
-    flexrt_status poll(bool wait);
+    flexrt_status poll();
     flexrt_status launch_step();
     flexrt_status launch_stage(int stage);
     flexrt_status read_acc(int slot, SimAcc &a);
@@ -169,16 +169,18 @@ class Engine {
     int march_agg_ = 0, march_minb_ = 3, march_blocks_ = 1, march_threads_ = 256, march_slab_ = OUT_SLAB;
     int chem_blocks_ = 1, emit_blocks_ = 1, sm_count_ = 1;
 
-    int32_t *h_err_ = nullptr;     // the last step's queue counts, parity and error word
+    // the last ended step's outcome, written by the GPU (ChemArgs::status),
+    // and the number of the last one seen
+    uint32_t *h_status_ = nullptr;
+    uint32_t seq_seen_ = 0;
     double *h_stage_ = nullptr;
     double *h_nh_ = nullptr;       // pinned staging of a member's n_H (engines of several members)
     void *h_fields_ = nullptr;     // pinned staging of the fields read-back, grown on demand
     size_t h_fields_bytes_ = 0;
     cudaEvent_t ev_nh_ = nullptr;  // its upload has been consumed
     long long q_used_ = 0;         // live rays after the last step the host has seen complete
-    cudaEvent_t ev_err_ = nullptr, ev_stage_ = nullptr;
+    cudaEvent_t ev_stage_ = nullptr;
     MergeSide mside_{nullptr, nullptr, nullptr};   // merging engines: the rotation pass's stream
-    bool err_pending_ = false;
 
     bool profiling_ = false;
     std::vector<cudaEvent_t> ev_pool_;
@@ -187,6 +189,15 @@ class Engine {
 
     cudaGraphExec_t graph_ = nullptr;
     bool graph_dirty_ = true;
+    bool graph_off_ = false;                // the stream cannot be captured
+    int direct_steps_ = 0;                  // steps launched directly since the graph became stale
+    // a step replayed from a graph: batches that ask for it, and single
+    // simulations once they have taken GRAPH_AFTER steps directly (capturing
+    // and instantiating it costs about as much host time as that many)
+    static constexpr int GRAPH_AFTER = 8;
+    void graph_stale() { graph_dirty_ = true; direct_steps_ = 0; }
+    bool graph_now();
+    flexrt_status run_graph();
     bool mid_step_ = false;                 // between the two stages of a staged step
 
     std::unordered_map<void *, size_t> alloc_sizes_;   // live device allocations

@@ -8,8 +8,8 @@
 //              Eq. 2-3 split and the compacted write of survivors and children;
 //   k_chem   : per cell, Gamma from the deposits, the ionisation update of
 //              Sec. 4.1 Eq. 7-10 (double precision), the temperature update
-//              of Eq. 12 (single precision) and kappa for the next step;
-//   k_end    : per simulation, commit of the step's photon budget.
+//              of Eq. 12 (single precision), kappa for the next step,
+//              and the commit of the step's photon budget by its last block.
 // All launches are sized on the host from capacities only; counts are read
 // from device memory, so the same launches can be replayed in a CUDA graph.
 #include <algorithm>
@@ -149,6 +149,23 @@ __global__ void k_init_cells(const SimDev *sims, int sim, Cells c) {
         const float nHf = (float)c.nH[g];
         c.nHf[g] = nHf;
         c.kap[g] = S.gen_mode ? gen_kappa(S, nHf, 0.0f, 0.0f) : cell_kappa(S, nHf, (float)y, y <= S.y_thr, 0.0f);
+    }
+}
+
+// the start of a run: no rays, no error, step 0, an empty photon budget (the
+// marched-ray counter is kept: profiling windows difference it)
+__global__ void k_reset(Ctl *C, SimDev *sims, SimAcc *acc, int nsims) {
+    for (int j = threadIdx.x; j < nsims; j += blockDim.x) {
+        if (!sims[j].active) continue;
+        const double marched = acc[j].rays_in_total;
+        acc[j] = SimAcc{};
+        acc[j].rays_in_total = marched;
+        sims[j].step = 0;
+    }
+    if (threadIdx.x == 0) {
+        C->cnt[0] = C->cnt[1] = 0;
+        C->par = 0;
+        C->err = 0;
     }
 }
 
@@ -316,7 +333,69 @@ __global__ void k_queue_words(Queue q, int merged, long long n, uint32_t *words,
 // ---------------------------------------------------------------------------
 // chemistry
 // ---------------------------------------------------------------------------
+// The last block of a pass ends it (kernels of their own for this were a fifth
+// of a small simulation's step: one more launch a step, and one a trial pass).
+// A trial pass of the Gamma - <n_HI> iteration: the next pass marches the same
+// rays again, so the march's output and the step's tallies are dropped
+// (emission happens once per step; the marched-ray counter keeps every pass).
+// A step: its photon budget is committed, the queues change places, and the
+// step's outcome goes to host memory.
+__device__ void end_pass(const ChemArgs &A) {
+    Ctl *C = A.ctl;
+    const bool err = C->err != 0;
+    if (!A.final_pass && err) return;
+    for (int j = threadIdx.x; j < A.nsims; j += blockDim.x) {
+        SimAcc &a = A.acc[j];
+        // (written by other blocks' and kernels' atomics: read past the L1)
+        const double emit = __ldcg(&a.p_emit), absd = __ldcg(&a.p_abs), esc = __ldcg(&a.p_esc), out = __ldcg(&a.p_out);
+        const double seg = __ldcg(&a.p_seg), rin = __ldcg(&a.p_rays_in), rout = __ldcg(&a.p_rays_out);
+        if (A.final_pass) {
+            if (!err && A.sims[j].active) {
+                a.emitted += emit;
+                a.absorbed += absd;
+                a.escaped += esc;
+                a.in_flight = out;
+                a.seg_last = seg;
+                a.seg_total += seg;
+                a.rays_live = rout;
+                a.rays_in_last = rin;
+                a.rays_in_total += rin;
+                a.lost += __ldcg(&a.p_lost);
+                A.sims[j].step += 1;
+            }
+            a.p_emit = 0.0;
+        } else {
+            a.rays_in_total += rin;
+        }
+        a.p_abs = a.p_esc = a.p_out = a.p_in = 0.0;
+        a.p_seg = a.p_rays_in = a.p_rays_out = a.p_lost = 0.0;
+    }
+    if (threadIdx.x != 0) return;
+    const int par = C->par;
+    C->far = 0;
+    if (!A.final_pass) {
+        C->cnt[par ^ 1] = 0;
+        return;
+    }
+    // the march wrote the live rays to the other queue (a merge step left
+    // holes there, which the next march skips)
+    long long live;
+    if (err) {
+        C->cnt[par ^ 1] = 0;
+        live = C->cnt[par];
+    } else {
+        live = C->cnt[par ^ 1];
+        C->cnt[par] = 0;
+        C->par = par ^ 1;
+    }
+    C->merged = 0;
+    const uint32_t seq = C->seq + 1;
+    C->seq = seq;
+    *A.status = make_uint4((uint32_t)live, (uint32_t)(live >> 32), (uint32_t)C->err, seq);
+}
+
 __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
+    __shared__ int s_last;
     // per-simulation absorbed totals and screens' excess photons, then the
     // active cell ranges
     extern __shared__ double sh_abs[];
@@ -328,7 +407,7 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
     // code photons
     float *s_apn = reinterpret_cast<float *>(s_sim + A.nsims);
     int *s_gen = reinterpret_cast<int *>(s_apn + A.nsims);
-    const Ctl *C = A.ctl;
+    Ctl *C = A.ctl;
     const int nrng = C->n_ranges;
     for (int i = threadIdx.x; i < A.nsims; i += blockDim.x) {
         sh_abs[i] = 0.0;
@@ -521,60 +600,16 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
         if (sh_abs[i] != 0.0) atomicAdd(&A.acc[i].p_abs, sh_abs[i]);
         if (sh_lost[i] != 0.0) atomicAdd(&A.acc[i].p_lost, sh_lost[i]);
     }
-}
-
-// ---------------------------------------------------------------------------
-// end of step
-// ---------------------------------------------------------------------------
-__global__ void k_end(Ctl *C, SimDev *sims, SimAcc *acc, int nsims) {
-    const bool err = C->err != 0;
-    for (int j = threadIdx.x; j < nsims; j += blockDim.x) {
-        SimAcc &a = acc[j];
-        if (!err && sims[j].active) {
-            a.emitted += a.p_emit;
-            a.absorbed += a.p_abs;
-            a.escaped += a.p_esc;
-            a.in_flight = a.p_out;
-            a.seg_last = a.p_seg;
-            a.seg_total += a.p_seg;
-            a.rays_live = a.p_rays_out;
-            a.rays_in_last = a.p_rays_in;
-            a.rays_in_total += a.p_rays_in;
-            a.lost += a.p_lost;
-            sims[j].step += 1;
-        }
-        a.p_emit = a.p_abs = a.p_esc = a.p_out = a.p_in = 0.0;
-        a.p_seg = a.p_rays_in = a.p_rays_out = a.p_lost = 0.0;
-    }
     __syncthreads();
     if (threadIdx.x == 0) {
-        // the march wrote the live rays to the other queue (a merge step
-        // left holes there, which the next march skips)
-        const int par = C->par;
-        if (err) C->cnt[par ^ 1] = 0;
-        else {
-            C->cnt[par] = 0;
-            C->par = par ^ 1;
-        }
-        C->merged = 0;
-        C->far = 0;
+        __threadfence();
+        s_last = atomicAdd(&C->ticket, 1u) == gridDim.x - 1u;
     }
-}
-
-// between passes of the Gamma - <n_HI> iteration: the next pass marches the
-// same rays again, so the march's output and the step's tallies are dropped
-// (emission happens once per step; the marched-ray counter keeps every pass)
-__global__ void k_iter_reset(Ctl *C, SimAcc *acc, int nsims) {
-    if (C->err) return;
-    for (int j = threadIdx.x; j < nsims; j += blockDim.x) {
-        SimAcc &a = acc[j];
-        a.rays_in_total += a.p_rays_in;
-        a.p_abs = a.p_esc = a.p_out = a.p_in = 0.0;
-        a.p_seg = a.p_rays_in = a.p_rays_out = a.p_lost = 0.0;
-    }
-    if (threadIdx.x == 0) {
-        C->cnt[C->par ^ 1] = 0;
-        C->far = 0;
+    __syncthreads();
+    if (s_last) {
+        __threadfence();
+        if (threadIdx.x == 0) C->ticket = 0u;
+        end_pass(A);
     }
 }
 
@@ -656,6 +691,10 @@ cudaError_t launch_init_cells(const SimDev *sims, int sim, Cells c, long long nc
     k_init_cells<<<blocks, 256, 0, st>>>(sims, sim, c);
     return cudaGetLastError();
 }
+cudaError_t launch_reset(Ctl *c, SimDev *sims, SimAcc *acc, int nsims, cudaStream_t st) {
+    k_reset<<<1, 256, 0, st>>>(c, sims, acc, nsims);
+    return cudaGetLastError();
+}
 cudaError_t launch_emit(const EmitArgs &a, int blocks, cudaStream_t st) {
     k_emit<<<blocks, 128, 0, st>>>(a);
     return cudaGetLastError();
@@ -715,14 +754,6 @@ cudaError_t launch_chem(const ChemArgs &a, int blocks, cudaStream_t st) {
     const size_t sh = (size_t)a.nsims * 2 * sizeof(double) + (size_t)(2 * a.nsims + 1) * sizeof(long long) +
                       (size_t)a.nsims * (2 * sizeof(int) + sizeof(float));
     k_chem<<<blocks, 256, sh, st>>>(a);
-    return cudaGetLastError();
-}
-cudaError_t launch_iter_reset(Ctl *c, SimAcc *acc, int nsims, cudaStream_t st) {
-    k_iter_reset<<<1, 256, 0, st>>>(c, acc, nsims);
-    return cudaGetLastError();
-}
-cudaError_t launch_end(Ctl *c, SimDev *sims, SimAcc *acc, int nsims, cudaStream_t st) {
-    k_end<<<1, 256, 0, st>>>(c, sims, acc, nsims);
     return cudaGetLastError();
 }
 cudaError_t launch_probe_pixvec(int level, long long p0, long long n, int32_t *out, cudaStream_t st) {

@@ -59,13 +59,14 @@ struct MergeArgs {
 };
 
 struct ChemArgs {
-    const Ctl *ctl;
-    const SimDev *sims;
+    Ctl *ctl;
+    SimDev *sims;
     SimAcc *acc;
     int nsims;
     Cells cells;
     Ranges rg;
     int final_pass;          // 0: a trial pass of the Gamma - <n_HI> iteration (state unchanged)
+    uint4 *status;           // host memory: the last step's queue slots in use (x, y), error word, number
 };
 
 // message of the last failed call that has no context (this host thread)
@@ -73,6 +74,7 @@ void set_free_error(const std::string &msg);
 
 cudaError_t launch_pixtab(int4 *tab, int L, cudaStream_t st);
 cudaError_t launch_init_cells(const SimDev *sims, int sim, Cells c, long long ncell, cudaStream_t st);
+cudaError_t launch_reset(Ctl *c, SimDev *sims, SimAcc *acc, int nsims, cudaStream_t st);
 cudaError_t launch_emit(const EmitArgs &a, int blocks, cudaStream_t st);
 // after a march: directions of children beyond the pixel table
 cudaError_t launch_far(const EmitArgs &a, int blocks, cudaStream_t st);
@@ -98,9 +100,6 @@ cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int bloc
                          int ext);
 int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, int ext, uint32_t tile);
 cudaError_t launch_chem(const ChemArgs &a, int blocks, cudaStream_t st);
-cudaError_t launch_end(Ctl *c, SimDev *sims, SimAcc *acc, int nsims, cudaStream_t st);
-// between passes of the iteration: drop the march's output and the step's tallies (not emission)
-cudaError_t launch_iter_reset(Ctl *c, SimAcc *acc, int nsims, cudaStream_t st);
 // the merge step (Sec. 3.3) between the march and the chemistry
 // a second stream for the merge's independent rotation pass, with the events
 // that fork it from the step's stream and join it back

@@ -102,7 +102,8 @@ struct Ctl {
     int32_t merged;          // a simulation merged rays this step
     int32_t far;             // the march left children beyond the pixel table
     long long mbase;         // the march's output count: merged rays are appended from here
-    long long pad2;
+    uint32_t ticket;         // blocks of the chemistry kernel done (the last one ends the pass or step)
+    uint32_t seq;            // steps ended since the engine was made
 };
 
 // Ray queue.  A record is 6 + nb words -- emitter, birth step, direction (dx,
