@@ -324,7 +324,10 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
     const int per_sm = march_max_blocks_per_sm(cfg_.nb, march_agg_, march_minb_, march_threads_, ms, ext, q_[0].tile);
     if (per_sm < 1) return fail(FLEXRT_E_INVALID, "too many simulation slots for one march block");
     march_blocks_ = sm_count_ * std::max(per_sm, 1);
-    chem_blocks_ = (int)std::max<long long>(1, std::min<long long>((nc + 255) / 256, (long long)sm_count_ * 8));
+    // the chemistry's blocks share the cells evenly: one wave of resident ones
+    // (eight a SM, of which five fit, ran as a wave of five and one of three)
+    chem_blocks_ = (int)std::max<long long>(
+        1, std::min<long long>((nc + 255) / 256, (long long)sm_count_ * std::max(1, chem_max_blocks_per_sm(ms))));
     CK(cudaStreamSynchronize(st_));
     return FLEXRT_OK;
 }
@@ -744,6 +747,7 @@ flexrt_status Engine::launch_stage(int stage) {
         MarchSim &o = ma.one;
         o.nx = h.nx; o.ny = h.ny; o.nz = h.nz; o.l_src = h.l_src; o.l_max = h.l_max; o.active = h.active;
         o.l_merge = h.l_merge; o.gen = h.gen_mode; o.coff = h.cell_off; o.eps = h.eps_term;
+        for (int l = 0; l < MAXL; ++l) o.K[l] = h.K[l];
         for (int b = 0; b < MAXB; ++b) {
             o.sig[b] = h.sig[b]; o.sige[b] = h.sige[b]; o.eh[b] = h.eh[b];
             if (b < h.nb) o.sig_max = std::max(o.sig_max, h.sig[b]);

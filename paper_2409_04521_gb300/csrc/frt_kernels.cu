@@ -407,6 +407,7 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
     // code photons
     float *s_apn = reinterpret_cast<float *>(s_sim + A.nsims);
     int *s_gen = reinterpret_cast<int *>(s_apn + A.nsims);
+    int *s_iso = s_gen + A.nsims;
     Ctl *C = A.ctl;
     const int nrng = C->n_ranges;
     for (int i = threadIdx.x; i < A.nsims; i += blockDim.x) {
@@ -415,6 +416,7 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
         const SimDev &S = A.sims[i];
         s_apn[i] = S.apn_f;
         s_gen[i] = S.gen_mode;
+        s_iso[i] = S.isothermal;
     }
     for (int i = threadIdx.x; i <= nrng; i += blockDim.x) s_pref[i] = A.rg.pref[i];
     for (int i = threadIdx.x; i < nrng; i += blockDim.x) { s_cell0[i] = A.rg.cell0[i]; s_sim[i] = A.rg.sim[i]; }
@@ -446,7 +448,8 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
             const bool gen = s_gen[sim] != 0;
             const float4 d = A.cells.dep[g];
             const float nHf = A.cells.nHf[g];
-            const float T0 = A.cells.T[g];
+            // (an isothermal member's temperature is neither read nor written)
+            const float T0 = s_iso[sim] ? 0.0f : A.cells.T[g];
             float2 fs = make_float2(0.f, 0.f);
             double xs;                     // Generalized: x_ion; Standard: neutral fraction y
             float x0f = 0.0f;
@@ -457,9 +460,12 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
                 xs = A.cells.y[g];
                 x0f = A.cells.x[g];
             }
-            A.cells.dep[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+            // cleared for the next pass, where there is something to clear: most
+            // cells of a large box are not lit, and their 16 (24) bytes are a
+            // fifth (a third) of what the cell moves
+            if (d.w != 0.0f || d.x != 0.0f || d.y != 0.0f || d.z != 0.0f) A.cells.dep[g] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (A.cells.segcnt) A.cells.segcnt[g] = (int)d.w;
-            if (gen) A.cells.fscr[g] = make_float2(0.f, 0.f);
+            if (gen && (fs.x != 0.0f || fs.y != 0.0f)) A.cells.fscr[g] = make_float2(0.f, 0.f);
             const SimDev &SG = A.sims[sim];
             if (gen) {
                 // Generalized mode (Sec. 4.2): Gamma of the ionised part (Eq. 17
@@ -566,7 +572,7 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
                 }
                 A.cells.y[g] = y1;
                 A.cells.x[g] = x1;
-                A.cells.T[g] = T;
+                if (!S.isothermal) A.cells.T[g] = T;
                 A.cells.gamma[g] = Gf;
                 A.cells.kap[g] = cell_kappa(S, nHf, (float)y1, y1 <= S.y_thr, Gf);
                 }
@@ -750,9 +756,17 @@ int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, i
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, threads, march_shared_bytes(nsims, tile, threads));
     return n;
 }
+static size_t chem_shared_bytes(int nsims) {
+    return (size_t)nsims * 2 * sizeof(double) + (size_t)(2 * nsims + 1) * sizeof(long long) +
+           (size_t)nsims * (3 * sizeof(int) + sizeof(float));
+}
+int chem_max_blocks_per_sm(int nsims) {
+    int n = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_chem, 256, chem_shared_bytes(nsims));
+    return n;
+}
 cudaError_t launch_chem(const ChemArgs &a, int blocks, cudaStream_t st) {
-    const size_t sh = (size_t)a.nsims * 2 * sizeof(double) + (size_t)(2 * a.nsims + 1) * sizeof(long long) +
-                      (size_t)a.nsims * (2 * sizeof(int) + sizeof(float));
+    const size_t sh = chem_shared_bytes(a.nsims);
     k_chem<<<blocks, 256, sh, st>>>(a);
     return cudaGetLastError();
 }

@@ -99,6 +99,8 @@ cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext, uint32_
 cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int blocks, int threads, cudaStream_t st,
                          int ext);
 int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, int ext, uint32_t tile);
+// blocks of the chemistry kernel that an SM holds at once
+int chem_max_blocks_per_sm(int nsims);
 cudaError_t launch_chem(const ChemArgs &a, int blocks, cudaStream_t st);
 // the merge step (Sec. 3.3) between the march and the chemistry
 // a second stream for the merge's independent rotation pass, with the events

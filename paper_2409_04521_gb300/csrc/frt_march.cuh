@@ -194,21 +194,37 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
     __shared__ unsigned char sh_parent[8][32];     // splitting lanes of each warp, in order
     unsigned char *const parent = sh_parent[threadIdx.x >> 5];
     MarchSim *msim = reinterpret_cast<MarchSim *>(sh_acc + A.nsims * NACC);
+    const int lane = lane_id();
     for (int i = threadIdx.x; i < A.nsims * NACC; i += blockDim.x) sh_acc[i] = 0ull;
-    for (int i = threadIdx.x; i < A.nsims; i += blockDim.x) {
-        const SimDev &S = A.sims[i];
-        MarchSim &m = msim[i];
-        m.nx = S.nx; m.ny = S.ny; m.nz = S.nz; m.step = S.step; m.l_src = S.l_src; m.l_max = S.l_max;
-        m.active = S.active; m.l_merge = S.l_merge; m.coff = S.cell_off; m.eps = S.eps_term;
-        m.gen = S.gen_mode; m.ring0 = S.step % A.em.ring_w; m.pad1 = m.pad2 = 0;
-        for (int l = 0; l < MAXL; ++l) m.K[l] = S.K[l];
-        m.sig_max = 0.0f;
-        for (int b = 0; b < MAXB; ++b) {
-            m.sig[b] = S.sig[b]; m.sige[b] = S.sige[b]; m.eh[b] = S.eh[b];
-            if (b < S.nb) m.sig_max = fmaxf(m.sig_max, S.sig[b]);
+    if (ONE) {
+        if (threadIdx.x < MAXL) msim[0].K[threadIdx.x] = A.one.K[threadIdx.x];
+        if (threadIdx.x == 0) {
+            const int s = A.sims[0].step;
+            msim[0].step = s;
+            msim[0].ring0 = s % A.em.ring_w;
+        }
+    } else {
+        // a warp a simulation
+        for (int i = threadIdx.x >> 5; i < A.nsims; i += blockDim.x >> 5) {
+            const SimDev &S = A.sims[i];
+            MarchSim &m = msim[i];
+            if (lane < MAXL) m.K[lane] = S.K[lane];
+            float sg = 0.0f;
+            if (lane < MAXB) {
+                sg = S.sig[lane];
+                m.sig[lane] = sg; m.sige[lane] = S.sige[lane]; m.eh[lane] = S.eh[lane];
+                if (lane >= S.nb) sg = 0.0f;
+            }
+            // (cross-sections are not negative: their bits order as integers)
+            const unsigned mx = __reduce_max_sync(FULL, __float_as_uint(sg));
+            if (lane == 0) {
+                m.nx = S.nx; m.ny = S.ny; m.nz = S.nz; m.step = S.step; m.l_src = S.l_src; m.l_max = S.l_max;
+                m.active = S.active; m.l_merge = S.l_merge; m.coff = S.cell_off; m.eps = S.eps_term;
+                m.gen = S.gen_mode; m.ring0 = S.step % A.em.ring_w; m.pad1 = m.pad2 = 0;
+                m.sig_max = __uint_as_float(mx);
+            }
         }
     }
-    const int lane = lane_id();
     const unsigned tile = A.q[0].tile;
     // this warp's two tiles and their barriers (one arrival each: lane 0's)
     char *const tiles = reinterpret_cast<char *>(sh_acc) + march_tiles_offset(A.nsims) +
