@@ -333,6 +333,64 @@ __global__ void k_queue_words(Queue q, int merged, long long n, uint32_t *words,
 // ---------------------------------------------------------------------------
 // chemistry
 // ---------------------------------------------------------------------------
+// double -> float rounded to nearest even, and float -> double, of
+// non-negative values on the integer pipe: the conversions share the FP64
+// pipe (two lanes a clock on this part), which bound the kernel -- a cell of a
+// step took six double-precision operations, of which one is left.  Values
+// outside the normal float range take the conversion instruction.
+__device__ __forceinline__ float narrow(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
+    if (hi - 0x38100000u >= 0x47e00000u - 0x38100000u) return (float)v;      // not within [2^-126, 2^127)
+    const unsigned f = ((hi << 3) | (lo >> 29)) - (896u << 23);
+    return __uint_as_float(f + (((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29));
+}
+__device__ __forceinline__ double widen(float v) {
+    const unsigned f = __float_as_uint(v);
+    if (f - 0x00800000u >= 0x7f000000u) return (double)v;                    // not a positive normal number
+    return __hiloint2double((int)((f >> 3) + (896u << 20)), (int)(f << 29));
+}
+
+// One sub-step of Eq. 12 at static density: heating minus cooling (per
+// n_H^2), at most 5% of T (the thousandth takes what is left).
+__device__ __forceinline__ void t_substep(const SimDev &S, float &T, float &left, int k, float heat, float xb, float yb,
+                                          float nHf) {
+    const float pref = 2.0f * nHf / (3.0f * KB_F * (1.0f + xb));
+    const float cc = S.compton_c / nHf;
+    const float lam = cooling_f(T, xb, yb, xb, cc, S.Tcmb);
+    const float dTdt = pref * (heat - lam);
+    float h = left;
+    if (k < 999 && dTdt != 0.0f) h = fminf(h, 0.05f * T / fabsf(dTdt));
+    T += dTdt * h;
+    left -= h;
+}
+// Cells whose temperature needs more than T_INLINE sub-steps (those an
+// ionisation front is heating take up to a hundred, most others one) wait in
+// shared memory and are worked off by the whole block, each thread taking the
+// next cell when its own is done: with every lane looping to its warp's
+// longest, 8 to 12 of 32 lanes were active and these loops most of the kernel.
+constexpr int T_INLINE = 2, T_CAP = 512;
+struct TQueue {
+    float T[T_CAP], left[T_CAP], heat[T_CAP], xb[T_CAP], yb[T_CAP], nH[T_CAP];
+    unsigned cell[T_CAP];
+    int sim[T_CAP];
+    int count, next;
+};
+__device__ void t_drain(const ChemArgs &A, TQueue &q) {
+    const int n = q.count;                         // (block-uniform: a barrier is behind the last push)
+    for (;;) {
+        const int w = atomicAdd(&q.next, 1);
+        if (w >= n) break;
+        const SimDev &S = A.sims[q.sim[w]];
+        float T = q.T[w], left = q.left[w];
+        const float heat = q.heat[w], xb = q.xb[w], yb = q.yb[w], nHf = q.nH[w];
+        for (int k = T_INLINE; k < 1000 && left > 0.0f; ++k) t_substep(S, T, left, k, heat, xb, yb, nHf);
+        A.cells.T[q.cell[w]] = T;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) q.count = q.next = 0;
+    __syncthreads();
+}
+
 // The last block of a pass ends it (kernels of their own for this were a fifth
 // of a small simulation's step: one more launch a step, and one a trial pass).
 // A trial pass of the Gamma - <n_HI> iteration: the next pass marches the same
@@ -396,6 +454,8 @@ __device__ void end_pass(const ChemArgs &A) {
 
 __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
     __shared__ int s_last;
+    __shared__ TQueue tq;
+    __shared__ int s_evolve;                       // a member's temperature evolves (Standard mode, committed pass)
     // per-simulation absorbed totals and screens' excess photons, then the
     // active cell ranges
     extern __shared__ double sh_abs[];
@@ -410,6 +470,8 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
     int *s_iso = s_gen + A.nsims;
     Ctl *C = A.ctl;
     const int nrng = C->n_ranges;
+    if (threadIdx.x == 0) tq.count = tq.next = s_evolve = 0;
+    __syncthreads();
     for (int i = threadIdx.x; i < A.nsims; i += blockDim.x) {
         sh_abs[i] = 0.0;
         sh_lost[i] = 0.0;
@@ -417,13 +479,14 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
         s_apn[i] = S.apn_f;
         s_gen[i] = S.gen_mode;
         s_iso[i] = S.isothermal;
+        if (A.final_pass && !S.isothermal && !S.gen_mode && S.active) s_evolve = 1;
     }
     for (int i = threadIdx.x; i <= nrng; i += blockDim.x) s_pref[i] = A.rg.pref[i];
     for (int i = threadIdx.x; i < nrng; i += blockDim.x) { s_cell0[i] = A.rg.cell0[i]; s_sim[i] = A.rg.sim[i]; }
     __syncthreads();
     const bool err = C->err != 0;
-    const long long n = C->ncell_active;
-    const long long nr = (n + 31) & ~31LL;
+    // cell keys are 32-bit integers (the march's bound)
+    const unsigned n = (unsigned)C->ncell_active;
     const int lane = lane_id();
     // absorbed photons: each thread sums its cells of one simulation in a
     // register pair (a single-precision sum and its exact rounding error,
@@ -432,17 +495,18 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
     // atomic per run of cells, not one per warp and cell)
     float t_hi = 0.0f, t_lo = 0.0f;
     int t_sim = -1;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nr; i += (long long)gridDim.x * blockDim.x) {
+    for (unsigned base = blockIdx.x * blockDim.x; base < n; base += gridDim.x * blockDim.x) {   // block-uniform
+        const unsigned i = base + threadIdx.x;
         int sim = -1;
         float a_abs = 0.0f;
         if (i < n) {
             int lo = 0, hi = nrng;  // largest r with pref[r] <= i
             while (hi - lo > 1) {
                 int mid = (lo + hi) >> 1;
-                if (s_pref[mid] <= i) lo = mid; else hi = mid;
+                if ((unsigned)s_pref[mid] <= i) lo = mid; else hi = mid;
             }
             sim = s_sim[lo];
-            const long long g = s_cell0[lo] + (i - s_pref[lo]);
+            const unsigned g = (unsigned)s_cell0[lo] + (i - (unsigned)s_pref[lo]);
             // every load of the cell first: the stores below would otherwise
             // hold the later loads back, one memory round trip each
             const bool gen = s_gen[sim] != 0;
@@ -480,6 +544,16 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
                     // atoms of the cell Ac and the photons in code units, and
                     // the recombinations per atom alpha n_H x dt
                     a_abs = d.x + fs.x;
+                    // a cell no front has reached and no photon entered keeps
+                    // x_ion, the neutral fraction and the ionised fraction
+                    // (0, 1, 0): the rest of this branch without its
+                    // double-precision arithmetic, most of the kernel's time
+                    // in a large box (240 us a committed pass at 200^3 cells)
+                    if ((__double2hiint(xs) | __double2loint(xs)) == 0 && a_abs == 0.0f && fs.y == 0.0f) {
+                        A.cells.rho[g] = 1.0f;
+                        A.cells.kap[g] = gen_kappa(SG, nHf, 0.0f, 0.0f);
+                        if (A.final_pass) A.cells.gamma[g] = 0.0f;
+                    } else {
                     const double x = xs;
                     const float xf = (float)x, omx = (float)(1.0 - x);
                     const float Ac = nHf * s_apn[sim];                           // atoms of a whole cell
@@ -513,13 +587,14 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
                         A.cells.gamma[g] = Gf;
                         A.cells.kap[g] = gen_kappa(SG, nHf, yi, Gf);
                     }
+                    }
                 }
             } else if (!err) {
                 a_abs = d.x;
                 const SimDev &S = A.sims[sim];
                 const float Gf = d.y * S.gscale_f;                    // Eq. 17, 1/s
                 const double y0 = xs;
-                const float y0f = (float)y0;
+                const float y0f = narrow(y0);
                 const float dtf = S.dt_f;
                 float alpha = S.alpha_iso, Cc = S.coll_iso;
                 if (!S.isothermal && S.rates) { alpha = alphaB_f(T0); Cc = collion_f(T0); }
@@ -551,30 +626,30 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
                 } else {
                 // x1 + y1 = 1 holds to rounding: keep x1 in [0, 1]
                 const float x1 = fminf(fmaf(x0f, ef, gf * idt), 1.0f);
-                const double y1 = fma(y0, (double)ef, (double)(gf * bdt));   // neutral fraction kept in FP64
-                float T = T0;
+                const double y1 = fma(y0, widen(ef), widen(gf * bdt));   // neutral fraction kept in FP64
+                const float y1f = narrow(y1);
+                // (the float decides unless it lies next to the threshold)
+                const bool ionised = fabsf(y1f - S.y_thr_dn) > 1e-6f ? y1f < S.y_thr_dn : y1 <= S.y_thr;
                 if (!S.isothermal) {
                     // Eq. 12 with static density: particle-number term, then
                     // sub-stepped heating minus cooling (per n_H^2)
-                    T = T0 * (1.0f + x0f) / (1.0f + x1);
+                    float T = T0 * (1.0f + x0f) / (1.0f + x1);
                     const float heat = d.z * S.hscale_f * yb / nHf;
-                    const float pref = 2.0f * nHf / (3.0f * KB_F * (1.0f + xb));
-                    const float cc = S.compton_c / nHf;
                     float left = dtf;
-                    for (int k = 0; k < 1000 && left > 0.0f; ++k) {
-                        const float lam = cooling_f(T, xb, yb, xb, cc, S.Tcmb);
-                        const float dTdt = pref * (heat - lam);
-                        float h = left;
-                        if (k < 999 && dTdt != 0.0f) h = fminf(h, 0.05f * T / fabsf(dTdt));
-                        T += dTdt * h;
-                        left -= h;
+                    for (int k = 0; k < T_INLINE && left > 0.0f; ++k) t_substep(S, T, left, k, heat, xb, yb, nHf);
+                    if (left > 0.0f) {
+                        const int w = atomicAdd(&tq.count, 1);
+                        tq.T[w] = T; tq.left[w] = left; tq.heat[w] = heat;
+                        tq.xb[w] = xb; tq.yb[w] = yb; tq.nH[w] = nHf;
+                        tq.cell[w] = g; tq.sim[w] = sim;
+                    } else {
+                        A.cells.T[g] = T;
                     }
                 }
                 A.cells.y[g] = y1;
                 A.cells.x[g] = x1;
-                if (!S.isothermal) A.cells.T[g] = T;
                 A.cells.gamma[g] = Gf;
-                A.cells.kap[g] = cell_kappa(S, nHf, (float)y1, y1 <= S.y_thr, Gf);
+                A.cells.kap[g] = cell_kappa(S, nHf, y1f, ionised, Gf);
                 }
             }
         }
@@ -587,6 +662,14 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
             const float s = t_hi + a_abs, bp = s - t_hi;
             t_lo += (t_hi - (s - bp)) + (a_abs - bp);
             t_hi = s;
+        }
+        // an iteration pushes at most a cell a thread: drain a half-full queue
+        // (and what is left after the last iteration)
+        if (s_evolve) {
+            __syncthreads();
+            const bool drain = tq.count > T_CAP - (int)blockDim.x || n - base <= gridDim.x * blockDim.x;
+            __syncthreads();
+            if (drain) t_drain(A, tq);
         }
     }
     {
