@@ -351,7 +351,9 @@ extern "C" flexrt_status flexrt_probe_direction(int32_t level, int64_t p0, int64
     cudaGetDevice(&dev);
     const int4 *tab = nullptr;
     int lt = std::min(level, 8);
-    if (get_pixtab(dev, lt, 0, &tab) != cudaSuccess) return FLEXRT_E_CUDA;
+    PixTableRef ref;
+    if (get_pixtab(dev, lt, 0, &ref) != cudaSuccess) return FLEXRT_E_CUDA;
+    tab = ref->ptr;
     DevBuf<int32_t> dr, d;
     if (dr.alloc(9) != cudaSuccess || d.alloc(3 * n) != cudaSuccess) return FLEXRT_E_OOM;
     if (cudaMemcpy(dr.p, Rq, 9 * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess) return FLEXRT_E_CUDA;
@@ -411,7 +413,9 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int4 *tab = nullptr;
     const int lt = p->l_merge;
-    if (get_pixtab(dev, lt, 0, &tab) != cudaSuccess) return free_fail(FLEXRT_E_CUDA, "probe_merge: pixel table");
+    PixTableRef ref;
+    if (get_pixtab(dev, lt, 0, &ref) != cudaSuccess) return free_fail(FLEXRT_E_CUDA, "probe_merge: pixel table");
+    tab = ref->ptr;
     // one simulation (slot 0) whose march left the n rays in queue 1
     SimDev h;
     std::memset(&h, 0, sizeof(h));

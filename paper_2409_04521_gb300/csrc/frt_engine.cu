@@ -25,13 +25,10 @@ static float atoms_per_nH(const frt::SimDev &h) {
 }
 constexpr double MYR_S = 3.15576e13;
 
-// process-wide fixed-point pixel vector tables, one per device, grown on demand
-struct PixTable {
-    int4 *ptr = nullptr;
-    int level = -1;
-};
+// process-wide fixed-point pixel vector tables, the deepest made so far on each
+// device (never destroyed: the CUDA runtime may be gone by then)
 std::mutex g_tab_mu;
-std::map<int, PixTable> g_tabs;
+std::map<int, std::shared_ptr<PixTable>> &g_tabs = *new std::map<int, std::shared_ptr<PixTable>>;
 
 void split_table(double nmin, int32_t *K) {
     const double f = std::sqrt(3.0 / (M_PI * nmin));
@@ -78,22 +75,22 @@ cudaError_t read_queue(const Queue &q, bool merged, long long n, HostRays &out) 
     return cudaSuccess;
 }
 
-cudaError_t get_pixtab(int device, int level, cudaStream_t st, const int4 **out) {
+cudaError_t get_pixtab(int device, int level, cudaStream_t st, PixTableRef *out) {
     std::lock_guard<std::mutex> lk(g_tab_mu);
-    PixTable &t = g_tabs[device];
-    if (t.level < level) {
-        int4 *p = nullptr;
+    std::shared_ptr<PixTable> &t = g_tabs[device];
+    if (!t || t->level < level) {
+        // (the one it replaces stays with the engines that hold it)
+        auto n = std::make_shared<PixTable>();
         const size_t bytes = (size_t)(4LL * ((1LL << (2 * (level + 1))) - 1)) * sizeof(int4);
-        cudaError_t e = cudaMalloc(&p, bytes);
-        if (e != cudaSuccess) return e;
-        e = launch_pixtab(p, level, st);
+        cudaError_t e = cudaMalloc(&n->ptr, bytes);
+        if (e != cudaSuccess) { n->ptr = nullptr; return e; }
+        e = launch_pixtab(n->ptr, level, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) { cudaFree(p); return e; }
-        if (t.ptr) cudaFree(t.ptr);
-        t.ptr = p;
-        t.level = level;
+        if (e != cudaSuccess) return e;
+        n->level = level;
+        t = n;
     }
-    *out = t.ptr;
+    *out = t;
     return cudaSuccess;
 }
 
@@ -312,8 +309,9 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
     CK(cudaMemsetAsync(ctl_, 0, sizeof(Ctl), st_));
     CK(cudaMemsetAsync(sims_, 0, (size_t)ms * sizeof(SimDev), st_));
     CK(cudaMemsetAsync(acc_, 0, (size_t)ms * sizeof(SimAcc), st_));
-    cudaError_t e = get_pixtab(device_, ltab_, st_, &pixtab_);
+    cudaError_t e = get_pixtab(device_, ltab_, st_, &pixref_);
     if (e != cudaSuccess) return cuda(e, "pixel table");
+    pixtab_ = pixref_->ptr;
 
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device_);

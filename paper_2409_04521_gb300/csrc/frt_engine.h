@@ -3,6 +3,7 @@
 // simulations, launch configuration, optional CUDA-graph replay of a step.
 #pragma once
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -12,8 +13,19 @@
 
 namespace frt {
 
-// Process-wide fixed-point pixel-vector table of levels 0..level on `device`.
-cudaError_t get_pixtab(int device, int level, cudaStream_t st, const int4 **out);
+// Process-wide fixed-point pixel-vector table of at least the levels 0..level
+// on `device`.  A deeper table replaces a shallower one for later callers; a
+// table lives as long as anyone holds it.
+struct PixTable {
+    int4 *ptr = nullptr;
+    int level = -1;
+    PixTable() = default;
+    PixTable(const PixTable &) = delete;
+    PixTable &operator=(const PixTable &) = delete;
+    ~PixTable() { if (ptr) cudaFree(ptr); }
+};
+using PixTableRef = std::shared_ptr<const PixTable>;
+cudaError_t get_pixtab(int device, int level, cudaStream_t st, PixTableRef *out);
 
 // A queue of cap records at `base` (host or device): its bytes, and its view.
 inline size_t queue_bytes(long long cap, int nb, bool merged) {
@@ -157,6 +169,7 @@ class Engine {
     Ranges rg_{};
     MergeWork mw_{};
     void *mwmem_ = nullptr;
+    PixTableRef pixref_;       // keeps the table the steps read
     const int4 *pixtab_ = nullptr;
     int ltab_ = 0;
     bool far_possible_ = false;   // a member's rays may reach levels beyond the table

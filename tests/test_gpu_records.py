@@ -2,6 +2,9 @@
 edges of a warp of emitters, against the oracle; the checkpoint's ray arrays
 keep one array a word."""
 import dataclasses as dc
+import os
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -73,3 +76,35 @@ def test_children_beyond_the_batch_pixel_table():
     assert np.array_equal(kb, ks) and np.array_equal(db, ds)
     b.close()
     s.close()
+
+
+_TWO_TABLES = """
+import dataclasses as dc, sys
+import numpy as np
+sys.path[:0] = [%r, %r]
+import paper_2409_04521_gb300 as F, workloads as W
+from parity_util import ray_table
+p = W.cosmo16(n=16, nsteps=8, nsrc=3, seed=5)
+a = F.Simulation(p, ray_capacity=1 << 18)
+a.step(p.dt)
+a.sync()
+# a simulation that splits deeper makes a deeper table; the first keeps its own
+b = F.Simulation(dc.replace(p, options=dc.replace(p.options, n_ray_min=5000.0)), ray_capacity=1 << 18)
+for _ in range(7):
+    a.step(p.dt)
+ka, da, _ = ray_table(a.rays())
+c = F.Simulation(p, ray_capacity=1 << 18)
+for _ in range(8):
+    c.step(p.dt)
+kc, dd, _ = ray_table(c.rays())
+assert np.array_equal(ka, kc) and np.array_equal(da, dd)
+print("same rays", len(ka))
+"""
+
+
+def test_a_deeper_pixel_table_leaves_the_older_one_to_its_simulation():
+    # in a process of its own: the tables are the process's
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _TWO_TABLES % (root, os.path.join(root, "tests"))], cwd=root,
+                       capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "same rays" in r.stdout, r.stdout + r.stderr
