@@ -441,7 +441,7 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
     DevBuf<SimDev> dsim;
     DevBuf<SimAcc> dacc;
     DevBuf<char> qmem[2];
-    DevBuf<uint32_t> hist, sel, tkey, cand, ckey, lead_slot, bcnt, bled;
+    DevBuf<uint32_t> hseg, hist, sel, tkey, cand, ckey, lead_slot, bcnt, bled;
     DevBuf<uint4> tgrp, gcm;
     DevBuf<int32_t> tsim, rsim, lead_sim;
     DevBuf<float> grp, n0;
@@ -450,7 +450,7 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
     bool ok = dctl.alloc(1) == cudaSuccess && dsim.alloc(1) == cudaSuccess && dacc.alloc(1) == cudaSuccess;
     const size_t qbytes = queue_bytes(mq, nb, true);
     for (int k = 0; k < 2 && ok; ++k) ok = qmem[k].alloc(qbytes) == cudaSuccess;
-    ok = ok && hist.alloc(HIST_BINS) == cudaSuccess && sel.alloc(8) == cudaSuccess && tkey.alloc(m) == cudaSuccess &&
+    ok = ok && hist.alloc(HIST_BINS) == cudaSuccess && hseg.alloc(HIST_BINS / 256) == cudaSuccess && sel.alloc(8) == cudaSuccess && tkey.alloc(m) == cudaSuccess &&
          tsim.alloc(m) == cudaSuccess && gcm.alloc(ncell * ndir) == cudaSuccess && tgrp.alloc(ml) == cudaSuccess &&
          cand.alloc(ml) == cudaSuccess && ckey.alloc(ml) == cudaSuccess && bcnt.alloc(MERGE_MAX_BLOCKS) == cudaSuccess &&
          bled.alloc(MERGE_MAX_BLOCKS) == cudaSuccess &&
@@ -491,7 +491,7 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
     em.cell = ecell.p; em.n0 = n0.p;
     Ranges rg{pref.p, cell0.p, rsim.p};
     MergeWork w{};
-    w.hist = hist.p; w.sel = sel.p; w.tkey = tkey.p; w.tsim = tsim.p;
+    w.hist = hist.p; w.hseg = hseg.p; w.sel = sel.p; w.tkey = tkey.p; w.tsim = tsim.p;
     w.grp = grp.p; w.gcm = gcm.p; w.cand = cand.p; w.ckey = ckey.p; w.tgrp = tgrp.p; w.rot = rot.p; w.ndir = ndir;
     w.grp_w = gw; w.hrep = 1; w.lead_slot = lead_slot.p; w.lead_sim = lead_sim.p;
     w.bcnt = bcnt.p; w.bled = bled.p; w.lead_cap = ml;

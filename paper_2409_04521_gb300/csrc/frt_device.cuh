@@ -130,21 +130,24 @@ __device__ __forceinline__ uint64_t sm64(uint64_t z) {
 }
 constexpr uint64_t GOLD = 0x9E3779B97F4A7C15ULL;
 
-// num / den rounded half to even, for 0 < den <= 2^30 and |num / den| <= 2^24,
-// given rden, the single-precision reciprocal of den: an estimate within a
-// few units (three single-precision roundings of a quotient below 2^24)
-// corrected exactly by the remainder
-__device__ __forceinline__ int32_t div_round_even(long long num, int32_t den, float rden) {
-    int32_t q = __float2int_rz((float)num * rden);
-    long long r = num - (long long)q * den;
-    for (int k = 0; k < 16 && r < 0; ++k) { --q; r += den; }
-    for (int k = 0; k < 16 && r >= den; ++k) { ++q; r -= den; }
-    if (2 * r > den || (2 * r == den && (q & 1))) ++q;
+// Q 2^24 / den rounded half to even, for 0 < den <= 2^30 and |Q| <= den,
+// given rden, the single-precision reciprocal of den: an estimate within four
+// of the quotient (three single-precision roundings of a number up to 2^24),
+// corrected by the rounded quotient of its exact remainder, which leaves at
+// most a little over half of den
+__device__ __forceinline__ int32_t div24_round_even(int32_t Q, int32_t den, float rden) {
+    const int32_t q0 = __float2int_rn((float)Q * rden * 16777216.0f);
+    const long long r0 = ((long long)Q << 24) - (long long)q0 * den;
+    const int32_t q1 = __float2int_rn((float)(int32_t)(r0 >> 2) * rden * 4.0f);
+    int32_t q = q0 + q1, r = (int32_t)(r0 - (long long)q1 * den);
+    if (2 * r > den) { ++q; r -= den; }
+    if (2 * r < -den) { --q; r += den; }
+    if (q & 1) q += (2 * r == den) - (2 * r == -den);
     return q;
 }
 
-__device__ inline void rotation_rows(uint64_t seed, long long e, long long s, int rotate, int4 rows[3]) {
-    long long w = 1, x = 0, y = 0, z = 0;
+__device__ __forceinline__ void rotation_rows(uint64_t seed, long long e, long long s, int rotate, int4 rows[3]) {
+    int w = 1, x = 0, y = 0, z = 0;
     if (rotate) {
         uint64_t h = sm64(seed + GOLD);
         h = sm64(h + GOLD * (uint64_t)(e + 1));
@@ -157,14 +160,15 @@ __device__ inline void rotation_rows(uint64_t seed, long long e, long long s, in
             if (n2 > 0u && n2 <= (1u << 30)) { w = a; x = b; y = c; z = d; break; }
         }
     }
-    const long long n = w * w + x * x + y * y + z * z;
-    const long long Q[9] = {w * w + x * x - y * y - z * z, 2 * (x * y - w * z), 2 * (x * z + w * y),
-                            2 * (x * y + w * z), w * w - x * x + y * y - z * z, 2 * (y * z - w * x),
-                            2 * (x * z - w * y), 2 * (y * z + w * x), w * w - x * x - y * y + z * z};
+    // |q|^2 <= 2^30: every product sum below fits 32 bits
+    const int n = w * w + x * x + y * y + z * z;
+    const int Q[9] = {w * w + x * x - y * y - z * z, 2 * (x * y - w * z), 2 * (x * z + w * y),
+                      2 * (x * y + w * z), w * w - x * x + y * y - z * z, 2 * (y * z - w * x),
+                      2 * (x * z - w * y), 2 * (y * z + w * x), w * w - x * x - y * y + z * z};
     int32_t q[9];
     const float rn = __frcp_rn((float)n);          // one reciprocal for the nine entries
 #pragma unroll
-    for (int i = 0; i < 9; ++i) q[i] = div_round_even(Q[i] * (1LL << VQ_BITS), (int32_t)n, rn);
+    for (int i = 0; i < 9; ++i) q[i] = div24_round_even(Q[i], n, rn);
     for (int r = 0; r < 3; ++r) rows[r] = make_int4(q[3 * r], q[3 * r + 1], q[3 * r + 2], 0);
 }
 

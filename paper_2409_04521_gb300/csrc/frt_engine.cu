@@ -270,7 +270,8 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
         const size_t sz[] = {(size_t)ms * mw_.hrep * HIST_BINS * 4, (size_t)ms * 32, (size_t)cap * 4,
                              (size_t)cap * 4, (size_t)ngrp * mw_.grp_w * 4, (size_t)ngrp * 16,
                              (size_t)nc * 48, nl * 4, nl * 4, nl * 4, nl * 4, nl * 16,
-                             (size_t)MERGE_MAX_BLOCKS * 4, (size_t)MERGE_MAX_BLOCKS * 4};
+                             (size_t)MERGE_MAX_BLOCKS * 4, (size_t)MERGE_MAX_BLOCKS * 4,
+                             (size_t)ms * (HIST_BINS / 256) * 4};
         size_t tot = 0;
         for (size_t v : sz) tot += (v + 255) & ~(size_t)255;
         if (dev_alloc(&mwmem_, tot) != cudaSuccess) return fail(FLEXRT_E_OOM, "merge scratch allocation failed");
@@ -278,7 +279,7 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
         void **dst[] = {(void **)&mw_.hist, (void **)&mw_.sel, (void **)&mw_.tkey, (void **)&mw_.tsim,
                         (void **)&mw_.grp, (void **)&mw_.gcm, (void **)&mw_.rot, (void **)&mw_.cand,
                         (void **)&mw_.ckey, (void **)&mw_.lead_slot, (void **)&mw_.lead_sim, (void **)&mw_.tgrp,
-                        (void **)&mw_.bcnt, (void **)&mw_.bled};
+                        (void **)&mw_.bcnt, (void **)&mw_.bled, (void **)&mw_.hseg};
         static_assert(sizeof(sz) / sizeof(sz[0]) == sizeof(dst) / sizeof(dst[0]), "merge scratch layout");
         for (size_t k = 0; k < sizeof(sz) / sizeof(sz[0]); ++k) { *dst[k] = p; p += (sz[k] + 255) & ~(size_t)255; }
         if (cap >= (1LL << 32)) return fail(FLEXRT_E_INVALID, "merging needs fewer than 2^32 queue slots");

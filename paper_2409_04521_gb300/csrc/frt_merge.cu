@@ -5,7 +5,8 @@
 // K = floor(N_ex * N_RT)):
 //   k_mrot    : per cell, the random rotation of the cell's merge sphere for
 //               this step, drawn like an emitter's sphere (key 2^31 + local
-//               cell index; exact integer arithmetic);
+//               cell index; exact integer arithmetic); not for a simulation
+//               with few candidates (draws_late);
 //   k_mhist1  : per ray, its content (single-precision sum of its bins, the
 //               quantity ranked) and a histogram of the content's upper 16 bits;
 //   k_mfind   : per simulation, a two-pass radix select of the K-th largest
@@ -40,6 +41,7 @@
 // survivors densely into the other queue, so no compaction pass is needed.
 // Contents are non-negative floats, so their bit patterns order as unsigned
 // integers and the select and the group maximum work on the bits.
+#include <algorithm>
 #include "frt_march.cuh"
 
 namespace frt {
@@ -52,8 +54,8 @@ MarchFn march_fn_merge(int nb, int agg, int minb) { return march_pick<1, false>(
 namespace {
 
 // per-simulation selection words: state, upper bits, rays above, T_ref bits,
-// any exempt, rays removed by this step's merge
-constexpr int SEL_STATE = 0, SEL_HIGH = 1, SEL_ABOVE = 2, SEL_T = 3, SEL_EXEMPT = 4, SEL_DROP = 5, SEL_W = 8;
+// any exempt, rays removed by this step's merge, rotations drawn late
+constexpr int SEL_STATE = 0, SEL_HIGH = 1, SEL_ABOVE = 2, SEL_T = 3, SEL_EXEMPT = 4, SEL_DROP = 5, SEL_LATE = 6, SEL_W = 8;
 constexpr uint32_t SEL_OFF = 0, SEL_PASS2 = 1, SEL_DONE = 2;
 constexpr int WBITS = 28;                    // merge weights below 2^28
 constexpr uint32_t NO_GROUP = 0xffffffffu;   // a queue slot that is in no group
@@ -79,6 +81,17 @@ __device__ __forceinline__ unsigned long long div_rne(unsigned long long num, un
 // does simulation `sim` merge at the end of this step
 __device__ __forceinline__ bool merges(const SimDev &S, const SimAcc &a) {
     return S.active && S.merge && a.p_rays_out > (double)S.k_ex;
+}
+
+// whether the merging simulation's rotations are drawn by the passes that use
+// them, for each candidate and merged ray, instead of for every cell
+// beforehand: when its candidates (at most the rays beyond the exempt ones)
+// are fewer than half its cells.  Drawing 8e6 rotations took 250 us a step
+// (and hid the 75 us of selection passes beside it) where 1.2e6 candidates
+// need 40 us in the group pass; with more candidates than cells (2e6 cells,
+// 5e6 candidates) the rotations drawn beforehand cost nothing, hidden.
+__device__ __forceinline__ bool draws_late(const SimDev &S, double rays_out) {
+    return 2.0 * (rays_out - (double)S.k_ex) < (double)S.ncell;
 }
 
 // warp-aggregated histogram increment; bin < 0: nothing
@@ -114,67 +127,16 @@ __device__ __forceinline__ unsigned long long warp_incl_scan64(unsigned long lon
     return v;
 }
 
-// In hist[0..HIST_BINS) find the largest bin b with above + count(bins >= b)
-// >= K (K > above, and the total reaches K).  Returns b and the count above
-// b.  A block of 1024 threads visits the bins from the top, d = HIST_BINS - 1
-// - bin: warp w owns d in [2048 w, 2048 w + 2048), in rows of 32 bins (128
-// contiguous bytes); lane l sums the rows l and l + 32 of its warp.  The warp
-// holding the K-th ray then finds its row from the row sums, and the bin
-// within the row.
-__device__ void select_bin(const uint32_t *hist, unsigned long long above, unsigned long long K, uint32_t *out_bin,
-                           unsigned long long *out_above, uint32_t (*s_rows)[64], unsigned long long *s_w) {
-    constexpr int WB = HIST_BINS / 32;
-    const int lane = lane_id(), w = threadIdx.x >> 5;
-    uint32_t rs[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int d0 = w * WB + 32 * (lane + 32 * h);
-        const uint4 *src = reinterpret_cast<const uint4 *>(hist + (HIST_BINS - 32 - d0));
-        uint4 v[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) v[k] = src[k];
-        uint32_t t = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) t += v[k].x + v[k].y + v[k].z + v[k].w;
-        rs[h] = t;
-        s_rows[w][lane + 32 * h] = t;
-    }
-    unsigned long long tw = (unsigned long long)rs[0] + rs[1];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) tw += __shfl_xor_sync(FULL, tw, o);
-    if (lane == 0) s_w[w] = tw;
+// Block-wide inclusive prefix sum over 256 threads in order (s_w: 8 words;
+// every thread calls it; a barrier ends it, so that s_w can be used again).
+__device__ __forceinline__ unsigned long long block_incl_scan(unsigned long long v, unsigned long long *s_w) {
+    const unsigned long long inc = warp_incl_scan64(v);
+    if (lane_id() == 31) s_w[threadIdx.x >> 5] = inc;
     __syncthreads();
-    if (w == 0) {
-        const unsigned long long v = s_w[lane], inc = warp_incl_scan64(v);
-        s_w[32 + lane] = inc;
-        __syncwarp();
-        s_w[lane] = inc - v;
-    }
+    unsigned long long before = 0;
+    for (int k = 0; k < (int)(threadIdx.x >> 5); ++k) before += s_w[k];
     __syncthreads();
-    unsigned long long acc = above + s_w[w];
-    if (!(acc < K && K <= above + s_w[32 + w])) return;      // warp-uniform
-    int row = -1;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        if (row >= 0) break;
-        const unsigned long long v = s_rows[w][lane + 32 * h], inc = acc + warp_incl_scan64(v);
-        const unsigned hit = __ballot_sync(FULL, inc - v < K && K <= inc);
-        if (hit) {
-            const int src = __ffs(hit) - 1;
-            row = 32 * h + src;
-            acc = __shfl_sync(FULL, inc - v, src);
-        } else {
-            acc = __shfl_sync(FULL, inc, 31);
-        }
-    }
-    if (row < 0) return;                                     // not reached: the warp holds the K-th
-    const int d = w * WB + 32 * row + lane;
-    const unsigned long long c = hist[HIST_BINS - 1 - d], inc = acc + warp_incl_scan64(c);
-    const unsigned hit = __ballot_sync(FULL, inc - c < K && K <= inc);
-    if (lane == __ffs(hit) - 1) {
-        *out_bin = (uint32_t)(HIST_BINS - 1 - d);
-        *out_above = inc - c;
-    }
+    return before + inc;
 }
 
 }  // namespace
@@ -189,9 +151,14 @@ __global__ void __launch_bounds__(256) k_mrot(MergeArgs A) {
     const Ctl *C = A.ctl;
     const int nrng = C->n_ranges;
     for (int i = threadIdx.x; i <= nrng; i += blockDim.x) s_pref[i] = A.rg.pref[i];
-    for (int i = threadIdx.x; i < nrng; i += blockDim.x) { s_cell0[i] = A.rg.cell0[i]; s_sim[i] = A.rg.sim[i]; }
-    __syncthreads();
-    if (C->err) return;
+    bool any = false;                              // a simulation whose rotations are drawn here
+    for (int i = threadIdx.x; i < nrng; i += blockDim.x) {
+        const int s = A.rg.sim[i];
+        s_cell0[i] = A.rg.cell0[i];
+        s_sim[i] = s;
+        any = any || (merges(A.sims[s], A.acc[s]) && !draws_late(A.sims[s], A.acc[s].p_rays_out));
+    }
+    if (!__syncthreads_or(any) || C->err) return;
     const long long n = C->ncell_active;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         int lo = 0, hi = nrng;
@@ -201,7 +168,7 @@ __global__ void __launch_bounds__(256) k_mrot(MergeArgs A) {
         }
         const int sim = s_sim[lo];
         const SimDev &S = A.sims[sim];
-        if (!merges(S, A.acc[sim])) continue;
+        if (!merges(S, A.acc[sim]) || draws_late(S, A.acc[sim].p_rays_out)) continue;
         const long long local = i - s_pref[lo];
         int4 rows[3];
         rotation_rows(S.seed, (1LL << 31) + local, S.step, S.rotate, rows);
@@ -213,9 +180,12 @@ __global__ void __launch_bounds__(256) k_mrot(MergeArgs A) {
 // ---------------------------------------------------------------------------
 // rank contents and the first histogram
 // ---------------------------------------------------------------------------
-// the histogram copy a block adds to (copies spread the atomics on hot bins)
+// A simulation's histogram is kept in hrep rows of HIST_BINS: with more than
+// one, blocks add to all but the last in turn (copies spread the atomics on hot
+// bins) and the last takes their sum; a single row is both.
 __device__ __forceinline__ long long hist_row(const MergeWork &w, int sim) {
-    return ((long long)sim * w.hrep + (long long)(blockIdx.x % w.hrep)) * HIST_BINS;
+    const int adds = w.hrep > 1 ? w.hrep - 1 : 1;
+    return ((long long)sim * w.hrep + (long long)(blockIdx.x % adds)) * HIST_BINS;
 }
 
 __global__ void __launch_bounds__(256) k_mhist1(MergeArgs A) {
@@ -258,79 +228,89 @@ __global__ void __launch_bounds__(256) k_mhist1(MergeArgs A) {
     }
 }
 
-// sum each simulation's histogram copies into copy 0 (and clear the others)
+// A block sums one segment (256 bins) of one simulation's copies: the counts
+// into the sum row, the segment's total into hseg; the copies are cleared for
+// the next pass.
+constexpr int SEGS = HIST_BINS / 256;
 __global__ void __launch_bounds__(256) k_mreduce(MergeArgs A, int pass) {
+    __shared__ unsigned long long s_w[8];
     const Ctl *C = A.ctl;
     if (C->err) return;
     const int hrep = A.w.hrep;
-    const long long n = (long long)A.nsims * HIST_BINS;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int s = (int)(i / HIST_BINS);
+    for (int j = blockIdx.x; j < A.nsims * SEGS; j += gridDim.x) {
+        const int s = j / SEGS, seg = j % SEGS;
         const bool on = pass == 1 ? merges(A.sims[s], A.acc[s]) : A.w.sel[SEL_W * s + SEL_STATE] == SEL_PASS2;
-        if (!on) continue;
-        uint32_t *h = A.w.hist + (long long)s * hrep * HIST_BINS + (i % HIST_BINS);
-        // every copy's count first (independent loads in flight together),
-        // then the clears
-        uint32_t cnt[32];
-#pragma unroll
-        for (int c = 0; c < 32; ++c) cnt[c] = c < hrep ? h[(long long)c * HIST_BINS] : 0u;
+        if (!on) continue;                                   // block-uniform
+        uint32_t *h = A.w.hist + (long long)s * hrep * HIST_BINS + 256 * seg + threadIdx.x;
         uint32_t sum = 0u;
+        if (hrep > 1) {
+            // every copy's count first (independent loads in flight together),
+            // then the clears
+            uint32_t cnt[31];
 #pragma unroll
-        for (int c = 0; c < 32; ++c) sum += cnt[c];
-        for (int c = 1; c < hrep; ++c) h[(long long)c * HIST_BINS] = 0u;
-        h[0] = sum;
+            for (int c = 0; c < 31; ++c) cnt[c] = c < hrep - 1 ? h[(long long)c * HIST_BINS] : 0u;
+#pragma unroll
+            for (int c = 0; c < 31; ++c) {
+                sum += cnt[c];
+                if (cnt[c]) h[(long long)c * HIST_BINS] = 0u;
+            }
+            h[(long long)(hrep - 1) * HIST_BINS] = sum;
+        } else {
+            sum = *h;
+        }
+        const unsigned long long inc = block_incl_scan(sum, s_w);
+        if (threadIdx.x == 255) A.w.hseg[j] = (uint32_t)inc;
     }
 }
 
 // ---------------------------------------------------------------------------
-// per simulation: the threshold's upper 16 bits (pass 1) or all 32 (pass 2)
+// per simulation: the threshold's upper 16 bits (pass 1) or all 32 (pass 2):
+// the largest bin b with above + count(bins >= b) >= K, found from the
+// segments' totals, then within one segment (one block over all 65536 bins,
+// which it also cleared, took 14 us a pass, these 512 words a few).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(1024) k_mfind(MergeArgs A, int pass) {
-    __shared__ uint32_t s_rows[32][64];
-    __shared__ unsigned long long s_w[64];
-    __shared__ uint32_t s_bin;
+__global__ void __launch_bounds__(256) k_mfind(MergeArgs A, int pass) {
+    __shared__ unsigned long long s_w[8];
+    __shared__ int s_seg, s_bin;
     __shared__ unsigned long long s_above;
     Ctl *C = A.ctl;
-    const int s = blockIdx.x;
+    const int s = blockIdx.x, t = threadIdx.x;
     if (C->err) return;
     uint32_t *sel = A.w.sel + SEL_W * s;
-    uint32_t *hist = A.w.hist + (long long)s * A.w.hrep * HIST_BINS;
     const SimDev &S = A.sims[s];
-    if (pass == 1) {
-        if (!merges(S, A.acc[s])) {
-            if (threadIdx.x == 0) sel[SEL_STATE] = SEL_OFF;
-            return;
-        }
-        if (threadIdx.x == 0) {
+    if (pass == 1 ? !merges(S, A.acc[s]) : sel[SEL_STATE] != SEL_PASS2) {
+        if (pass == 1 && t == 0) sel[SEL_STATE] = SEL_OFF;
+        return;
+    }
+    const unsigned long long K = S.k_ex > 0 ? (unsigned long long)S.k_ex : 1ull;
+    const unsigned long long above = pass == 1 ? 0ull : sel[SEL_ABOVE];
+    uint32_t *hist = A.w.hist + ((long long)s * A.w.hrep + A.w.hrep - 1) * HIST_BINS;
+    if (t == 0) { s_seg = 0; s_bin = 0; s_above = above; }
+    __syncthreads();
+    // thread t takes the t-th segment (then bin) from the top
+    unsigned long long c = A.w.hseg[s * SEGS + SEGS - 1 - t];
+    unsigned long long inc = above + block_incl_scan(c, s_w);
+    if (inc - c < K && K <= inc) { s_seg = SEGS - 1 - t; s_above = inc - c; }
+    __syncthreads();
+    c = hist[256 * s_seg + 255 - t];
+    inc = s_above + block_incl_scan(c, s_w);
+    if (inc - c < K && K <= inc) { s_bin = 256 * s_seg + 255 - t; s_above = inc - c; }
+    __syncthreads();
+    if (t == 0) {
+        if (pass == 1) {
             C->merged = 1;
-            s_bin = 0u;
-            s_above = 0ull;
-        }
-        const unsigned long long K = S.k_ex > 0 ? (unsigned long long)S.k_ex : 1ull;
-        select_bin(hist, 0ull, K, &s_bin, &s_above, s_rows, s_w);
-        __syncthreads();
-        if (threadIdx.x == 0) {
             sel[SEL_STATE] = SEL_PASS2;
-            sel[SEL_HIGH] = s_bin;
+            sel[SEL_HIGH] = (uint32_t)s_bin;
             sel[SEL_ABOVE] = (uint32_t)s_above;
             sel[SEL_EXEMPT] = S.k_ex > 0 ? 1u : 0u;
-        }
-    } else {
-        if (sel[SEL_STATE] != SEL_PASS2) return;
-        if (threadIdx.x == 0) {
-            s_bin = 0u;
-            s_above = 0ull;
-        }
-        const unsigned long long K = S.k_ex > 0 ? (unsigned long long)S.k_ex : 1ull;
-        select_bin(hist, (unsigned long long)sel[SEL_ABOVE], K, &s_bin, &s_above, s_rows, s_w);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            sel[SEL_T] = (sel[SEL_HIGH] << 16) | s_bin;
+            sel[SEL_LATE] = draws_late(S, A.acc[s].p_rays_out) ? 1u : 0u;
+        } else {
+            sel[SEL_T] = (sel[SEL_HIGH] << 16) | (uint32_t)s_bin;
             sel[SEL_STATE] = SEL_DONE;
         }
     }
-    __syncthreads();
-    for (int k = threadIdx.x; k < HIST_BINS; k += blockDim.x) hist[k] = 0u;   // ready for the next pass
+    if (A.w.hrep == 1)
+        for (int k = t; k < HIST_BINS; k += 256) hist[k] = 0u;   // ready for the next pass
 }
 
 // The candidate and merged-ray lists are built without a global counter:
@@ -533,8 +513,13 @@ __global__ void __launch_bounds__(256, 4) k_mgroup(MergeArgs A) {
                 const long long cx = p[0] >> FRAC_BITS, cy = p[1] >> FRAC_BITS, cz = p[2] >> FRAC_BITS;
                 if (cx >= 0 && cy >= 0 && cz >= 0 && cx < S.nx && cy < S.ny && cz < S.nz) {
                     const long long g = S.cell_off + (cz * S.ny + cy) * S.nx + cx;
-                    const int4 *rp = A.w.rot + 3 * g;
-                    const int4 rows[3] = {rp[0], rp[1], rp[2]};
+                    int4 rows[3];
+                    if (sel[SEL_LATE]) {
+                        rotation_rows(S.seed, (1LL << 31) + (g - S.cell_off), S.step, S.rotate, rows);
+                    } else {
+                        const int4 *rp = A.w.rot + 3 * g;
+                        rows[0] = rp[0]; rows[1] = rp[1]; rows[2] = rp[2];
+                    }
                     slot = g * ndir + merge_pixel(S.l_merge, rows, dx, dy, dz);
                     // the end point's offsets in its cell (21 bits each), the
                     // distance (16 bits) and the level (4 bits), packed
@@ -760,8 +745,13 @@ __global__ void __launch_bounds__(256, 4) k_memit(MergeArgs A) {
         const int Adist = (int)min(div_rne(gs[4], W), 65535ull);
         const int L2 = min(max((int)div_rne(gs[5], W), S.l_merge), S.l_max);
         const float *gph = gp + 2 * GSUMS;
-        const int4 *rp = A.w.rot + 3 * g;
-        const int4 rows[3] = {rp[0], rp[1], rp[2]};
+        int4 rows[3];
+        if (A.w.sel[SEL_W * sim + SEL_LATE]) {
+            rotation_rows(S.seed, (1LL << 31) + local, S.step, S.rotate, rows);
+        } else {
+            const int4 *rp = A.w.rot + 3 * g;
+            rows[0] = rp[0]; rows[1] = rp[1]; rows[2] = rp[2];
+        }
         const int4 vq = S.l_merge <= A.ltab ? __ldg(&A.pixtab[level_offset(S.l_merge) + pm])
                                             : healpix_vq(S.l_merge, pm);
         int32_t dx, dy, dz;
@@ -812,11 +802,11 @@ cudaError_t launch_merge(const MergeArgs &a, int sm_count, cudaStream_t st, cons
         k_mrot<<<rblocks, 256, rng_sh, st>>>(a);
     }
     k_mhist1<<<rblocks, 256, 0, st>>>(a);
-    if (a.w.hrep > 1) k_mreduce<<<rblocks, 256, 0, st>>>(a, 1);
-    k_mfind<<<a.nsims, 1024, 0, st>>>(a, 1);
+    k_mreduce<<<std::min(a.nsims * SEGS, rblocks), 256, 0, st>>>(a, 1);
+    k_mfind<<<a.nsims, 256, 0, st>>>(a, 1);
     k_mhist2<<<rblocks, 256, 0, st>>>(a);
-    if (a.w.hrep > 1) k_mreduce<<<rblocks, 256, 0, st>>>(a, 2);
-    k_mfind<<<a.nsims, 1024, 0, st>>>(a, 2);
+    k_mreduce<<<std::min(a.nsims * SEGS, rblocks), 256, 0, st>>>(a, 2);
+    k_mfind<<<a.nsims, 256, 0, st>>>(a, 2);
     if (side && (e = cudaStreamWaitEvent(st, side->join, 0)) != cudaSuccess) return e;
     k_mgroup<<<rblocks, 256, 0, st>>>(a);
     k_mweight<<<rblocks, 256, (size_t)a.nsims * sizeof(uint32_t), st>>>(a);

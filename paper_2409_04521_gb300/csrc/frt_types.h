@@ -182,7 +182,8 @@ struct Emitters {
 
 // Scratch of the merge step (Sec. 3.3).
 struct MergeWork {
-    uint32_t *hist;          // [slot][hrep][HIST_BINS] radix-select counts
+    uint32_t *hist;          // [slot][hrep][HIST_BINS] radix-select counts (the last of several: their sum)
+    uint32_t *hseg;          // [slot][HIST_BINS / 256] their totals over 256 bins
     uint32_t *sel;           // [slot][8]: selection state, upper bits, rays above, T_ref bits, any exempt
     uint32_t *tkey;          // per queue slot: rank content (float bits)
     int32_t *tsim;           // per queue slot: simulation taking part, -1 none
@@ -203,7 +204,7 @@ struct MergeWork {
     long long lead_cap;      // entries of the candidate and merged-ray lists
     int32_t ndir;            // group slots per cell (12 * 4^l_merge of the deepest allowed level)
     int32_t grp_w;           // floats per group
-    int32_t hrep;            // copies of each simulation's histogram (spreads hot bins)
+    int32_t hrep;            // rows of each simulation's histogram (1, or copies that spread hot bins and their sum)
     int32_t pad;
 };
 
