@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 SO = os.path.join(BUILD, "libflexrt.so")
 SOURCES = ["flexrt_api.cu", "frt_engine.cu", "frt_kernels.cu", "frt_merge.cu", "frt_march_gen.cu", "frt_march_one.cu",
-           "frt_march_one_gen.cu", "frt_static.cu"]
+           "frt_march_one_gen.cu", "frt_march_two.cu", "frt_march_two_gen.cu", "frt_static.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]
 

@@ -746,13 +746,16 @@ flexrt_status Engine::launch_stage(int stage) {
         MarchSim &o = ma.one;
         o.nx = h.nx; o.ny = h.ny; o.nz = h.nz; o.l_src = h.l_src; o.l_max = h.l_max; o.active = h.active;
         o.l_merge = h.l_merge; o.gen = h.gen_mode; o.coff = h.cell_off; o.eps = h.eps_term;
+        // decided by the march (an aggregating variant is the general one, which
+        // deposits four words) for the chemistry that reads its deposits
+        if (stage == 1) dep_two_ = march_agg_ == 0 && !cells_.segcnt && (h.isothermal || h.gen_mode);
         for (int l = 0; l < MAXL; ++l) o.K[l] = h.K[l];
         for (int b = 0; b < MAXB; ++b) {
             o.sig[b] = h.sig[b]; o.sige[b] = h.sige[b]; o.eh[b] = h.eh[b];
             if (b < h.nb) o.sig_max = std::max(o.sig_max, h.sig[b]);
         }
     }
-    ChemArgs ca{ctl_, sims_, acc_, ms, cells_, rg_, 1, reinterpret_cast<uint4 *>(h_status_)};
+    ChemArgs ca{ctl_, sims_, acc_, ms, cells_, rg_, dep_two_ ? 1 : 0, 1, reinterpret_cast<uint4 *>(h_status_)};
     const bool prof = profiling_ && !cfg_.use_graph;      // (a profiled single simulation is never replayed)
     cudaEvent_t e0 = nullptr;
     auto tic = [&]() {
@@ -773,7 +776,8 @@ flexrt_status Engine::launch_stage(int stage) {
             if (sl.used) iters = std::max(iters, (int)sl.h.gamma_iters);
         for (int it = 0; it + 1 < iters; ++it) {
             tic();
-            CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, st_, ext_variants()));
+            CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, st_,
+                            ext_variants() | (dep_two_ ? 8 : 0)));
             toc(1);
             ChemArgs ct = ca;
             ct.final_pass = 0;
@@ -782,7 +786,8 @@ flexrt_status Engine::launch_stage(int stage) {
             toc(2);
     }
         tic();
-        CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, st_, ext_variants()));
+        CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, st_,
+                            ext_variants() | (dep_two_ ? 8 : 0)));
         toc(1);
         if (far_possible_) CK(launch_far(ea, sm_count_, st_));
         return FLEXRT_OK;

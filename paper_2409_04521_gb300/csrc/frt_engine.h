@@ -172,6 +172,7 @@ class Engine {
     PixTableRef pixref_;       // keeps the table the steps read
     const int4 *pixtab_ = nullptr;
     int ltab_ = 0;
+    bool dep_two_ = false;        // the march's deposits are two words (Cells::dep)
     bool far_possible_ = false;   // a member's rays may reach levels beyond the table
     int em_cap_ = 0;
     long long qcap_ = 0;       // allocated queue slots (capacity plus run-tail margin)

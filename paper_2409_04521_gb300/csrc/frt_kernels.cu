@@ -510,7 +510,13 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
             // every load of the cell first: the stores below would otherwise
             // hold the later loads back, one memory round trip each
             const bool gen = s_gen[sim] != 0;
-            const float4 d = A.cells.dep[g];
+            float4 d;
+            if (A.two) {
+                const float2 d2 = reinterpret_cast<const float2 *>(A.cells.dep)[g];
+                d = make_float4(d2.x, d2.y, 0.0f, 0.0f);
+            } else {
+                d = A.cells.dep[g];
+            }
             const float nHf = A.cells.nHf[g];
             // (an isothermal member's temperature is neither read nor written)
             const float T0 = s_iso[sim] ? 0.0f : A.cells.T[g];
@@ -527,7 +533,10 @@ __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {
             // cleared for the next pass, where there is something to clear: most
             // cells of a large box are not lit, and their 16 (24) bytes are a
             // fifth (a third) of what the cell moves
-            if (d.w != 0.0f || d.x != 0.0f || d.y != 0.0f || d.z != 0.0f) A.cells.dep[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (d.w != 0.0f || d.x != 0.0f || d.y != 0.0f || d.z != 0.0f) {
+                if (A.two) reinterpret_cast<float2 *>(A.cells.dep)[g] = make_float2(0.f, 0.f);
+                else A.cells.dep[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
             if (A.cells.segcnt) A.cells.segcnt[g] = (int)d.w;
             if (gen && (fs.x != 0.0f || fs.y != 0.0f)) A.cells.fscr[g] = make_float2(0.f, 0.f);
             const SimDev &SG = A.sims[sim];
@@ -807,11 +816,14 @@ static MarchFn march_fn(int nb, int agg, int minb, int ext) {
             case 4: return march_fn_one(nb, agg, minb);
             case 5: return march_fn_one_merge(nb, agg, minb);
             case 7: return march_fn_one_gen(nb, agg, minb);
+            case 12: return march_fn_two(nb, agg, minb);
+            case 13: return march_fn_two_merge(nb, agg, minb);
+            case 15: return march_fn_two_gen(nb, agg, minb);
             default: break;
         }
     }
     switch (ext & 3) {
-        case 0: return march_pick<0, false>(nb, agg, minb);
+        case 0: return march_pick<0, 0>(nb, agg, minb);
         case 1: return march_fn_merge(nb, agg, minb);
         case 3: return march_fn_gen(nb, agg, minb);
         default: return nullptr;
@@ -822,8 +834,11 @@ cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext, uint32_
     MarchFn f = march_fn(nb, agg, minb, ext);
     if (!f) return cudaErrorInvalidValue;
     const size_t sh = march_shared_bytes(nsims, tile, 256);
-    if (sh > 48 * 1024) return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
-    return cudaSuccess;
+    if (sh <= 48 * 1024) return cudaSuccess;
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    MarchFn two = ext & 4 ? march_fn(nb, agg, minb, ext | 8) : f;      // a launch may take either
+    if (e == cudaSuccess && two != f) e = cudaFuncSetAttribute(two, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    return e;
 }
 cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int blocks, int threads, cudaStream_t st,
                          int ext) {

@@ -65,6 +65,7 @@ struct ChemArgs {
     int nsims;
     Cells cells;
     Ranges rg;
+    int two;                 // deposits of two words (Cells::dep)
     int final_pass;          // 0: a trial pass of the Gamma - <n_HI> iteration (state unchanged)
     uint4 *status;           // host memory: the last step's queue slots in use (x, y), error word, number
 };
@@ -90,9 +91,12 @@ MarchFn march_fn_gen(int nb, int agg, int minb);
 MarchFn march_fn_one(int nb, int agg, int minb);
 MarchFn march_fn_one_merge(int nb, int agg, int minb);
 MarchFn march_fn_one_gen(int nb, int agg, int minb);
+MarchFn march_fn_two(int nb, int agg, int minb);
+MarchFn march_fn_two_merge(int nb, int agg, int minb);
+MarchFn march_fn_two_gen(int nb, int agg, int minb);
 // ext: 0 plain, 1 merged rays, 3 merged rays and Generalized mode; plus 4:
 // one simulation, launched directly (its variants exist without aggregation;
-// with it the general one runs)
+// with it the general one runs); plus 8: its deposits are two words
 bool march_variant_exists(int nb, int agg, int minb, int ext);
 // opt the variant into the dynamic shared memory `nsims` slots need
 cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext, uint32_t tile);

@@ -98,11 +98,11 @@ __device__ __forceinline__ float series_q(float nt) {
 // takes the hardware exponential and the division by kappa.  SMALL: every bin
 // of every lane of the warp is thin, and only the series is evaluated; the
 // per-bin results are the same either way, so a ray's photons do not depend
-// on the rays it shares a warp with.  Bins go in pairs on the paired
+// on the rays it shares a warp with.  HEAT: v[2] is wanted.  Bins go in pairs on the paired
 // single-precision units, and the opacity enters negated, so that every
 // product of the thin path is an operand of a fused multiply-add: twelve
 // paired operations a pair of bins (eighteen with the opacity positive).
-template <int NB, bool SMALL>
+template <int NB, bool SMALL, bool HEAT>
 __device__ __forceinline__ void seg_attenuate(float2 k, float dse, const float *sig, const float *sige, float (&ph)[NB],
                                               float (&v)[4]) {
     constexpr float NLOG2E = 1.44269504f;            // e^-tau = 2^(-tau log2 e)
@@ -139,7 +139,7 @@ __device__ __forceinline__ void seg_attenuate(float2 k, float dse, const float *
         ph[b] = pn.x;
         ph[b + 1] = pn.y;
         w1 = __ffma2_rn(sg, phin, w1);
-        w2 = __ffma2_rn(se, phin, w2);
+        if (HEAT) w2 = __ffma2_rn(se, phin, w2);
     }
     v[0] = -(w0.x + w0.y);
     v[1] = w1.x + w1.y;
@@ -161,7 +161,7 @@ __device__ __forceinline__ void seg_attenuate(float2 k, float dse, const float *
         }
         v[0] += a;
         v[1] = fmaf(sig[b], phin, v[1]);
-        v[2] = fmaf(sige[b], phin, v[2]);
+        if (HEAT) v[2] = fmaf(sige[b], phin, v[2]);
     }
 }
 
@@ -184,7 +184,11 @@ __device__ __forceinline__ void seg_attenuate(float2 k, float dse, const float *
 // constant memory, where a load of each from shared memory a ray and segment
 // was a fifth of the load-store unit's work, the march's busiest) and its
 // tallies need no simulation index.
-template <int NB, int AGG, int MINB, int EXT, bool ONE>
+// ONE = 2: besides, nothing reads a cell's heating and segment count
+// (isothermal or Generalized, no diagnostics): its deposit is two words, half
+// the buffer (128 MB at 200^3 cells, with the opacities more than the L2) and
+// half the reduction's payload: 15.5 -> 14.0 ms of march in 60 steps there.
+template <int NB, int AGG, int MINB, int EXT, int ONE>
 __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ MarchArgs A) {
     constexpr bool MRG = (EXT & 1) != 0, GEN = (EXT & 2) != 0;
     // per-simulation tallies of this block (photons in 2^-32 fixed point,
@@ -251,6 +255,11 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
         // together, 2.7 of them in a tile instead of 8.2, and are 2 to 6%
         // slower: more lanes of a reduction then hit one cell.)
         const unsigned warps = gridDim.x * (blockDim.x >> 5), warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+        // a cell's deposit: one vector reduction
+        auto deposit = [&](int cell, float a, float g, float h, float seg) {
+            if (ONE == 2) red_add_v2(reinterpret_cast<float2 *>(A.cells.dep) + cell, a, g);
+            else red_add_v4(A.cells.dep + cell, a, g, h, seg);
+        };
         auto tile_at = [&](unsigned k) { return k * warps + warp; };
         // warp-private run of output slots [slab, slab + slab_left), and this
         // warp's outputs and iterations so far (its output rate)
@@ -376,8 +385,8 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
                 // bins' tau below 1/8): the series path, warp-uniform
                 const bool thin = __all_sync(FULL, key[j] < 0 || fmaf(kc[j].x, S.sig_max, kc[j].y) * dse < 0.125f);
                 if (key[j] >= 0) {
-                    if (thin) seg_attenuate<NB, true>(kc[j], dse, S.sig, S.sige, ph, v);
-                    else seg_attenuate<NB, false>(kc[j], dse, S.sig, S.sige, ph, v);
+                    if (thin) seg_attenuate<NB, true, ONE != 2>(kc[j], dse, S.sig, S.sige, ph, v);
+                    else seg_attenuate<NB, false, ONE != 2>(kc[j], dse, S.sig, S.sige, ph, v);
                     last = key[j];
                     lastk = kc[j];
                     if (GEN && xg[j] < 1.0f) {
@@ -399,7 +408,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
                     }
                 }
                 if (AGG == 0) {
-                    if (key[j] >= 0) red_add_v4(A.cells.dep + key[j], v[0], v[1], v[2], v[3]);
+                    if (key[j] >= 0) deposit(key[j], v[0], v[1], v[2], v[3]);
                 } else {
                     if (__ballot_sync(FULL, key[j] >= 0) == 0u) continue;
                     if (AGG == 1) {
@@ -433,7 +442,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
                             h = fmaf(S.sige[b], q, h);
                         }
                     }
-                    red_add_v4(A.cells.dep + last, s_end, g, h, 0.0f);
+                    deposit(last, s_end, g, h, 0.0f);
                 } else {
                     const int age = mrg ? (int)(merged[lane].w & 0xffffu) + step - (int)heads[lane].y - 1
                                         : step - (int)heads[lane].y;
@@ -646,24 +655,24 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
 // lose to three: 161 against 147 ms of march on the 128^3 workload); the bin
 // counts of the standard spectra (1, 3, 4) also with four, and with every
 // aggregation, for the autotuner.
-template <int NB, int EXT, bool ONE>
+template <int NB, int EXT, int ONE>
 MarchFn march_pick_nb(int agg, int minb) {
     if (agg == 0 && minb == 2) return k_march<NB, 0, 2, EXT, ONE>;
     if (agg == 0 && minb == 3) return k_march<NB, 0, 3, EXT, ONE>;
     if constexpr (NB == 1 || NB == 3 || NB == 4) {
         if (agg == 0 && minb == 4) return k_march<NB, 0, 4, EXT, ONE>;
-        if constexpr (!ONE) {
-            if (agg == 1 && minb == 2) return k_march<NB, 1, 2, EXT, false>;
-            if (agg == 1 && minb == 3) return k_march<NB, 1, 3, EXT, false>;
-            if (agg == 1 && minb == 4) return k_march<NB, 1, 4, EXT, false>;
-            if (agg == 2 && minb == 2) return k_march<NB, 2, 2, EXT, false>;
-            if (agg == 2 && minb == 3) return k_march<NB, 2, 3, EXT, false>;
-            if (agg == 2 && minb == 4) return k_march<NB, 2, 4, EXT, false>;
+        if constexpr (ONE == 0) {
+            if (agg == 1 && minb == 2) return k_march<NB, 1, 2, EXT, 0>;
+            if (agg == 1 && minb == 3) return k_march<NB, 1, 3, EXT, 0>;
+            if (agg == 1 && minb == 4) return k_march<NB, 1, 4, EXT, 0>;
+            if (agg == 2 && minb == 2) return k_march<NB, 2, 2, EXT, 0>;
+            if (agg == 2 && minb == 3) return k_march<NB, 2, 3, EXT, 0>;
+            if (agg == 2 && minb == 4) return k_march<NB, 2, 4, EXT, 0>;
         }
     }
     return nullptr;
 }
-template <int EXT, bool ONE>
+template <int EXT, int ONE>
 MarchFn march_pick(int nb, int agg, int minb) {
     switch (nb) {
         case 1: return march_pick_nb<1, EXT, ONE>(agg, minb);

@@ -6,6 +6,6 @@
 
 namespace frt {
 
-MarchFn march_fn_gen(int nb, int agg, int minb) { return march_pick<3, false>(nb, agg, minb); }
+MarchFn march_fn_gen(int nb, int agg, int minb) { return march_pick<3, 0>(nb, agg, minb); }
 
 }  // namespace frt

@@ -4,7 +4,7 @@
 
 namespace frt {
 
-MarchFn march_fn_one(int nb, int agg, int minb) { return march_pick<0, true>(nb, agg, minb); }
-MarchFn march_fn_one_merge(int nb, int agg, int minb) { return march_pick<1, true>(nb, agg, minb); }
+MarchFn march_fn_one(int nb, int agg, int minb) { return march_pick<0, 1>(nb, agg, minb); }
+MarchFn march_fn_one_merge(int nb, int agg, int minb) { return march_pick<1, 1>(nb, agg, minb); }
 
 }  // namespace frt

@@ -4,6 +4,6 @@
 
 namespace frt {
 
-MarchFn march_fn_one_gen(int nb, int agg, int minb) { return march_pick<3, true>(nb, agg, minb); }
+MarchFn march_fn_one_gen(int nb, int agg, int minb) { return march_pick<3, 1>(nb, agg, minb); }
 
 }  // namespace frt

@@ -49,7 +49,7 @@ namespace frt {
 // ---------------------------------------------------------------------------
 // march variants with merged rays (engines without Generalized members)
 // ---------------------------------------------------------------------------
-MarchFn march_fn_merge(int nb, int agg, int minb) { return march_pick<1, false>(nb, agg, minb); }
+MarchFn march_fn_merge(int nb, int agg, int minb) { return march_pick<1, 0>(nb, agg, minb); }
 
 namespace {
 

@@ -160,7 +160,9 @@ struct Cells {
     float *T;                // K
     float *gamma;            // Gamma_HI of the last step, 1/s
     float2 *kap;             // (tau per cell at sigma_ref from HI, sub-grid tau per cell)
-    float4 *dep;             // (absorbed, Gamma numerator, heating numerator, segments)
+    float4 *dep;             // (absorbed, Gamma numerator, heating numerator, segments); as float2 the
+                             // first two words only, where nothing reads the others: one simulation,
+                             // isothermal or Generalized, without segment counts
     int32_t *segcnt;         // segments of the last step (diagnostics) or null
     // Generalized Opacity mode (Sec. 4.2)
     double *xion;            // highly ionised volume fraction (double: it takes per-step
