@@ -495,7 +495,7 @@ extern "C" flexrt_status flexrt_probe_merge(const flexrt_merge_probe *p, int64_t
     w.grp = grp.p; w.gcm = gcm.p; w.cand = cand.p; w.ckey = ckey.p; w.tgrp = tgrp.p; w.rot = rot.p; w.ndir = ndir;
     w.grp_w = gw; w.hrep = 1; w.lead_slot = lead_slot.p; w.lead_sim = lead_sim.p;
     w.bcnt = bcnt.p; w.bled = bled.p; w.lead_cap = ml;
-    MergeArgs a{dctl.p, dsim.p, dacc.p, 1, {q0, q1}, em, rg, tab, lt, w, nb, mq};
+    MergeArgs a{dctl.p, dsim.p, dacc.p, 1, {q0, q1}, em, rg, tab, lt, w, mq};
     if (launch_merge(a, sms, 0, nullptr) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess)
         return free_fail(FLEXRT_E_CUDA, "probe_merge: kernels failed");
     Ctl hc;

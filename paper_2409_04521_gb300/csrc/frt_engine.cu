@@ -227,7 +227,6 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
         const size_t per = (queue_bytes(cap, cfg_.nb, mrg) + 255) & ~(size_t)255;
         char *base = nullptr;
         if (dev_alloc((void **)&base, 2 * per + 256) != cudaSuccess) return fail(FLEXRT_E_OOM, "ray queue allocation failed");
-        qmem_ = base;
         for (int k = 0; k < 2; ++k) q_[k] = queue_at(base + k * per, cfg_.nb, mrg);
     }
     const long long nc = cfg_.cell_capacity;
@@ -318,7 +317,6 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device_);
     sm_count_ = std::max(sms, 1);
     const int ext = ext_variants();
-    if (!march_variant_exists(cfg_.nb, march_agg_, march_minb_, ext)) { march_agg_ = 0; march_minb_ = 2; }
     CK(march_prepare(cfg_.nb, march_agg_, march_minb_, ms, ext, q_[0].tile));
     const int per_sm = march_max_blocks_per_sm(cfg_.nb, march_agg_, march_minb_, march_threads_, ms, ext, q_[0].tile);
     if (per_sm < 1) return fail(FLEXRT_E_INVALID, "too many simulation slots for one march block");
@@ -739,7 +737,7 @@ flexrt_status Engine::launch_step() {
 // one); stage 2: merge, chemistry and the budget's commit
 flexrt_status Engine::launch_stage(int stage) {
     const int ms = (int)slots_.size();
-    EmitArgs ea{ctl_, sims_, acc_, {q_[0], q_[1]}, qcap_, em_, pixtab_, ltab_, cfg_.nb};
+    EmitArgs ea{ctl_, sims_, acc_, {q_[0], q_[1]}, qcap_, em_, pixtab_, ltab_};
     MarchArgs ma{ctl_, sims_, acc_, ms, {q_[0], q_[1]}, qcap_, em_, cells_, pixtab_, ltab_, march_slab_, {}};
     if (one_sim()) {
         const SimDev &h = slots_[0].h;
@@ -793,7 +791,7 @@ flexrt_status Engine::launch_stage(int stage) {
         return FLEXRT_OK;
     }
     if (merge_built()) {
-        MergeArgs ga{ctl_, sims_, acc_, ms, {q_[0], q_[1]}, em_, rg_, pixtab_, ltab_, mw_, cfg_.nb, qcap_};
+        MergeArgs ga{ctl_, sims_, acc_, ms, {q_[0], q_[1]}, em_, rg_, pixtab_, ltab_, mw_, qcap_};
         tic();
         CK(launch_merge(ga, sm_count_, st_, &mside_));
         toc(3);

@@ -162,7 +162,6 @@ class Engine {
     Ctl *ctl_ = nullptr;
     SimDev *sims_ = nullptr;
     SimAcc *acc_ = nullptr;
-    void *qmem_ = nullptr;
     Queue q_[2]{};
     Cells cells_{};
     Emitters em_{};

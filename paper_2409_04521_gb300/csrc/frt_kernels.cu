@@ -175,9 +175,9 @@ __global__ void k_reset(Ctl *C, SimDev *sims, SimAcc *acc, int nsims) {
 // A warp takes 32 emitters: a lane draws one emitter's rotation, stores it in
 // the ring and sums its photons; then the warp's lanes write the 32 emitters'
 // rays together, one ray a lane, with the rows of its emitter from the lane
-// that drew them.  (One thread an emitter wrote its 12 rays one after another,
-// ten scattered words each: 25 us a step at 2e4 emitters and 17 us for the
-// single emitter of a Stromgren sphere.)
+// that drew them.  Bound by the chain control words, list, cell, constants,
+// draw.  (One thread an emitter wrote its 12 rays one after another, ten
+// scattered words each: 25 us a step at 2e4 emitters, now 13.)
 __global__ void __launch_bounds__(128) k_emit(EmitArgs A) {
     Ctl *C = A.ctl;
     if (C->err) return;

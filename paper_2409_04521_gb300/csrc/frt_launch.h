@@ -14,7 +14,6 @@ struct EmitArgs {
     Emitters em;
     const int4 *pixtab;
     int ltab;
-    int nb;
 };
 
 // The per-simulation constants the march needs, staged in shared
@@ -54,7 +53,6 @@ struct MergeArgs {
     const int4 *pixtab;
     int ltab;
     MergeWork w;
-    int nbq;                 // photon bins of the queue layout
     long long cap;           // queue slots (merged rays are appended)
 };
 
