@@ -628,11 +628,16 @@ __device__ __forceinline__ void red_add_v4(float4 *addr, float a, float b, float
 // ---------------------------------------------------------------------------
 // Bulk copies global -> shared with an mbarrier (sizes and addresses multiples
 // of 16 bytes).  One thread announces the bytes and starts the copy; every
-// reader waits for the barrier's phase.
+// reader waits for the barrier's phase.  A thread whose ordinary stores to the
+// destination come before the copy fences them, then meets the copying thread
+// at a barrier.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(unsigned bar, unsigned arrivals) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(arrivals) : "memory");
+}
+__device__ __forceinline__ void fence_proxy_async() {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 __device__ __forceinline__ void bulk_load(unsigned dst, const void *src, unsigned bytes, unsigned bar) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");

@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
     if (lane == 0) {
         mbar_init(bars_s, 1);
         mbar_init(bars_s + 8, 1);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        fence_proxy_async();
     }
     __syncthreads();
     Ctl *C = A.ctl;
@@ -583,6 +583,9 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
 #pragma unroll
                         for (int b = 0; b < NB; ++b) w[2 + b] = __float_as_uint(ph[b] * scale);
                         store_tail<NB, false>(rec, lane, w);
+                        // these stores come before the copy that refills the
+                        // tile, which goes through another proxy
+                        fence_proxy_async();
                     }
                     __syncwarp();
                     const unsigned all = (unsigned)__popc(grp) << (2 * mm);
