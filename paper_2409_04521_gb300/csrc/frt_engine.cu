@@ -1282,10 +1282,16 @@ flexrt_status Engine::load_state(int s, const void *buf, int64_t bytes) {
     size_t tot = sizeof(StateHeader);
     for (auto &p : parts) tot += p.second;
     if ((int64_t)tot != bytes) return fail(FLEXRT_E_INVALID, "checkpoint size does not match its header");
+    // everything in the engine's stream: a copy from pageable memory in another
+    // one may return before its bytes have reached the device, and the kernel
+    // below would not wait for them
     CK(cudaStreamSynchronize(st_));
+    auto up = [&](void *dst, const void *from, size_t n) {
+        return cudaMemcpyAsync(dst, from, n, cudaMemcpyHostToDevice, st_);
+    };
     const char *src = (const char *)buf + sizeof(h);
     for (auto &p : parts) {
-        if (p.second) CK(cudaMemcpy(p.first, src, p.second, cudaMemcpyHostToDevice));
+        if (p.second) CK(up(p.first, src, p.second));
         src += p.second;
     }
     CK(launch_queue_words(q_[0], merge_built(), nray, reinterpret_cast<uint32_t *>(q_[1].base), true, st_));
@@ -1293,10 +1299,10 @@ flexrt_status Engine::load_state(int s, const void *buf, int64_t bytes) {
     const long long cnt[2] = {nray, 0};
     const int32_t par_err[2] = {0, 0};
     static_assert(offsetof(Ctl, err) == offsetof(Ctl, par) + sizeof(int32_t), "ctl layout");
-    CK(cudaMemcpy(ctl_->cnt, cnt, sizeof(cnt), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(&ctl_->par, par_err, sizeof(par_err), cudaMemcpyHostToDevice));
+    CK(up(ctl_->cnt, cnt, sizeof(cnt)));
+    CK(up(&ctl_->par, par_err, sizeof(par_err)));
     sl->h.step = (int32_t)h.step;
-    CK(cudaMemcpy((char *)(sims_ + s) + offsetof(SimDev, step), &sl->h.step, sizeof(int32_t), cudaMemcpyHostToDevice));
+    CK(up((char *)(sims_ + s) + offsetof(SimDev, step), &sl->h.step, sizeof(int32_t)));
     latched_ = FLEXRT_OK;
     seq_seen_ = h_status_[3];
     if (h.dt > 0.0) {
