@@ -293,7 +293,9 @@ __global__ void __launch_bounds__(256) k_mfind(MergeArgs A, int pass) {
     if (inc - c < K && K <= inc) { s_seg = SEGS - 1 - t; s_above = inc - c; }
     __syncthreads();
     c = hist[256 * s_seg + 255 - t];
-    inc = s_above + block_incl_scan(c, s_w);
+    // read before the scan's barriers: one thread writes it after them
+    const unsigned long long seg_above = s_above;
+    inc = seg_above + block_incl_scan(c, s_w);
     if (inc - c < K && K <= inc) { s_bin = 256 * s_seg + 255 - t; s_above = inc - c; }
     __syncthreads();
     if (t == 0) {
