@@ -317,7 +317,7 @@ flexrt_status Engine::init(const EngineConfig &cfg) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device_);
     sm_count_ = std::max(sms, 1);
     const int ext = ext_variants();
-    CK(march_prepare(cfg_.nb, march_agg_, march_minb_, ms, ext, q_[0].tile));
+    CK(march_prepare(cfg_.nb, march_agg_, march_minb_, ext));
     const int per_sm = march_max_blocks_per_sm(cfg_.nb, march_agg_, march_minb_, march_threads_, ms, ext, q_[0].tile);
     if (per_sm < 1) return fail(FLEXRT_E_INVALID, "too many simulation slots for one march block");
     march_blocks_ = sm_count_ * std::max(per_sm, 1);
@@ -1122,7 +1122,7 @@ flexrt_status Engine::set_launch(int agg, int minb, int blocks_per_sm, int threa
     if (!march_variant_exists(cfg_.nb, agg, minb, ext_variants()) || blocks_per_sm < 0 || blocks_per_sm > 32 ||
         (threads != 128 && threads != 256) || slab < 32 || slab > 4096)
         return fail(FLEXRT_E_INVALID, "march kernel variant not built or launch shape out of range");
-    CK(march_prepare(cfg_.nb, agg, minb, (int)slots_.size(), ext_variants(), q_[0].tile));
+    CK(march_prepare(cfg_.nb, agg, minb, ext_variants()));
     const int lim = march_max_blocks_per_sm(cfg_.nb, agg, minb, threads, (int)slots_.size(), ext_variants(), q_[0].tile);
     if (lim < 1) return fail(FLEXRT_E_INVALID, "variant cannot be resident");
     const int bps = blocks_per_sm == 0 ? lim : std::min(blocks_per_sm, lim);

@@ -830,14 +830,25 @@ static MarchFn march_fn(int nb, int agg, int minb, int ext) {
     }
 }
 bool march_variant_exists(int nb, int agg, int minb, int ext) { return march_fn(nb, agg, minb, ext) != nullptr; }
-cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext, uint32_t tile) {
+// Always the device's whole opt-in limit less the kernel's static part, never
+// this engine's own need: the attribute is the process's, so a smaller engine
+// would take a larger one's away, and the limit without it counts the static
+// part too.  A launch still asks for what its slots need.
+static cudaError_t raise_shared_limit(MarchFn f) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, f);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+}
+cudaError_t march_prepare(int nb, int agg, int minb, int ext) {
     MarchFn f = march_fn(nb, agg, minb, ext);
     if (!f) return cudaErrorInvalidValue;
-    const size_t sh = march_shared_bytes(nsims, tile, 256);
-    if (sh <= 48 * 1024) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    cudaError_t e = raise_shared_limit(f);
     MarchFn two = ext & 4 ? march_fn(nb, agg, minb, ext | 8) : f;      // a launch may take either
-    if (e == cudaSuccess && two != f) e = cudaFuncSetAttribute(two, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    if (e == cudaSuccess && two != f) e = raise_shared_limit(two);
     return e;
 }
 cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int blocks, int threads, cudaStream_t st,

@@ -96,8 +96,8 @@ MarchFn march_fn_two_gen(int nb, int agg, int minb);
 // one simulation, launched directly (its variants exist without aggregation;
 // with it the general one runs); plus 8: its deposits are two words
 bool march_variant_exists(int nb, int agg, int minb, int ext);
-// opt the variant into the dynamic shared memory `nsims` slots need
-cudaError_t march_prepare(int nb, int agg, int minb, int nsims, int ext, uint32_t tile);
+// opt the variant into all the dynamic shared memory a block may have
+cudaError_t march_prepare(int nb, int agg, int minb, int ext);
 cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int blocks, int threads, cudaStream_t st,
                          int ext);
 int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, int ext, uint32_t tile);
