@@ -191,7 +191,8 @@ flexrt_status flexrt_step(flexrt_ctx *ctx, double dt_s);
  * of length dt_s; stage 2 (dt_s ignored) the merge, the chemistry and the
  * commit.  Between the two, flexrt_get_rays and flexrt_get_rays_merged
  * return the march's output, before merging; flexrt_step, the checkpoint
- * calls and another stage 1 return FLEXRT_E_STATE. */
+ * calls and another stage 1 return FLEXRT_E_STATE, and flexrt_reset drops the
+ * open step. */
 flexrt_status flexrt_step_stage(flexrt_ctx *ctx, double dt_s, int32_t stage);
 
 /* Wait for all enqueued work; returns a latched device error if any.  No

@@ -906,6 +906,7 @@ flexrt_status Engine::reset_all() {
     CK(cudaStreamSynchronize(st_));
     const bool failed = latched_ != FLEXRT_OK || h_status_[2] != 0 || mid_step_;
     latched_ = FLEXRT_OK;
+    mid_step_ = false;                           // an open step is dropped
     seq_seen_ = h_status_[3];                    // what ended before is not reported any more
     if (failed && mwmem_) {
         // a step that failed may have stopped inside the merge, with groups

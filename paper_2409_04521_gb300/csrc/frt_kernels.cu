@@ -166,6 +166,7 @@ __global__ void k_reset(Ctl *C, SimDev *sims, SimAcc *acc, int nsims) {
         C->cnt[0] = C->cnt[1] = 0;
         C->par = 0;
         C->err = 0;
+        C->merged = C->far = 0;                    // a step dropped between its stages may have set them
     }
 }
 
