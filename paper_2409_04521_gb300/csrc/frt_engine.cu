@@ -822,7 +822,7 @@ bool Engine::graph_now() {
 
 flexrt_status Engine::run_graph() {
     if (graph_dirty_) {
-        CK(cudaStreamSynchronize(st_));
+        // (an executable graph in flight is freed when it has run)
         if (graph_) { cudaGraphExecDestroy(graph_); graph_ = nullptr; }
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamBeginCapture(st_, cudaStreamCaptureModeThreadLocal);
