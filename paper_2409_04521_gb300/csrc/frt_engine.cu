@@ -728,14 +728,14 @@ static cudaEvent_t take_event(std::vector<cudaEvent_t> &pool) {
     return e;
 }
 
-flexrt_status Engine::launch_step() {
-    flexrt_status r = launch_stage(1);
-    return r == FLEXRT_OK ? launch_stage(2) : r;
+flexrt_status Engine::launch_step(Sink to) {
+    flexrt_status r = launch_stage(1, to);
+    return r == FLEXRT_OK ? launch_stage(2, to) : r;
 }
 
 // stage 1: emission and the marches (the trial passes and the committed
 // one); stage 2: merge, chemistry and the budget's commit
-flexrt_status Engine::launch_stage(int stage) {
+flexrt_status Engine::launch_stage(int stage, Sink &to) {
     const int ms = (int)slots_.size();
     EmitArgs ea{ctl_, sims_, acc_, {q_[0], q_[1]}, qcap_, em_, pixtab_, ltab_};
     MarchArgs ma{ctl_, sims_, acc_, ms, {q_[0], q_[1]}, qcap_, em_, cells_, pixtab_, ltab_, march_slab_, {}};
@@ -754,7 +754,7 @@ flexrt_status Engine::launch_stage(int stage) {
         }
     }
     ChemArgs ca{ctl_, sims_, acc_, ms, cells_, rg_, dep_two_ ? 1 : 0, 1, reinterpret_cast<uint4 *>(h_status_)};
-    const bool prof = profiling_ && !cfg_.use_graph;      // (a profiled single simulation is never replayed)
+    const bool prof = profiling_ && !to.graph;
     cudaEvent_t e0 = nullptr;
     auto tic = [&]() {
         if (prof) { e0 = take_event(ev_pool_); cudaEventRecord(e0, st_); }
@@ -764,7 +764,7 @@ flexrt_status Engine::launch_stage(int stage) {
     };
     if (stage == 1) {
         tic();
-        CK(launch_emit(ea, emit_blocks_, st_));
+        CK(launch_emit(ea, emit_blocks_, to));
         toc(0);
         // passes of the Gamma - <n_HI> iteration before the committed one: march,
         // trial chemistry (opacity of the time-averaged state), reset of the
@@ -774,30 +774,30 @@ flexrt_status Engine::launch_stage(int stage) {
             if (sl.used) iters = std::max(iters, (int)sl.h.gamma_iters);
         for (int it = 0; it + 1 < iters; ++it) {
             tic();
-            CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, st_,
+            CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, to,
                             ext_variants() | (dep_two_ ? 8 : 0)));
             toc(1);
             ChemArgs ct = ca;
             ct.final_pass = 0;
             tic();
-            CK(launch_chem(ct, chem_blocks_, st_));
+            CK(launch_chem(ct, chem_blocks_, to));
             toc(2);
-    }
+        }
         tic();
-        CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, st_,
+        CK(launch_march(ma, cfg_.nb, march_agg_, march_minb_, march_blocks_, march_threads_, to,
                             ext_variants() | (dep_two_ ? 8 : 0)));
         toc(1);
-        if (far_possible_) CK(launch_far(ea, sm_count_, st_));
+        if (far_possible_) CK(launch_far(ea, sm_count_, to));
         return FLEXRT_OK;
     }
     if (merge_built()) {
         MergeArgs ga{ctl_, sims_, acc_, ms, {q_[0], q_[1]}, em_, rg_, pixtab_, ltab_, mw_, qcap_};
         tic();
-        CK(launch_merge(ga, sm_count_, st_, &mside_));
+        CK(launch_merge(ga, sm_count_, to, &mside_));
         toc(3);
     }
     tic();
-    CK(launch_chem(ca, chem_blocks_, st_));
+    CK(launch_chem(ca, chem_blocks_, to));
     toc(2);
     return FLEXRT_OK;
 }
@@ -817,29 +817,45 @@ bool Engine::graph_now() {
     if (graph_dirty_ && direct_steps_ < GRAPH_AFTER) { ++direct_steps_; return false; }
     // a caller that captures the stream itself gets the kernels
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    return cudaStreamIsCapturing(st_, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st_, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cs == cudaStreamCaptureStatusNone;
+}
+
+// The step's kernels as an executable graph in place of the present one (an
+// executable graph in flight is freed when it has run).
+cudaError_t Engine::make_graph(flexrt_status &built) {
+    Sink to;
+    cudaError_t e = cudaGraphCreate(&to.graph, 0);
+    if (e != cudaSuccess) return e;
+    built = launch_step(to);
+    cudaGraphExec_t x = nullptr;
+    if (built == FLEXRT_OK) e = cudaGraphInstantiate(&x, to.graph, 0);
+    cudaGraphDestroy(to.graph);
+    if (built != FLEXRT_OK || e != cudaSuccess) return e;
+    if (graph_) cudaGraphExecDestroy(graph_);
+    graph_ = x;
+    graph_dirty_ = false;
+    return cudaSuccess;
 }
 
 flexrt_status Engine::run_graph() {
     if (graph_dirty_) {
-        // (an executable graph in flight is freed when it has run)
-        if (graph_) { cudaGraphExecDestroy(graph_); graph_ = nullptr; }
-        cudaGraph_t g = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(st_, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess && !cfg_.use_graph) {
-            cudaGetLastError();                  // a stream that cannot be captured: direct launches
+        // none of its calls touches a stream or waits: allowed beside a capture
+        // that another host thread has open, and not to end it
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        flexrt_status built = FLEXRT_OK;
+        const cudaError_t e = make_graph(built);
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (built != FLEXRT_OK || e != cudaSuccess) {
+            if (cfg_.use_graph) return built != FLEXRT_OK ? built : cuda(e, "step graph");
+            cudaGetLastError();                  // no graph: direct launches
             graph_off_ = true;
-            return launch_step();
+            return launch_step(on_stream());
         }
-        CK(e);
-        flexrt_status r = launch_step();
-        e = cudaStreamEndCapture(st_, &g);
-        if (r != FLEXRT_OK) { if (g) cudaGraphDestroy(g); return r; }
-        if (e != cudaSuccess) return cuda(e, "graph capture");
-        e = cudaGraphInstantiate(&graph_, g, 0);
-        cudaGraphDestroy(g);
-        if (e != cudaSuccess) return cuda(e, "graph instantiate");
-        graph_dirty_ = false;
     }
     CK(cudaGraphLaunch(graph_, st_));
     return FLEXRT_OK;
@@ -850,7 +866,7 @@ flexrt_status Engine::step() {
     flexrt_status s = poll();
     if (s != FLEXRT_OK) return s;
     free_retired();
-    s = graph_now() ? run_graph() : launch_step();
+    s = graph_now() ? run_graph() : launch_step(on_stream());
     if (s != FLEXRT_OK) return s;
     ++steps_taken_;
     for (auto &sl : slots_)
@@ -867,14 +883,16 @@ flexrt_status Engine::step_stage(int stage) {
         if (mid_step_) return fail(FLEXRT_E_STATE, "a staged step is already open");
         flexrt_status s = poll();
         if (s != FLEXRT_OK) return s;
-        s = launch_stage(1);
+        Sink to = on_stream();
+        s = launch_stage(1, to);
         if (s != FLEXRT_OK) return s;
         mid_step_ = true;
         return FLEXRT_OK;
     }
     if (stage != 2 || !mid_step_) return fail(FLEXRT_E_STATE, "no staged step to finish");
     mid_step_ = false;
-    flexrt_status s = launch_stage(2);
+    Sink to = on_stream();
+    flexrt_status s = launch_stage(2, to);
     if (s != FLEXRT_OK) return s;
     ++steps_taken_;
     for (auto &sl : slots_)

@@ -147,8 +147,9 @@ class Engine {
     flexrt_status grow_emitters(int need);
     flexrt_status upload_lists();             // active emitters, cell ranges, counters
     flexrt_status poll();
-    flexrt_status launch_step();
-    flexrt_status launch_stage(int stage);
+    Sink on_stream() const { Sink s; s.st = st_; return s; }
+    flexrt_status launch_step(Sink to);
+    flexrt_status launch_stage(int stage, Sink &to);
     flexrt_status read_acc(int slot, SimAcc &a);
     void free_retired();
 
@@ -202,14 +203,15 @@ class Engine {
 
     cudaGraphExec_t graph_ = nullptr;
     bool graph_dirty_ = true;
-    bool graph_off_ = false;                // the stream cannot be captured
+    bool graph_off_ = false;                // a graph could not be made
     int direct_steps_ = 0;                  // steps launched directly since the graph became stale
     // a step replayed from a graph: batches that ask for it, and single
-    // simulations once they have taken GRAPH_AFTER steps directly (capturing
+    // simulations once they have taken GRAPH_AFTER steps directly (making
     // and instantiating it costs about as much host time as that many)
     static constexpr int GRAPH_AFTER = 8;
     void graph_stale() { graph_dirty_ = true; direct_steps_ = 0; }
     bool graph_now();
+    cudaError_t make_graph(flexrt_status &built);
     flexrt_status run_graph();
     bool mid_step_ = false;                 // between the two stages of a staged step
 

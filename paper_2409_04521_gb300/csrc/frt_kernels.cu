@@ -11,7 +11,7 @@
 //              of Eq. 12 (single precision), kappa for the next step,
 //              and the commit of the step's photon budget by its last block.
 // All launches are sized on the host from capacities only; counts are read
-// from device memory, so the same launches can be replayed in a CUDA graph.
+// from device memory, so the same launches can be replayed from a CUDA graph.
 #include <algorithm>
 #include <cstdio>
 #include "frt_march.cuh"
@@ -794,14 +794,8 @@ cudaError_t launch_reset(Ctl *c, SimDev *sims, SimAcc *acc, int nsims, cudaStrea
     k_reset<<<1, 256, 0, st>>>(c, sims, acc, nsims);
     return cudaGetLastError();
 }
-cudaError_t launch_emit(const EmitArgs &a, int blocks, cudaStream_t st) {
-    k_emit<<<blocks, 128, 0, st>>>(a);
-    return cudaGetLastError();
-}
-cudaError_t launch_far(const EmitArgs &a, int blocks, cudaStream_t st) {
-    k_far<<<blocks, 256, 0, st>>>(a);
-    return cudaGetLastError();
-}
+cudaError_t launch_emit(const EmitArgs &a, int blocks, Sink &to) { return enqueue(to, k_emit, blocks, 128, 0, a); }
+cudaError_t launch_far(const EmitArgs &a, int blocks, Sink &to) { return enqueue(to, k_far, blocks, 256, 0, a); }
 cudaError_t launch_queue_words(const Queue &q, bool merged, long long n, uint32_t *words, bool join,
                                cudaStream_t st) {
     if (n < 1) return cudaSuccess;
@@ -852,12 +846,10 @@ cudaError_t march_prepare(int nb, int agg, int minb, int ext) {
     if (e == cudaSuccess && two != f) e = raise_shared_limit(two);
     return e;
 }
-cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int blocks, int threads, cudaStream_t st,
-                         int ext) {
+cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int blocks, int threads, Sink &to, int ext) {
     MarchFn f = march_fn(nb, agg, minb, ext);
     if (!f) return cudaErrorInvalidValue;
-    f<<<blocks, threads, march_shared_bytes(a.nsims, a.q[0].tile, threads), st>>>(a);
-    return cudaGetLastError();
+    return enqueue(to, f, blocks, threads, march_shared_bytes(a.nsims, a.q[0].tile, threads), a);
 }
 int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, int ext, uint32_t tile) {
     MarchFn f = march_fn(nb, agg, minb, ext);
@@ -875,10 +867,8 @@ int chem_max_blocks_per_sm(int nsims) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_chem, 256, chem_shared_bytes(nsims));
     return n;
 }
-cudaError_t launch_chem(const ChemArgs &a, int blocks, cudaStream_t st) {
-    const size_t sh = chem_shared_bytes(a.nsims);
-    k_chem<<<blocks, 256, sh, st>>>(a);
-    return cudaGetLastError();
+cudaError_t launch_chem(const ChemArgs &a, int blocks, Sink &to) {
+    return enqueue(to, k_chem, blocks, 256, chem_shared_bytes(a.nsims), a);
 }
 cudaError_t launch_probe_pixvec(int level, long long p0, long long n, int32_t *out, cudaStream_t st) {
     int blocks = (int)((n + 255) / 256);

@@ -1,6 +1,7 @@
 // frt_launch.h -- kernel argument blocks and launchers (host side).
 #pragma once
 #include <string>
+#include <tuple>
 #include "frt_types.h"
 
 namespace frt {
@@ -68,15 +69,47 @@ struct ChemArgs {
     uint4 *status;           // host memory: the last step's queue slots in use (x, y), error word, number
 };
 
+// Where a step's kernels go: onto a stream, or into a graph as nodes that run
+// one after another.  A graph is built from nodes, not by capturing a stream:
+// a capture nobody asked for makes other host threads' calls fail (their use
+// of the legacy stream, or a wait for the device), and theirs end it.
+struct Sink {
+    cudaStream_t st = nullptr;
+    cudaGraph_t graph = nullptr;             // null: launched on st
+    cudaGraphNode_t last[2] = {};            // the nodes the next one waits for
+    int nlast = 0;
+};
+template <typename... P, typename... A>
+cudaError_t enqueue(Sink &s, void (*k)(P...), int blocks, int threads, size_t shared, const A &...a) {
+    std::tuple<P...> args(a...);
+    return std::apply(
+        [&](auto &...x) {
+            void *ptr[] = {const_cast<void *>(static_cast<const void *>(&x))...};
+            const void *f = reinterpret_cast<const void *>(k);
+            if (!s.graph) return cudaLaunchKernel(f, dim3(blocks), dim3(threads), ptr, shared, s.st);
+            cudaKernelNodeParams p{};
+            p.func = const_cast<void *>(f);
+            p.gridDim = dim3(blocks);
+            p.blockDim = dim3(threads);
+            p.sharedMemBytes = (unsigned)shared;
+            p.kernelParams = ptr;
+            cudaGraphNode_t n = nullptr;
+            const cudaError_t e = cudaGraphAddKernelNode(&n, s.graph, s.last, s.nlast, &p);
+            if (e == cudaSuccess) { s.last[0] = n; s.nlast = 1; }
+            return e;
+        },
+        args);
+}
+
 // message of the last failed call that has no context (this host thread)
 void set_free_error(const std::string &msg);
 
 cudaError_t launch_pixtab(int4 *tab, int L, cudaStream_t st);
 cudaError_t launch_init_cells(const SimDev *sims, int sim, Cells c, long long ncell, cudaStream_t st);
 cudaError_t launch_reset(Ctl *c, SimDev *sims, SimAcc *acc, int nsims, cudaStream_t st);
-cudaError_t launch_emit(const EmitArgs &a, int blocks, cudaStream_t st);
+cudaError_t launch_emit(const EmitArgs &a, int blocks, Sink &to);
 // after a march: directions of children beyond the pixel table
-cudaError_t launch_far(const EmitArgs &a, int blocks, cudaStream_t st);
+cudaError_t launch_far(const EmitArgs &a, int blocks, Sink &to);
 // a queue's first n records to (join: from) one array of n words per word of the record
 cudaError_t launch_queue_words(const Queue &q, bool merged, long long n, uint32_t *words, bool join,
                                cudaStream_t st);
@@ -98,12 +131,11 @@ MarchFn march_fn_two_gen(int nb, int agg, int minb);
 bool march_variant_exists(int nb, int agg, int minb, int ext);
 // opt the variant into all the dynamic shared memory a block may have
 cudaError_t march_prepare(int nb, int agg, int minb, int ext);
-cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int blocks, int threads, cudaStream_t st,
-                         int ext);
+cudaError_t launch_march(const MarchArgs &a, int nb, int agg, int minb, int blocks, int threads, Sink &to, int ext);
 int march_max_blocks_per_sm(int nb, int agg, int minb, int threads, int nsims, int ext, uint32_t tile);
 // blocks of the chemistry kernel that an SM holds at once
 int chem_max_blocks_per_sm(int nsims);
-cudaError_t launch_chem(const ChemArgs &a, int blocks, cudaStream_t st);
+cudaError_t launch_chem(const ChemArgs &a, int blocks, Sink &to);
 // the merge step (Sec. 3.3) between the march and the chemistry
 // a second stream for the merge's independent rotation pass, with the events
 // that fork it from the step's stream and join it back
@@ -111,7 +143,7 @@ struct MergeSide {
     cudaStream_t st;
     cudaEvent_t fork, join;
 };
-cudaError_t launch_merge(const MergeArgs &a, int sm_count, cudaStream_t st, const MergeSide *side);
+cudaError_t launch_merge(const MergeArgs &a, int sm_count, Sink &to, const MergeSide *side);
 cudaError_t launch_probe_merge_pixel(int level, long long n, const int32_t *d, const int32_t *Rq, bool per_ray,
                                      uint32_t *out, cudaStream_t st);
 cudaError_t launch_probe_pixvec(int level, long long p0, long long n, int32_t *out, cudaStream_t st);

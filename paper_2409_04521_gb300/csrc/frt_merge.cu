@@ -786,35 +786,39 @@ __global__ void k_probe_merge_pixel(int level, long long n, const int32_t *d, co
     }
 }
 
-cudaError_t launch_merge(const MergeArgs &a, int sm_count, cudaStream_t st, const MergeSide *side) {
+cudaError_t launch_merge(const MergeArgs &a, int sm_count, Sink &to, const MergeSide *side) {
     const int rblocks = std::min(sm_count * 16, MERGE_MAX_BLOCKS);
     const size_t rng_sh = (size_t)(2 * a.nsims + 1) * sizeof(long long) + (size_t)a.nsims * sizeof(int);
-    // the merge spheres' rotations depend on no pass of the merge: with a
-    // side stream they are drawn (integer-bound) while the selection passes
-    // (memory-bound) run, and the group pass waits for both
+    // the merge spheres' rotations depend on no pass of the merge: beside it
+    // (on the side stream, or as a branch of the graph) they are drawn
+    // (integer-bound) while the selection passes (memory-bound) run, and the
+    // group pass waits for both
     cudaError_t e = cudaSuccess;
-    if (side) {
-        e = cudaEventRecord(side->fork, st);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(side->st, side->fork, 0);
-        if (e != cudaSuccess) return e;
-        k_mrot<<<rblocks, 256, rng_sh, side->st>>>(a);
-        e = cudaEventRecord(side->join, side->st);
-        if (e != cudaSuccess) return e;
-    } else {
-        k_mrot<<<rblocks, 256, rng_sh, st>>>(a);
+    auto run = [&](Sink &s, auto k, int blocks, int threads, size_t shared, auto... x) {
+        if (e == cudaSuccess) e = enqueue(s, k, blocks, threads, shared, a, x...);
+    };
+    Sink rot = to;
+    const bool fork = side && !to.graph;
+    if (fork) {
+        rot.st = side->st;
+        e = cudaEventRecord(side->fork, to.st);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(rot.st, side->fork, 0);
     }
-    k_mhist1<<<rblocks, 256, 0, st>>>(a);
-    k_mreduce<<<std::min(a.nsims * SEGS, rblocks), 256, 0, st>>>(a, 1);
-    k_mfind<<<a.nsims, 256, 0, st>>>(a, 1);
-    k_mhist2<<<rblocks, 256, 0, st>>>(a);
-    k_mreduce<<<std::min(a.nsims * SEGS, rblocks), 256, 0, st>>>(a, 2);
-    k_mfind<<<a.nsims, 256, 0, st>>>(a, 2);
-    if (side && (e = cudaStreamWaitEvent(st, side->join, 0)) != cudaSuccess) return e;
-    k_mgroup<<<rblocks, 256, 0, st>>>(a);
-    k_mweight<<<rblocks, 256, (size_t)a.nsims * sizeof(uint32_t), st>>>(a);
-    k_mscan<<<1, 1024, 0, st>>>(a, rblocks);
-    k_memit<<<rblocks, 256, 0, st>>>(a);
-    return cudaGetLastError();
+    run(rot, k_mrot, rblocks, 256, rng_sh);
+    if (fork && e == cudaSuccess) e = cudaEventRecord(side->join, rot.st);
+    run(to, k_mhist1, rblocks, 256, 0);
+    run(to, k_mreduce, std::min(a.nsims * SEGS, rblocks), 256, 0, 1);
+    run(to, k_mfind, a.nsims, 256, 0, 1);
+    run(to, k_mhist2, rblocks, 256, 0);
+    run(to, k_mreduce, std::min(a.nsims * SEGS, rblocks), 256, 0, 2);
+    run(to, k_mfind, a.nsims, 256, 0, 2);
+    if (fork && e == cudaSuccess) e = cudaStreamWaitEvent(to.st, side->join, 0);
+    if (to.graph && e == cudaSuccess) to.last[to.nlast++] = rot.last[0];
+    run(to, k_mgroup, rblocks, 256, 0);
+    run(to, k_mweight, rblocks, 256, (size_t)a.nsims * sizeof(uint32_t));
+    run(to, k_mscan, 1, 1024, 0, rblocks);
+    run(to, k_memit, rblocks, 256, 0);
+    return e;
 }
 
 cudaError_t launch_probe_merge_pixel(int level, long long n, const int32_t *d, const int32_t *Rq, bool per_ray,
