@@ -695,17 +695,13 @@ flexrt_status Engine::set_dt(int s, double dt) {
     return FLEXRT_OK;
 }
 
-// the outcome of the last step the GPU has ended, if it is a new one (the
-// GPU writes the four words as one 16-byte store; after a stream
-// synchronisation this is the last step enqueued)
+// the outcome of the last step the GPU has ended (after a stream
+// synchronisation, of the last one enqueued).  An error stays in its word
+// until clear_outcome: every step after a failed one writes it again.
 flexrt_status Engine::poll() {
     if (latched_ != FLEXRT_OK) return latched_;
-    const uint32_t seq = __atomic_load_n(h_status_ + 3, __ATOMIC_ACQUIRE);
-    if (seq == seq_seen_) return FLEXRT_OK;
-    seq_seen_ = seq;
-    const uint32_t v = __atomic_load_n(h_status_ + 2, __ATOMIC_RELAXED);
-    q_used_ = (long long)__atomic_load_n(h_status_, __ATOMIC_RELAXED) |
-              (long long)__atomic_load_n(h_status_ + 1, __ATOMIC_RELAXED) << 32;
+    q_used_ = (long long)__atomic_load_n(h_status_, __ATOMIC_RELAXED);
+    const uint32_t v = __atomic_load_n(h_status_ + 1, __ATOMIC_RELAXED);
     if (v) {
         latched_ = FLEXRT_E_CAPACITY;
         if (v & 1) err_ = "ray queue capacity exceeded; state kept at the last complete step";
@@ -715,6 +711,13 @@ flexrt_status Engine::poll() {
         else err_ = "ray crossed more than four cells in one step (internal bound)";
     }
     return latched_;
+}
+
+// a run starts anew: what ended before is not reported any more (nothing that
+// was enqueued is still running)
+void Engine::clear_outcome() {
+    latched_ = FLEXRT_OK;
+    h_status_[0] = h_status_[1] = 0;
 }
 
 static cudaEvent_t take_event(std::vector<cudaEvent_t> &pool) {
@@ -753,7 +756,7 @@ flexrt_status Engine::launch_stage(int stage, Sink &to) {
             if (b < h.nb) o.sig_max = std::max(o.sig_max, h.sig[b]);
         }
     }
-    ChemArgs ca{ctl_, sims_, acc_, ms, cells_, rg_, dep_two_ ? 1 : 0, 1, reinterpret_cast<uint4 *>(h_status_)};
+    ChemArgs ca{ctl_, sims_, acc_, ms, cells_, rg_, dep_two_ ? 1 : 0, 1, reinterpret_cast<uint2 *>(h_status_)};
     const bool prof = profiling_ && !to.graph;
     cudaEvent_t e0 = nullptr;
     auto tic = [&]() {
@@ -922,10 +925,9 @@ flexrt_status Engine::retire(int s) {
 
 flexrt_status Engine::reset_all() {
     CK(cudaStreamSynchronize(st_));
-    const bool failed = latched_ != FLEXRT_OK || h_status_[2] != 0 || mid_step_;
-    latched_ = FLEXRT_OK;
+    const bool failed = latched_ != FLEXRT_OK || h_status_[1] != 0 || mid_step_;
+    clear_outcome();
     mid_step_ = false;                           // an open step is dropped
-    seq_seen_ = h_status_[3];                    // what ended before is not reported any more
     if (failed && mwmem_) {
         // a step that failed may have stopped inside the merge, with groups
         // not cleared: clear the whole merge scratch
@@ -1322,8 +1324,7 @@ flexrt_status Engine::load_state(int s, const void *buf, int64_t bytes) {
     CK(up(&ctl_->par, par_err, sizeof(par_err)));
     sl->h.step = (int32_t)h.step;
     CK(up((char *)(sims_ + s) + offsetof(SimDev, step), &sl->h.step, sizeof(int32_t)));
-    latched_ = FLEXRT_OK;
-    seq_seen_ = h_status_[3];
+    clear_outcome();
     if (h.dt > 0.0) {
         flexrt_status r = set_dt(s, h.dt);
         if (r != FLEXRT_OK) return r;

@@ -147,6 +147,7 @@ class Engine {
     flexrt_status grow_emitters(int need);
     flexrt_status upload_lists();             // active emitters, cell ranges, counters
     flexrt_status poll();
+    void clear_outcome();
     Sink on_stream() const { Sink s; s.st = st_; return s; }
     flexrt_status launch_step(Sink to);
     flexrt_status launch_stage(int stage, Sink &to);
@@ -183,10 +184,9 @@ class Engine {
     int march_agg_ = 0, march_minb_ = 3, march_blocks_ = 1, march_threads_ = 256, march_slab_ = OUT_SLAB;
     int chem_blocks_ = 1, emit_blocks_ = 1, sm_count_ = 1;
 
-    // the last ended step's outcome, written by the GPU (ChemArgs::status),
-    // and the number of the last one seen
+    // the last ended step's outcome, written by the GPU (ChemArgs::status):
+    // queue slots in use, error word
     uint32_t *h_status_ = nullptr;
-    uint32_t seq_seen_ = 0;
     double *h_stage_ = nullptr;
     double *h_nh_ = nullptr;       // pinned staging of a member's n_H (engines of several members)
     void *h_fields_ = nullptr;     // pinned staging of the fields read-back, grown on demand

@@ -448,9 +448,8 @@ __device__ void end_pass(const ChemArgs &A) {
         C->par = par ^ 1;
     }
     C->merged = 0;
-    const uint32_t seq = C->seq + 1;
-    C->seq = seq;
-    *A.status = make_uint4((uint32_t)live, (uint32_t)(live >> 32), (uint32_t)C->err, seq);
+    // (each word stands for itself: the host relies on no order between them)
+    *A.status = make_uint2((uint32_t)live, (uint32_t)C->err);
 }
 
 __global__ void __launch_bounds__(256) k_chem(ChemArgs A) {

@@ -66,7 +66,7 @@ struct ChemArgs {
     Ranges rg;
     int two;                 // deposits of two words (Cells::dep)
     int final_pass;          // 0: a trial pass of the Gamma - <n_HI> iteration (state unchanged)
-    uint4 *status;           // host memory: the last step's queue slots in use (x, y), error word, number
+    uint2 *status;           // host memory: the last ended step's queue slots in use, error word
 };
 
 // Where a step's kernels go: onto a stream, or into a graph as nodes that run

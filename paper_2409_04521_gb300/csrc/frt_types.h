@@ -103,7 +103,7 @@ struct Ctl {
     int32_t far;             // the march left children beyond the pixel table
     long long mbase;         // the march's output count: merged rays are appended from here
     uint32_t ticket;         // blocks of the chemistry kernel done (the last one ends the pass or step)
-    uint32_t seq;            // steps ended since the engine was made
+    uint32_t pad;
 };
 
 // Ray queue.  A record is 6 + nb words -- emitter, birth step, direction (dx,
