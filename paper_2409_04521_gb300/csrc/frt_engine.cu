@@ -713,11 +713,20 @@ flexrt_status Engine::poll() {
     return latched_;
 }
 
-// a run starts anew: what ended before is not reported any more (nothing that
-// was enqueued is still running)
-void Engine::clear_outcome() {
+// a run starts anew (nothing that was enqueued is still running): what ended
+// before is not reported any more, and an open step is dropped
+flexrt_status Engine::start_anew() {
+    const bool failed = latched_ != FLEXRT_OK || h_status_[1] != 0;
     latched_ = FLEXRT_OK;
     h_status_[0] = h_status_[1] = 0;
+    mid_step_ = false;
+    if (failed && mwmem_) {
+        // a step that failed may have stopped inside the merge, with groups
+        // not cleared: clear the whole merge scratch
+        auto it = alloc_sizes_.find(mwmem_);
+        if (it != alloc_sizes_.end()) CK(cudaMemsetAsync(mwmem_, 0, it->second, st_));
+    }
+    return FLEXRT_OK;
 }
 
 static cudaEvent_t take_event(std::vector<cudaEvent_t> &pool) {
@@ -925,15 +934,8 @@ flexrt_status Engine::retire(int s) {
 
 flexrt_status Engine::reset_all() {
     CK(cudaStreamSynchronize(st_));
-    const bool failed = latched_ != FLEXRT_OK || h_status_[1] != 0 || mid_step_;
-    clear_outcome();
-    mid_step_ = false;                           // an open step is dropped
-    if (failed && mwmem_) {
-        // a step that failed may have stopped inside the merge, with groups
-        // not cleared: clear the whole merge scratch
-        auto it = alloc_sizes_.find(mwmem_);
-        if (it != alloc_sizes_.end()) CK(cudaMemsetAsync(mwmem_, 0, it->second, st_));
-    }
+    flexrt_status r = start_anew();
+    if (r != FLEXRT_OK) return r;
     // the rest in stream order, ahead of the steps that follow
     CK(launch_reset(ctl_, sims_, acc_, (int)slots_.size(), st_));
     for (int s = 0; s < (int)slots_.size(); ++s) {
@@ -1324,9 +1326,10 @@ flexrt_status Engine::load_state(int s, const void *buf, int64_t bytes) {
     CK(up(&ctl_->par, par_err, sizeof(par_err)));
     sl->h.step = (int32_t)h.step;
     CK(up((char *)(sims_ + s) + offsetof(SimDev, step), &sl->h.step, sizeof(int32_t)));
-    clear_outcome();
+    flexrt_status r = start_anew();
+    if (r != FLEXRT_OK) return r;
     if (h.dt > 0.0) {
-        flexrt_status r = set_dt(s, h.dt);
+        r = set_dt(s, h.dt);
         if (r != FLEXRT_OK) return r;
     }
     CK(cudaStreamSynchronize(st_));

@@ -147,7 +147,7 @@ class Engine {
     flexrt_status grow_emitters(int need);
     flexrt_status upload_lists();             // active emitters, cell ranges, counters
     flexrt_status poll();
-    void clear_outcome();
+    flexrt_status start_anew();
     Sink on_stream() const { Sink s; s.st = st_; return s; }
     flexrt_status launch_step(Sink to);
     flexrt_status launch_stage(int stage, Sink &to);
