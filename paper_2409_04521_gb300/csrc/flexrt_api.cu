@@ -1,9 +1,10 @@
 // flexrt_api.cu -- the C ABI declared in include/flexrt.h.
 //
-// A flexrt_ctx is an engine with one simulation slot, stepped by direct
-// launches; a flexrt_batch is an engine with many slots whose step (one RT
-// step of every active simulation) is replayed from a CUDA graph.  Both run
-// the same kernels; every size the kernels need is read from device memory.
+// A flexrt_ctx is an engine with one simulation slot, whose step is launched
+// directly at first and then replayed from a CUDA graph; a flexrt_batch is an
+// engine with many slots whose step (one RT step of every active simulation)
+// is replayed from a graph from the start.  Both run the same kernels; every
+// size the kernels need is read from device memory.
 #include <algorithm>
 #include <cstring>
 #include <new>

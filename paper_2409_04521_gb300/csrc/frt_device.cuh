@@ -386,10 +386,10 @@ __device__ __forceinline__ void walk_ties(int x, int y, int z, int sx, int sy, i
 // leaves the grid (it is outside, or a crossing leaves it).  A crossing that
 // leaves the grid, and an axis not crossed, set the key's sign, which stays
 // set for the slots after it.  Measured: the march is bound by instruction
-// issue and latency; with this walk and seg_attenuate it issues 820 warp
-// instructions per 32 rays (1030 with three cross-multiplied 64-bit
-// comparisons a ray and a position update a slot): 647 -> 571 us on 1.45e7
-// rays, 4 bins.
+// issue and latency; this walk and seg_attenuate, put in place of three
+// cross-multiplied 64-bit comparisons a ray and a position update a slot, took
+// it from 1030 to 820 warp instructions per 32 rays and from 647 to 571 us on
+// 1.45e7 rays, 4 bins (k_march gives what later changes made of it).
 __device__ __forceinline__ void walk_step(bool valid, int px, int py, int pz, int dx, int dy, int dz, int nx, int ny,
                                           int nz, int coff, int (&key)[4], float (&ds)[4], bool &esc) {
     constexpr int SIGN = (int)0x80000000u;
@@ -515,27 +515,28 @@ __device__ __forceinline__ int warp_incl_scan(int x) {
 }
 
 // ---------------------------------------------------------------------------
-// Ray records (frt_types.h): tail words of record r of a tile as vector pieces.  STREAM:
-// evict-first accesses (the queue streams through once per step, and the
-// cells' opacities and deposit buffers stay resident in L2).
+// Ray records (frt_types.h): tail words of record r of a tile as vector pieces.
+// STREAM: evict-first stores (a surviving ray's record is read once, a step
+// later, while the cells' opacities and deposit buffers are used all along).
+// The bulk copies that bring the march's records in carry no such hint.
 // ---------------------------------------------------------------------------
-template <int NB, bool STREAM>
+template <int NB>
 __device__ __forceinline__ void load_tail(const char *tile, unsigned r, uint32_t (&w)[2 + NB]) {
     constexpr int T = 2 + NB, N4 = T / 4;
 #pragma unroll
     for (int k = 0; k < N4; ++k) {
         const uint4 *p = reinterpret_cast<const uint4 *>(tile + 512 * (1 + k)) + r;
-        const uint4 v = STREAM ? __ldcs(p) : *p;
+        const uint4 v = *p;
         w[4 * k] = v.x; w[4 * k + 1] = v.y; w[4 * k + 2] = v.z; w[4 * k + 3] = v.w;
     }
     if (T & 2) {
         const uint2 *p = reinterpret_cast<const uint2 *>(tile + 512 * (1 + N4)) + r;
-        const uint2 v = STREAM ? __ldcs(p) : *p;
+        const uint2 v = *p;
         w[4 * N4] = v.x; w[4 * N4 + 1] = v.y;
     }
     if (T & 1) {
         const uint32_t *p = reinterpret_cast<const uint32_t *>(tile + 512 * (1 + N4) + ((T & 2) ? 256 : 0)) + r;
-        w[T - 1] = STREAM ? __ldcs(p) : *p;
+        w[T - 1] = *p;
     }
 }
 template <int NB, bool STREAM>
@@ -558,14 +559,13 @@ __device__ __forceinline__ void store_tail(char *tile, unsigned r, const uint32_
     }
 }
 // the same for a bin count known at run time; words past the record are zero
-template <bool STREAM>
 __device__ __forceinline__ void load_tail_n(const Queue &q, unsigned i, uint32_t (&w)[2 + MAXB]) {
 #pragma unroll
     for (int k = 0; k < 2 + MAXB; ++k) w[k] = 0u;
     auto get = [&](auto tag) {
         constexpr int NB = decltype(tag)::value;
         uint32_t v[2 + NB];
-        load_tail<NB, STREAM>(tile_of(q, i), i & 31u, v);
+        load_tail<NB>(tile_of(q, i), i & 31u, v);
 #pragma unroll
         for (int k = 0; k < 2 + NB; ++k) w[k] = v[k];
     };

@@ -117,9 +117,11 @@ class Engine {
     bool merge_built() const { return cfg_.merge_l_max >= 0; }
     // the march variants: 0 plain, 1 with merged rays, 3 with merged rays
     // and the moving screen (engines that may run Generalized members); plus 4
+    // with one simulation
     int ext_variants() const { return (cfg_.gen_capable ? 3 : (merge_built() ? 1 : 0)) | (one_sim() ? 4 : 0); }
-    // one simulation, steps launched directly (a graph would keep the
-    // constants of a member replaced since)
+    // one simulation whose constants are launch arguments: its graph is made
+    // again when it changes (a batch's graph is made once, for members that
+    // come and go)
     bool one_sim() const { return cfg_.max_sims == 1 && !cfg_.use_graph; }
     flexrt_status ionized_volume(int slot, double *x_ion);
     // checkpoint of a single-simulation engine (slot 0): bytes needed, save, load

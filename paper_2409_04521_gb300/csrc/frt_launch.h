@@ -126,8 +126,9 @@ MarchFn march_fn_two(int nb, int agg, int minb);
 MarchFn march_fn_two_merge(int nb, int agg, int minb);
 MarchFn march_fn_two_gen(int nb, int agg, int minb);
 // ext: 0 plain, 1 merged rays, 3 merged rays and Generalized mode; plus 4:
-// one simulation, launched directly (its variants exist without aggregation;
-// with it the general one runs); plus 8: its deposits are two words
+// one simulation whose constants are launch arguments (its variants exist
+// without aggregation; with it the general one runs); plus 8: its deposits are
+// two words
 bool march_variant_exists(int nb, int agg, int minb, int ext);
 // opt the variant into all the dynamic shared memory a block may have
 cudaError_t march_prepare(int nb, int agg, int minb, int ext);

@@ -185,7 +185,7 @@ __device__ __forceinline__ void seg_attenuate(float2 k, float dse, const float *
 // (Eq. 18-19).  A merging engine without Generalized members runs EXT = 1
 // (fewer registers: 10% less march time on the merging workloads than with
 // both), an engine that may run Generalized members EXT = 3.
-// ONE: an engine with one simulation whose steps are launched directly: its
+// ONE: an engine with one simulation (not a batch of one slot): its
 // constants come with the launch (A.one: the instructions take them from
 // constant memory, where a load of each from shared memory a ray and segment
 // was a fifth of the load-store unit's work, the march's busiest) and its
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
             float ph[NB];
             {
                 uint32_t w[2 + NB];
-                load_tail<NB, false>(rec, lane, w);
+                load_tail<NB>(rec, lane, w);
 #pragma unroll
                 for (int b = 0; b < NB; ++b) ph[b] = __uint_as_float(w[2 + b]);
             }
@@ -594,7 +594,7 @@ __global__ void __launch_bounds__(256, MINB) k_march(const __grid_constant__ Mar
                         const unsigned sub = c & ((1u << (2 * mm)) - 1u);
                         const uint4 pa = heads[src];
                         uint32_t cw[2 + NB];
-                        load_tail<NB, false>(rec, src, cw);
+                        load_tail<NB>(rec, src, cw);
                         const int4 rows[3] = {rowbuf[src], rowbuf[32 + src], rowbuf[64 + src]};
                         const uint32_t ppl = cw[1];
                         const int psim = rows[1].w;

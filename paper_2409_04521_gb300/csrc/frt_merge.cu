@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(256) k_mhist1(MergeArgs A) {
             // emitter lookup); bins past a member's own are zero
             const uint32_t e = A.nsims > 1 ? ray_head(q, i)->x : 0u;
             uint32_t w[2 + MAXB];
-            load_tail_n<false>(q, (unsigned)i, w);
+            load_tail_n(q, (unsigned)i, w);
             const uint32_t pl = w[1];
             int sim = -1;
             uint32_t key = 0;
@@ -602,7 +602,7 @@ __global__ void __launch_bounds__(256, 4) k_mweight(MergeArgs A) {
             const uint32_t e = ray_head(q, qi)->x;
             nbf = S.nb;
             uint32_t w[2 + MAXB];
-            load_tail_n<false>(q, qi, w);
+            load_tail_n(q, qi, w);
 #pragma unroll
             for (int b = 0; b < MAXB; ++b)
                 if (b < nbf) f[b] = __uint_as_float(w[2 + b]);
